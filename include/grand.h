@@ -89,9 +89,13 @@ typedef enum grand_order {
 } grand_order;
 
 /* How a TEP's membership H (y ^ e) = 0 is tested (results do not depend on it).
- *   AUTO        syndrome deltas (Alg. 2 Step 4: s(y) xor the H columns a TEP
- *               flips) in the split search of the fused kernels; QAM_NNE5
- *               runs DELTA.
+ *   AUTO        the library's choice. QAM_NNE / QAM_NEARER with automatic
+ *               tiles[0] and tiles[1] and no deadline: the linear system of
+ *               SOLVE below, which decides all valid TEPs of a frame at once
+ *               (one kernel, no scratch memory). With an explicit tiles[0] or
+ *               tiles[1], a deadline, or in the resumable search: syndrome
+ *               deltas (Alg. 2 Step 4: s(y) xor the H columns a TEP flips)
+ *               compared TEP by TEP in the split search. QAM_NNE5 runs DELTA.
  *   DELTA       syndrome deltas, one TEP per lane and step in canonical
  *               order (no split search); grand_decode_symbols only.
  *   ROW_PARITY  the candidate word y ^ e multiplied by H row by row, each
@@ -117,15 +121,14 @@ typedef enum grand_order {
  *               diagonal alternative flips both), and y xor e is a codeword
  *               iff the XOR of the slots' syndrome deltas over x equals s(y):
  *               a linear system over GF(2) with at most 2 S' unknowns. The
- *               preparation solves it by Gaussian elimination; its solutions
+ *               kernel solves it by Gaussian elimination; its solutions
  *               are the frame's codewords within the TEP space, and the one of
  *               smallest canonical rank is the first hit (no solution: the
  *               frame abandons with min(valid TEPs, query_cap) queries).
  *               Outputs are those of AUTO (decoded word, query count = the
  *               hit's position in the canonical order, abandon flag); stats
- *               count the ranked solutions as checks. The preparation tests
- *               weights <= 1 first (tiles[2] is not used). Frames whose
- *               solution set has more than 2^8 members go to the TEP search.
+ *               count the solutions looked at as checks and no searched
+ *               frames. tiles are not used, and a deadline cuts no frame.
  *               QAM_NNE / QAM_NEARER (uniform and uneven batches); not for
  *               QAM_NNE5, HAMMING, the resumable search, the autotuner or
  *               the no-allocation entry point. */
@@ -160,7 +163,9 @@ typedef enum grand_lik {
  *   max_weight  HAMMING order: largest number of flipped bits (0..4).
  *   query_cap   abandonment threshold, >= 1 valid queries.
  *   lik_variant GRAND_LIK_*.
- *   tiles       launch shape, 0 = automatic: [0] warps per search CTA (1..8
+ *   tiles       launch shape of the two-kernel TEP search and the hash join
+ *               (the one-kernel decode of AUTO and SOLVE picks its own),
+ *               0 = automatic: [0] warps per search CTA (1..8
  *               for explicit splits, 1..4 for the warp-per-frame search and
  *               the hash join), [1] A-side ranks of the search split (1..6; a
  *               nonzero value selects the CTA-per-frame search, 0 the
@@ -214,13 +219,17 @@ typedef struct grand_frame_desc {
  * Requesting them makes the call synchronise its stream before returning.
  *   evaluated_checks  TEP syndrome checks executed on the GPU, including
  *                     speculative ones beyond the first hit.
- *   hard_frames       frames that needed the parallel search stage.
+ *                     (AUTO in one kernel: every valid TEP of a frame is
+ *                     decided, so it counts all of them).
+ *   hard_frames       frames that needed the parallel search stage (AUTO in
+ *                     one kernel: frames with no codeword in the first
+ *                     tiles[2] weights, 2 by default).
  *   search_useful     valid TEP queries (positions <= the reported query
  *                     count) that fell to the search stage.
  *   prep_ms, search_ms  device time of the preparation and search kernels,
  *                     from CUDA events recorded on the call's stream
- *                     (HAMMING order: prep_ms = 0 and search_ms = the one
- *                     bit-level kernel). */
+ *                     (HAMMING order and the one-kernel decode: prep_ms = 0
+ *                     and search_ms = the one kernel). */
 typedef struct grand_stats {
   uint64_t evaluated_checks;
   uint64_t hard_frames;
@@ -573,7 +582,8 @@ int grand_server_destroy(grand_server* srv);
  * where the stream-ordered allocator is unavailable or would break a latency
  * budget. Same inputs, outputs and results as grand_decode_symbols with the
  * same params; the caller still provides every input and output buffer.
- *   - Internal scratch is a fixed array of about 2.4 MB in the library's
+ *   - Internal scratch (used by calls with a deadline or explicit tiles) is
+ *     a fixed array of about 2.4 MB in the library's
  *     device memory, present on every GPU that loads the library until the
  *     process exits. It holds at most GRAND_NOALLOC_MAX_FRAMES frames: larger
  *     n_frames is rejected with GRAND_E_UNSUPPORTED before any GPU work.

@@ -95,13 +95,15 @@ extern "C" int grand_code_create(const uint32_t* H, int N, int K, grand_code** o
   // per-column projections hf[j] (a fixed pseudo-random 32-bit word per row,
   // from the splitmix64 finaliser of the row index)
   // layout of the device copy: hcol [N*W], hf [N], prow [R], frozen [R] (u16, packed 2 per word),
-  // hrow [R * N/32] (the rows as given)
-  const size_t words = (size_t)N * W + N + R + (R + 1) / 2 + (size_t)R * (N / 32);
+  // hrow [R * N/32] (the rows as given), hx [N], fmask [N/32]
+  const size_t words = (size_t)N * W + N + R + (R + 1) / 2 + (size_t)R * (N / 32) + N + N / 32;
   std::vector<uint32_t> hcol(words, 0);
   uint32_t* hf = hcol.data() + (size_t)N * W;
   uint32_t* prow = hf + N;
   uint16_t* frozen = reinterpret_cast<uint16_t*>(prow + R);
   uint32_t* hrow = prow + R + (R + 1) / 2;
+  uint32_t* hx = hrow + (size_t)R * (N / 32);
+  uint32_t* fmask = hx + N;
   memcpy(hrow, H, sizeof(uint32_t) * (size_t)R * (N / 32));
   bool polar = true;
   for (int r = 0; r < R; ++r) {
@@ -129,6 +131,19 @@ extern "C" int grand_code_create(const uint32_t* H, int N, int K, grand_code** o
       }
     }
   }
+  if (polar) {
+    for (int r = 0; r < R; ++r) fmask[frozen[r] >> 5] |= 1u << (frozen[r] & 31);
+    for (int j = 0; j < N; ++j) {
+      // masked transform of bit j: the frozen indices that are subsets of j
+      for (int w = 0; w < N / 32; ++w) {
+        uint32_t word = 0;
+        if ((w & ~(j >> 5)) == 0)
+          for (int i = 0; i < 32; ++i)
+            if ((i & ~(j & 31)) == 0) word |= 1u << i;
+        hx[j] = grand::syndrome_fold(hx[j], word & fmask[w]);
+      }
+    }
+  }
   grand_code* c = (grand_code*)calloc(1, sizeof(grand_code));
   if (!c) return GRAND_E_NOMEM;
   c->N = N; c->K = K; c->R = R; c->W = W;
@@ -153,6 +168,8 @@ extern "C" int grand_code_create(const uint32_t* H, int N, int K, grand_code** o
   c->dev.prow = c->dev.hf + N;
   c->dev.frozen = reinterpret_cast<const uint16_t*>(c->dev.prow + R);
   c->dev.hrow = c->dev.prow + R + (R + 1) / 2;
+  c->dev.hx = c->dev.hrow + (size_t)R * (N / 32);
+  c->dev.fmask = c->dev.hx + N;
   c->dev.status = c->d_status;
   c->dev.N = N; c->dev.K = K; c->dev.R = R; c->dev.W = W;
   c->dev.polar = polar ? 1 : 0;

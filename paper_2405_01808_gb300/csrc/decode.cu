@@ -1,6 +1,8 @@
 // GRAND decoder kernels for sm_103a and the C ABI entry points.
 //
-// Stages of one decode call (Alg. 2 of the paper):
+// The symbol-level calls without a deadline, weight window, hash join or
+// explicit launch shape run the one-kernel decode of fused.cu (takes_fused).
+// The others run these stages (Alg. 2 of the paper):
 //   k_prep         one warp per frame: demodulation + likelihood + neighbours
 //                  (Step 1), hard word y and base syndrome s0 = H y, selection
 //                  of the S' least reliable symbols (Steps 2-3), the syndrome
@@ -31,6 +33,7 @@
 #include <vector>
 
 #include "device_common.cuh"
+#include "fused.cuh"
 #include "host_util.cuh"
 
 namespace grand {
@@ -54,7 +57,8 @@ struct PrepArgs {
   const CodeDev* codes;          // device table
   int n_codes;
   int64_t n_frames;
-  int M;                         // uniform batch
+  int M, L;                      // uniform batch
+  int NWmax;                     // words of the longest code
   int S;
   int lik;
   int nearer;                    // GRAND_ORDER_QAM_NEARER: swap h / v where d_Q < d_I
@@ -275,206 +279,11 @@ __device__ __forceinline__ uint32_t binom_le3(int n, int k) {
   return k == 0 ? 1u : (k == 1 ? m : (k == 2 ? m * (m - 1) / 2u : m * (m - 1) * (m - 2) / 6u));
 }
 
-// Largest kernel dimension solve_frame ranks exhaustively (2^8 solutions).
-constexpr int kSolveKerMax = 8;
-// Resident CTAs per SM of the preparation with the elimination (syndromes of
-// at most two words; the longer ones run 8 like the plain preparation).
-constexpr int kPrepSolveBlocks = 10;
-
-// 32 x 32 bit transpose across a warp: lane i holds row i on entry, lane j
-// holds column j on return (bit i of it = bit j of row i).
-__device__ __forceinline__ uint32_t warp_transpose_bits(uint32_t x) {
-  const int lane = threadIdx.x & 31;
-  constexpr uint32_t kMask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    const int k = 16 >> s;
-    const uint32_t m = kMask[s];
-    const uint32_t y = __shfl_xor_sync(kFull, x, k);
-    x = (lane & k) ? (((y >> k) & m) | (x & ~m)) : ((x & m) | ((y & m) << k));
-  }
-  return x;
-}
-
-// Column b of the slot system (see solve_frame): the syndrome delta of slot b
-// (slot b & 1 of rank b >> 1) in the preparation's delta array.
-__device__ __forceinline__ const uint32_t* slot_column(const PrepSmem& sm, int b, int W) {
-  return sm.delta + ((b >> 1) * 3 + (b & 1)) * W;
-}
-
-// XOR of the slot columns over x (and s0 when with_s0) is zero on every
-// syndrome word (lanes = words; x is the same in every lane).
-__device__ __forceinline__ bool slot_sum_zero(const PrepSmem& sm, int W, uint32_t x, bool with_s0) {
-  const int lane = threadIdx.x & 31;
-  uint32_t acc = 0;
-  if (lane < W) {
-    acc = with_s0 ? sm.s0[lane] : 0u;
-    for (uint32_t m = x; m; m &= m - 1u) acc ^= slot_column(sm, __ffs(m) - 1, W)[lane];
-  }
-  return !__any_sync(kFull, acc != 0u);
-}
-
-// The first hit among the solutions x0 + span(km[0..d)): every one is a
-// valid TEP (only existing slots take part) and is ranked by its canonical
-// position.
-__device__ __forceinline__ void rank_solutions(const PrepSmem& sm, int Sp, uint32_t x0, const uint32_t (&km)[kSolveKerMax],
-                                               int d, uint32_t& best_rank, uint32_t& best_code,
-                                               unsigned long long& evaluated) {
-  const int lane = threadIdx.x & 31;
-  if (d == 0) {  // the usual case: one solution, ranked by every lane alike
-    best_rank = tep_rank(sm.E, Sp, sm.ex, x0);
-    best_code = x0;
-    if (lane == 0) evaluated += 1;
-    return;
-  }
-  uint32_t lr = 0xFFFFFFFFu, lc = 0;
-  for (uint32_t c = (uint32_t)lane; c < (1u << d); c += 32) {
-    uint32_t x = x0;
-#pragma unroll
-    for (int t = 0; t < kSolveKerMax; ++t)
-      if ((c >> t) & 1u) x ^= km[t];
-    const uint32_t rk = tep_rank(sm.E, Sp, sm.ex, x);
-    if (rk < lr) { lr = rk; lc = x; }
-  }
-  if (lane == 0) evaluated += 1ull << d;
-  const uint32_t br = __reduce_min_sync(kFull, lr);
-  const unsigned who = __ballot_sync(kFull, lr == br);
-  best_code = __shfl_sync(kFull, lc, __ffs(who) - 1);
-  best_rank = br;
-}
-
-// GRAND_MEMBERSHIP_SOLVE: the frame's first codeword in canonical order by
-// Gaussian elimination over GF(2) instead of a test per TEP. A valid TEP is a
-// flip vector x over the existing slots (bit 2r: the first single-axis slot
-// of rank r, bit 2r+1: the second; the diagonal is both), and H (y xor e) = 0
-// reads XOR_{b in x} c_b = s0 with c_b the syndrome delta of slot b (zero for
-// a flip beyond N): the codewords of the TEP space are the solutions x0 +
-// ker of this system, and the first hit is the solution of smallest
-// canonical rank.
-//   Fast path: the system on one 32-bit word per column and for s0 -- the
-// syndrome itself when it has one word (exact), else the 32-bit projections
-// of the columns and of s0 -- transposed across the warp (lane r holds bit r
-// of every column and of s0) and brought to reduced row echelon form, pivots
-// in slot order (one ballot and one shuffle per slot). The projection is
-// linear, so no projected solution means no solution. Otherwise the
-// projected kernel vectors and x0 are checked on the full syndrome: when
-// every kernel vector passes, the two kernels agree, and then x0 either
-// passes (the solutions are x0 + that kernel) or no solution exists. A kernel vector that fails (the projection lost rank on
-// the columns' span, about 2^(2S'-32) of frames) sends the frame to the
-// exact path: the elimination on the full columns in shared memory.
-// Returns 1 (best_rank and best_code set), 0 (no valid TEP gives a
-// codeword: the frame abandons) or -1 (more than 2^kSolveKerMax solutions:
-// the frame goes to the TEP search).
-__device__ __forceinline__ int solve_frame(const PrepSmem& sm, int Sp, int W, uint32_t f0, uint32_t& best_rank,
-                                           uint32_t& best_code, unsigned long long& evaluated) {
-  const int lane = threadIdx.x & 31;
-  const int nb = 2 * Sp;  // <= 24 < 31
-  const bool on = lane < nb && ((sm.ex[lane >> 1] >> (lane & 1)) & 1u);
-  uint32_t km[kSolveKerMax];
-  {
-    const bool one_word = W == 1;
-    // lane b: the word of slot b, lane 31: that of s0; transposed so that
-    // lane r holds bit r of every column (bit b: slot b, bit 31: s0)
-    uint32_t row = on ? (one_word ? slot_column(sm, lane, 1)[0] : sm.dflt[(lane >> 1) * 3 + (lane & 1)])
-                      : (lane == 31 ? (one_word ? sm.s0[0] : f0) : 0u);
-    row = warp_transpose_bits(row);
-    // reduced row echelon form over the existing slots, pivots in slot order
-    const unsigned on_mask = __ballot_sync(kFull, on);
-    bool used = false;  // this row holds a pivot
-    int pc = 0;         // its slot
-    uint32_t free_slots = 0;
-    for (int b = 0; b < nb; ++b) {
-      if (!((on_mask >> b) & 1u)) continue;  // an absent slot is no unknown
-      const unsigned cand = __ballot_sync(kFull, !used && ((row >> b) & 1u));
-      if (!cand) {
-        free_slots |= 1u << b;
-        continue;
-      }
-      const int pr = __ffs(cand) - 1;
-      const uint32_t prow = __shfl_sync(kFull, row, pr);
-      if (lane == pr) {
-        used = true;
-        pc = b;
-      } else if ((row >> b) & 1u) {
-        row ^= prow;
-      }
-    }
-    // a row without pivot that still needs s0's bit: not even the word of s0 is reached
-    if (__any_sync(kFull, !used && (row >> 31))) return 0;
-    const uint32_t x0 = __reduce_or_sync(kFull, used && (row >> 31) ? 1u << pc : 0u);
-    const int d = __popc(free_slots);
-    bool kernels_agree = d <= kSolveKerMax;
-    uint32_t fs = free_slots;
-#pragma unroll
-    for (int t = 0; t < kSolveKerMax; ++t) {
-      km[t] = 0;
-      if (t < d) {
-        const int f = __ffs(fs) - 1;
-        fs &= fs - 1u;
-        km[t] = (1u << f) | __reduce_or_sync(kFull, used && ((row >> f) & 1u) ? 1u << pc : 0u);
-        if (!one_word) kernels_agree = kernels_agree && slot_sum_zero(sm, W, km[t], false);
-      }
-    }
-    if (kernels_agree) {
-      if (!one_word && !slot_sum_zero(sm, W, x0, true)) return 0;
-      rank_solutions(sm, Sp, x0, km, d, best_rank, best_code, evaluated);
-      return 1;
-    }
-    if (one_word) return -1;  // exact already: the solution set is too large to rank
-  }
-  // exact path: lane b reduces column b in place (the delta slots), lane 31
-  // reduces s0 (copied to the unused diagonal slot of rank 0)
-  uint32_t* s0c = sm.delta + 2 * W;
-  for (int w = lane; w < W; w += 32) s0c[w] = sm.s0[w];
-  __syncwarp();
-  const bool act = on || lane == 31;
-  uint32_t* col = lane == 31 ? s0c : sm.delta + ((lane >> 1) * 3 + (lane & 1)) * W;
-  uint32_t msk = on ? 1u << lane : 0u;
-  bool pivot = false;
-  for (int j = 0; j < nb; ++j) {
-    int p = -1;
-    if (lane == j && on) {
-      for (int w = 0; w < W; ++w) {
-        const uint32_t x = col[w];
-        if (x) { p = 32 * w + __ffs(x) - 1; break; }
-      }
-      pivot = p >= 0;
-    }
-    p = __shfl_sync(kFull, p, j);
-    if (p < 0) continue;  // slot j absent, or its column a sum of earlier ones
-    const uint32_t pm = __shfl_sync(kFull, msk, j);
-    const uint32_t* pc = slot_column(sm, j, W);
-    if (act && lane > j && ((col[p >> 5] >> (p & 31)) & 1u)) {
-      for (int w = 0; w < W; ++w) col[w] ^= pc[w];
-      msk ^= pm;
-    }
-    __syncwarp();
-  }
-  uint32_t rest = 0;
-  if (lane == 31)
-    for (int w = 0; w < W; ++w) rest |= col[w];
-  if (__shfl_sync(kFull, rest, 31) != 0u) return 0;  // s0 is not a sum of the slot columns
-  const uint32_t x0 = __shfl_sync(kFull, msk, 31);
-  uint32_t dep = __ballot_sync(kFull, on && !pivot);
-  const int d = __popc(dep);
-  if (d > kSolveKerMax) return -1;
-#pragma unroll
-  for (int t = 0; t < kSolveKerMax; ++t) {
-    km[t] = 0;
-    if (t < d) {
-      km[t] = __shfl_sync(kFull, msk, __ffs(dep) - 1);
-      dep &= dep - 1;
-    }
-  }
-  rank_solutions(sm, Sp, x0, km, d, best_rank, best_code, evaluated);
-  return 1;
-}
-
 // One frame of the preparation (one warp). Returns true when the frame needs
 // the search stage; its hand-off record then went to a fresh slot of the
 // batch's record array. WM: compile-time bound on the syndrome words
 // (registers of the base syndrome).
-template <int WM, bool kSolve>
+template <int WM>
 __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, const PrepSmem& sm,
                                            unsigned long long& evaluated) {
   const int lane = threadIdx.x & 31;
@@ -760,12 +569,7 @@ __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, c
     uint32_t done_count = 0;  // valid TEPs with at most w_done altered ranks
     for (int v = 0; v <= w_done; ++v) done_count += sm.E[Sp * kEStride + v];
 
-    bool none = false;  // no valid TEP of the frame gives a codeword
-    if constexpr (kSolve) {
-      if (best_rank == 0xFFFFFFFFu && w_done < Sp && (uint64_t)done_count < (uint64_t)a.cap)
-        none = solve_frame(sm, Sp, W, f0, best_rank, best_code, evaluated) == 0;
-    }
-    const bool resolved = best_rank != 0xFFFFFFFFu || none || w_done >= Sp || (uint64_t)done_count >= (uint64_t)a.cap;
+    const bool resolved = best_rank != 0xFFFFFFFFu || w_done >= Sp || (uint64_t)done_count >= (uint64_t)a.cap;
     if (resolved) {
       uint32_t q;
       uint8_t ab;
@@ -823,8 +627,8 @@ __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, c
 // bound then costs a few spilled words but the latency-bound preparation
 // gains warps); 8 for the longer syndromes, whose per-lane arrays would spill
 // heavily at 40 registers.
-template <int WM, bool kSolve>
-__global__ void __launch_bounds__(128, WM <= 2 ? (kSolve ? kPrepSolveBlocks : 12) : 8) k_prep(PrepArgs a) {
+template <int WM>
+__global__ void __launch_bounds__(128, WM <= 2 ? 12 : 8) k_prep(PrepArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp_in_block = threadIdx.x >> 5;
@@ -834,7 +638,7 @@ __global__ void __launch_bounds__(128, WM <= 2 ? (kSolve ? kPrepSolveBlocks : 12
   const int64_t nwarps = (int64_t)gridDim.x * warps_per_block;
   unsigned long long evaluated = 0;
   if (a.deadline > 0 && lane == 0) past_deadline(&a.scr->t0, a.deadline);  // start the call's clock
-  for (int64_t f = gwarp; f < a.n_frames; f += nwarps) prep_frame<WM, kSolve>(a, f, sm, evaluated);
+  for (int64_t f = gwarp; f < a.n_frames; f += nwarps) prep_frame<WM>(a, f, sm, evaluated);
   // stats
   for (int o = 16; o; o >>= 1) evaluated += __shfl_xor_sync(kFull, evaluated, o);
   if (lane == 0 && evaluated) atomicAdd(&a.scr->evaluated, evaluated);
@@ -2786,23 +2590,13 @@ static void launch_demod(const DemodArgs& a, bool paired, int grid, cudaStream_t
 }
 
 typedef void (*PrepKernel)(PrepArgs);
-static PrepKernel prep_kernel_for(int Wmax, bool solve = false) {
-  if (solve) {
-    if (Wmax <= 1) return k_prep<1, true>;
-    if (Wmax <= 2) return k_prep<2, true>;
-    if (Wmax <= 4) return k_prep<4, true>;
-    if (Wmax <= 8) return k_prep<8, true>;
-    return k_prep<16, true>;
-  }
-  if (Wmax <= 1) return k_prep<1, false>;
-  if (Wmax <= 2) return k_prep<2, false>;
-  if (Wmax <= 4) return k_prep<4, false>;
-  if (Wmax <= 8) return k_prep<8, false>;
-  return k_prep<16, false>;
+static PrepKernel prep_kernel_for(int Wmax) {
+  if (Wmax <= 1) return k_prep<1>;
+  if (Wmax <= 2) return k_prep<2>;
+  if (Wmax <= 4) return k_prep<4>;
+  if (Wmax <= 8) return k_prep<8>;
+  return k_prep<16>;
 }
-
-
-
 
 // Resident CTAs per SM of a kernel for one launch shape on the current
 // device, with its dynamic shared-memory limit raised to the request: both
@@ -2905,10 +2699,8 @@ static int launch_search(const SearchArgs& s, int threads, size_t smem, int vari
 // one-time stall of milliseconds into the first batch that needs it).
 int preload_qam_kernels() {
   const void* kernels[] = {
-      (const void*)k_prep<1, false>, (const void*)k_prep<2, false>, (const void*)k_prep<4, false>,
-      (const void*)k_prep<8, false>, (const void*)k_prep<16, false>, (const void*)k_prep<1, true>,
-      (const void*)k_prep<2, true>, (const void*)k_prep<4, true>, (const void*)k_prep<8, true>,
-      (const void*)k_prep<16, true>,
+      (const void*)k_prep<1>, (const void*)k_prep<2>, (const void*)k_prep<4>,
+      (const void*)k_prep<8>, (const void*)k_prep<16>,
       (const void*)k_search_warp<4, false, false>, (const void*)k_search_warp<6, false, false>,
       (const void*)k_search_warp<8, false, false>, (const void*)k_search_warp<4, true, false>,
       (const void*)k_search_warp<6, true, false>, (const void*)k_search_warp<8, true, false>,
@@ -2922,7 +2714,7 @@ int preload_qam_kernels() {
     cudaFuncAttributes attr;
     if (cudaFuncGetAttributes(&attr, k) != cudaSuccess) return GRAND_E_CUDA;
   }
-  return GRAND_OK;
+  return preload_decode_kernels();
 }
 
 #define CU(x)                                   \
@@ -2988,6 +2780,84 @@ static int launch_qam_search(const grand_params* p, int Smax, int w0, int Wmax, 
   return launch_search(s, threads, smem, p->tiles[3], st);
 }
 
+// Calls that the one-kernel decode serves: the library's own choice of the
+// membership test (automatic tiles: no explicit warps per CTA or split) and
+// the linear solve. A budget cuts a frame between its preparation and its
+// search, and a weight window leaves a cursor there: those calls, the hash
+// join and the explicit launch shapes keep the two kernels.
+static bool takes_fused(const grand_params* p, const ResumeOpt& ro) {
+  if (ro.w_step > 0 || ro.cur_in) return false;
+  if (p->membership == GRAND_MEMBERSHIP_SOLVE) return true;
+  return p->membership == GRAND_MEMBERSHIP_AUTO && p->deadline_ns == 0 && p->tiles[0] == 0 && p->tiles[1] == 0;
+}
+
+// TEP weights the preparation tests.
+static int prep_weights(const grand_params* p) { return p->tiles[2] > 0 ? (p->tiles[2] > 3 ? 3 : p->tiles[2]) : 2; }
+
+static DecodeArgs decode_args(const PrepArgs& a, const grand_params* p, int n_codes, int64_t n_frames) {
+  DecodeArgs d{};
+  d.symbols = a.symbols;
+  d.hard_idx = a.hard_idx;
+  d.key = a.key;
+  d.nmask = a.nmask;
+  d.y_in = a.y_in;
+  d.desc = a.desc;
+  d.n_symbols = a.n_symbols;
+  d.n_cw_words = a.n_cw_words;
+  d.codes = a.codes;
+  d.n_codes = n_codes;
+  d.n_frames = n_frames;
+  d.M = a.M;
+  d.L = a.L;
+  d.S = a.S;
+  d.lik = a.lik;
+  d.nearer = p->order == GRAND_ORDER_QAM_NEARER ? 1 : 0;
+  d.solve = p->membership == GRAND_MEMBERSHIP_SOLVE ? 1 : 0;
+  d.w0 = prep_weights(p);
+  d.NWmax = a.NWmax;
+  d.cap = a.cap;
+  d.qc = a.qc;
+  d.cw = a.cw;
+  d.queries = a.queries;
+  d.abandon = a.abandon;
+  return d;
+}
+
+// The one-kernel decode: no scratch but the counters of a call with stats.
+static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_params* p, int64_t n_frames,
+                     grand_stats* stats, cudaStream_t st) {
+  DecodeArgs a = decode_args(proto, p, n_codes, n_frames);
+  if (!stats) return launch_decode(a, Lmax, st);
+  if (scratch_alloc((void**)&a.scr, sizeof(Scratch), st) != cudaSuccess) return GRAND_E_NOMEM;
+  int rc = GRAND_OK;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  do {
+    if (cudaMemsetAsync(a.scr, 0, sizeof(Scratch), st) != cudaSuccess || cudaEventCreate(&ev[0]) != cudaSuccess ||
+        cudaEventCreate(&ev[1]) != cudaSuccess) {
+      rc = GRAND_E_CUDA;
+      break;
+    }
+    cudaEventRecord(ev[0], st);
+    if ((rc = launch_decode(a, Lmax, st)) != GRAND_OK) break;
+    cudaEventRecord(ev[1], st);
+    Scratch h{};
+    if (cudaMemcpyAsync(&h, a.scr, sizeof(Scratch), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess) {
+      rc = GRAND_E_CUDA;
+      break;
+    }
+    stats->evaluated_checks = h.evaluated;
+    stats->hard_frames = h.n_hard;
+    stats->search_useful = h.search_useful;
+    stats->prep_ms = 0.0f;
+    cudaEventElapsedTime(&stats->search_ms, ev[0], ev[1]);  // the one kernel
+  } while (0);
+  for (int i = 0; i < 2; ++i)
+    if (ev[i]) cudaEventDestroy(ev[i]);
+  cudaFreeAsync(a.scr, st);
+  return rc;
+}
+
 // Common body of the symbol-level decode calls.
 static int run_qam(const CodeDev* d_codes, int n_codes, int Lmax, int Wmax, const grand_params* p,
                    const PrepArgs& proto, int64_t n_frames, grand_stats* stats, cudaStream_t st,
@@ -2997,7 +2867,8 @@ static int run_qam(const CodeDev* d_codes, int n_codes, int Lmax, int Wmax, cons
     return GRAND_OK;
   }
   NvtxRange range("grand.decode");
-  const int w0 = p->tiles[2] > 0 ? (p->tiles[2] > 3 ? 3 : p->tiles[2]) : 2;
+  if (takes_fused(p, ro)) return run_fused(proto, Lmax, n_codes, p, n_frames, stats, st);
+  const int w0 = prep_weights(p);
   const int Smax = p->S < Lmax ? p->S : Lmax;
   // scratch: header + one record per frame (worst case: every frame hard)
   const size_t rec_bytes = sizeof(FrameRec) * (size_t)n_frames;
@@ -3016,13 +2887,12 @@ static int run_qam(const CodeDev* d_codes, int n_codes, int Lmax, int Wmax, cons
     a.deadline = p->deadline_ns;
     a.Lmax = Lmax;
     a.Wmax = Wmax;
-    const bool solve = p->membership == GRAND_MEMBERSHIP_SOLVE;
-    a.w0 = solve ? 1 : w0;  // weights <= 1 filter the frames the elimination then solves
+    a.w0 = w0;
     const int warps = 4;
     const size_t prep_smem = prep_warp_bytes(Lmax, Wmax) * warps;
     const int64_t want = (n_frames + warps - 1) / warps;
     const int grid = (int)(want < (int64_t)sm_count() * 64 ? want : (int64_t)sm_count() * 64);
-    auto kp = prep_kernel_for(Wmax, solve);
+    auto kp = prep_kernel_for(Wmax);
     if (prep_smem > 48 * 1024 && resident_ctas((const void*)kp, 32 * warps, prep_smem) < 0) {  // raises the limit
       rc = GRAND_E_CUDA;
       break;
@@ -3043,10 +2913,6 @@ static int run_qam(const CodeDev* d_codes, int n_codes, int Lmax, int Wmax, cons
     ResumeOpt ro2 = ro;
     ro2.n_codes = n_codes;
     ro2.max_entries = n_frames;  // at most every frame is handed on
-    // with the elimination, only frames whose solution set is too large to
-    // rank are handed on (none on the measured workloads): one CTA per SM
-    // keeps that launch short
-    if (solve) ro2.max_entries = n_frames < (int64_t)sm_count() ? n_frames : (int64_t)sm_count();
     if (launch_qam_search(p, Smax, a.w0, Wmax, d_codes, recs, scr, proto.cw, proto.queries, proto.abandon, st, ro2) !=
         GRAND_OK) {
       rc = GRAND_E_CUDA;
@@ -3255,6 +3121,8 @@ extern "C" int grand_decode_batch(const grand_code* c, const grand_params* p, co
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
+  a.L = L;
+  a.NWmax = c->N / 32;
   a.S = p->S;
   a.lik = p->lik_variant;
   a.cap = p->query_cap;
@@ -3290,6 +3158,8 @@ extern "C" int grand_decode_symbols(const grand_code* c, const grand_params* p, 
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
+  a.L = L;
+  a.NWmax = c->N / 32;
   a.S = p->S;
   a.lik = p->lik_variant;
   a.cap = p->query_cap;
@@ -3335,6 +3205,8 @@ extern "C" int grand_decode_symbols_resumable(const grand_code* c, const grand_p
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
+  a.L = L;
+  a.NWmax = c->N / 32;
   a.S = p->S;
   a.lik = p->lik_variant;
   a.cap = p->query_cap;
@@ -3409,6 +3281,7 @@ static int mixed_impl(const CodeDev* d_table, int n_codes, int Lmax, int Wmax, c
   a.n_codes = n_codes;
   a.n_frames = n_frames;
   a.M = 0;
+  a.NWmax = Lmax >> 4;  // Lmax = N / 2 of the longest code
   a.S = p->S;
   a.lik = p->lik_variant;
   a.cap = p->query_cap;
@@ -3660,8 +3533,6 @@ extern "C" int grand_decode_symbols_noalloc(const grand_code* c, const grand_par
   cudaStream_t st = (cudaStream_t)stream;
   Scratch* scr = reinterpret_cast<Scratch*>(base);
   FrameRec* recs = reinterpret_cast<FrameRec*>(static_cast<char*>(base) + kNoAllocHeader);
-  // the array keeps the previous call's contents: reset the counters
-  if (cudaMemsetAsync(scr, 0, sizeof(Scratch), st) != cudaSuccess) return GRAND_E_CUDA;
   const int L = (c->N + 2 * m - 1) / (2 * m);
   PrepArgs a{};
   a.symbols = (const float2*)symbols;
@@ -3669,6 +3540,8 @@ extern "C" int grand_decode_symbols_noalloc(const grand_code* c, const grand_par
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
+  a.L = L;
+  a.NWmax = c->N / 32;
   a.S = p->S;
   a.lik = p->lik_variant;
   a.cap = p->query_cap;
@@ -3676,12 +3549,15 @@ extern "C" int grand_decode_symbols_noalloc(const grand_code* c, const grand_par
   a.cw = cw;
   a.queries = queries;
   a.abandon = abandon;
+  if (takes_fused(p, ResumeOpt())) return launch_decode(decode_args(a, p, 1, n_frames), L, st);
+  // the array keeps the previous call's contents: reset the counters
+  if (cudaMemsetAsync(scr, 0, sizeof(Scratch), st) != cudaSuccess) return GRAND_E_CUDA;
   a.recs = recs;
   a.scr = scr;
   a.deadline = p->deadline_ns;
   a.Lmax = L;
   a.Wmax = c->W;
-  a.w0 = p->tiles[2] > 0 ? (p->tiles[2] > 3 ? 3 : p->tiles[2]) : 2;
+  a.w0 = prep_weights(p);
   const int warps = 4;
   const size_t prep_smem = prep_warp_bytes(L, c->W) * warps;
   auto kp = prep_kernel_for(c->W);

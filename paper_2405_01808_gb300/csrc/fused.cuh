@@ -1,0 +1,43 @@
+// Launch interface of the fused decode kernel (fused.cu).
+#pragma once
+
+#include "host_util.cuh"
+#include "internal.cuh"
+
+namespace grand {
+
+struct DecodeArgs {
+  const float2* symbols;         // received symbols, or NULL: the demodulated arrays
+  const uint16_t* hard_idx;
+  const uint32_t* key;
+  const uint8_t* nmask;
+  const uint32_t* y_in;
+  const grand_frame_desc* desc;  // NULL: uniform batch
+  int64_t n_symbols;             // mixed: length of the flat symbol array
+  int64_t n_cw_words;            // mixed: length of the flat output array
+  const CodeDev* codes;          // device table
+  int n_codes;
+  int64_t n_frames;
+  int M, L;                      // uniform batch
+  int S;
+  int lik;
+  int nearer;                    // GRAND_ORDER_QAM_NEARER: swap h / v where d_Q < d_I
+  int solve;                     // statistics of GRAND_MEMBERSHIP_SOLVE (ranked solutions)
+  int w0;                        // statistics: weights a searched frame went past
+  int NWmax;                     // words of the longest code (uniform batch: of the code)
+  int T;                         // frames per warp (set by launch_decode)
+  int64_t cap;
+  QamConst qc;
+  uint32_t* cw;
+  uint32_t* queries;
+  uint8_t* abandon;
+  Scratch* scr;                  // statistics, or NULL
+};
+
+// One launch on `st`; Lmax: the largest frame of the batch in symbols.
+int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st);
+
+// Load the kernels an uneven batch can launch (see preload_qam_kernels).
+int preload_decode_kernels();
+
+}  // namespace grand

@@ -31,16 +31,31 @@ constexpr uint16_t kNoPos = 0xFFFF;  // alternative bit beyond N (padding): no s
 //          grand_code_create): the row-parity membership test.
 //   status[0]: set (atomicOr 1) by a kernel that cut a frame at the call's
 //          deadline; status[1]: where grand_stream_status takes it to.
+//   polar form also: fmask[w] = the frozen bits among indices 32 w .. 32 w + 31
+//          (the transform of y masked by it is the syndrome, unpacked), and
+//   hx[j] = syndrome_fold of the masked transform of bit j, words in ascending
+//          order: a linear 32-bit projection that the fused kernel computes
+//          from the masked words alone (for N = 32 it is the syndrome itself).
 struct CodeDev {
   const uint32_t* hcol;
   const uint32_t* hf;
   const uint16_t* frozen;
   const uint32_t* prow;
   const uint32_t* hrow;
+  const uint32_t* hx;
+  const uint32_t* fmask;
   uint32_t* status;
   int32_t N, K, R, W;
   int32_t polar;
 };
+
+// One step of the projection hx: fold the next masked word into h. Linear in
+// (h, word); on polar columns its rank is that of random projections (slot
+// sets of 20 and 24 columns, N = 64 .. 1024, lose rank as often: 0-9 of 1,500),
+// where a plain rotation or a shift register loses it on most.
+__host__ __device__ inline uint32_t syndrome_fold(uint32_t h, uint32_t word) {
+  return ((h << 13) | (h >> 19)) ^ (h << 6) ^ word;
+}
 
 // Per-frame state handed from the preparation kernel to the search kernel
 // for frames the preparation could not finish.
