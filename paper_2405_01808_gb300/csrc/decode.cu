@@ -2816,7 +2816,6 @@ static DecodeArgs decode_args(const PrepArgs& a, const grand_params* p, int n_co
   d.w0 = prep_weights(p);
   d.NWmax = a.NWmax;
   d.cap = a.cap;
-  d.qc = a.qc;
   d.cw = a.cw;
   d.queries = a.queries;
   d.abandon = a.abandon;

@@ -35,7 +35,10 @@ namespace {
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr int kWarps = 4;               // warps per CTA
 constexpr uint32_t kNone = 0xFFFFFFFFu;
-constexpr uint32_t kKeySat = 0x7FFFFFu; // packed selection keys hold 23 bits of the reliability
+constexpr uint32_t kKeySat = 0x7FFFFEu; // packed selection keys hold 23 bits of the reliability
+constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low bits) without a symbol
+constexpr uint32_t kPicked = 0xFFFFFFE0u;  // above those: a key taken as rank (low bits)
+constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to the nearest integer, ties to even
 constexpr int kLanePick = 3;            // smallest keys kept per lane of a long frame
 
 // e_v(n1, n3): valid TEPs altering exactly v of n1 ranks with one alternative
@@ -63,38 +66,113 @@ constexpr EspTable make_esp() {
 }
 __device__ const EspTable g_esp = make_esp();
 
-// One axis on the Q8.8 grid (the reading of demod_axis_q): k = the inner
-// decision threshold nearest to the received value (k separates the levels
-// k - 1 and k), e = the signed distance to it. Ties between two thresholds go
-// to the lower one, so that the neighbour of a value on a level is the lower
-// level; |e| > 256 says the value lies beyond the outermost level, where the
-// neighbouring level across the far threshold does not exist.
-struct Axis {
-  int k, e;
-};
-__device__ __forceinline__ Axis axis_at(float a, float q, int side) {
-  int aq;
-  const float x = fminf(fmaxf(__fmul_rn(a, q), -32768.0f), 32767.0f);
-  aq = __float2int_rn(x);
-  const int t = aq + 256 * side;
-  Axis r;
-  r.k = min(max((t + 255) >> 9, 1), side - 1);
-  r.e = t - (r.k << 9);
+// Two floats in one 64-bit register pair, one instruction for both.
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 pack2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
   return r;
 }
-// Distance of the ordering key (threshold or literal reading).
-__device__ __forceinline__ int axis_dist(int e, int literal) {
-  const int m = e < 0 ? -e : e;
-  const int lit = max(0, 512 - m);
-  return literal && m > 256 ? lit : min(m, 32767);
+__device__ __forceinline__ F2 pack2(float2 v) { return pack2(v.x, v.y); }
+__device__ __forceinline__ float2 unpack2(F2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// Both axes of a symbol on the Q8.8 grid (the reading of demod_axis_q) in
+// floating point: the integers involved are below 2^24, so every step is
+// exact, the FMA pipe takes what would crowd the integer ALU, and the packed
+// forms do I and Q in one instruction (about 10 instructions for what took
+// 50 in integer form). x = a q rounded to float. k = index of the inner
+// decision threshold nearest to the received value (threshold k separates the
+// levels k and k + 1), e = the signed distance to it. Ties between two
+// thresholds go to the lower one, so that the neighbour of a value on a level
+// is the lower level; |e| > 256 says the value lies beyond the outermost level,
+// where the far threshold has no neighbour level. For |x| up to 2^22; beyond,
+// k stays right and |e| stays above 256.
+struct Axes {
+  float2 kb;  // k plus 1.5 * 2^23: k in the low 6 bits of the representation
+  float2 k, e;
+};
+
+// The constants of one constellation in registers. The empty statements keep
+// the compiler from building the pairs anew for every symbol (packed
+// instructions take no immediates), which was 30 of 240 instructions a frame.
+struct AxisRegs {
+  F2 q, t0, g, magic, unmagic, m512;
+  float s, c, lim, side;
+};
+__device__ __forceinline__ AxisRegs axis_regs(const AxisConst& a) {
+  AxisRegs r;
+  r.q = pack2(a.q);
+  r.t0 = pack2(a.t0);
+  r.g = pack2(a.g);
+  r.magic = pack2(kMagic, kMagic);
+  r.unmagic = pack2(-kMagic, -kMagic);
+  r.m512 = pack2(-512.0f, -512.0f);
+  asm volatile("" : "+l"(r.q), "+l"(r.t0), "+l"(r.g), "+l"(r.magic), "+l"(r.unmagic), "+l"(r.m512));
+  r.s = a.s;
+  r.c = a.c;
+  r.lim = a.lim;
+  r.side = a.side;
+  return r;
+}
+__device__ __forceinline__ Axes axes_fast(F2 x, const AxisRegs& c) {
+  const F2 t = add2(add2(x, c.magic), c.t0);  // round(x) + 256 sqrt(M) - 512
+  const float2 ts = unpack2(t);
+  // threshold index: the nearest one, clamped to the inner thresholds by the
+  // saturation, rounded by the addition; no value lies on a tie (the offset is
+  // a quarter of the grid)
+  const float uI = __saturatef(__fmaf_rn(ts.x, c.s, c.c)), uQ = __saturatef(__fmaf_rn(ts.y, c.s, c.c));
+  const F2 kb = fma2(pack2(uI, uQ), c.g, c.magic);
+  const F2 k = add2(kb, c.unmagic);
+  Axes r;
+  r.kb = unpack2(kb);
+  r.k = unpack2(k);
+  r.e = unpack2(fma2(k, c.m512, t));
+  return r;
+}
+// Distance of the ordering key (threshold or literal reading), unclamped above.
+__device__ __forceinline__ float axis_dist(float e, int literal) {
+  const float m = fabsf(e);
+  return literal ? fmaxf(0.0f, 256.0f - fabsf(m - 256.0f)) : m;
 }
 
-// A selected symbol: index (bits 0..8), threshold of each axis (9..14,
-// 15..20), existing alternatives (21 I, 22 Q), Q nearer than I (23).
-__device__ __forceinline__ uint32_t pack_rec(int i, int kI, int kQ, bool exI, bool exQ, bool near) {
-  return (uint32_t)i | ((uint32_t)kI << 9) | ((uint32_t)kQ << 15) | (exI ? 1u << 21 : 0u) | (exQ ? 1u << 22 : 0u) |
-         (near ? 1u << 23 : 0u);
+// The alternatives of a selected symbol: the threshold toward each axis's
+// neighbour (k) and whether it exists; near: Q's distance is below I's.
+struct Alt {
+  uint32_t kI, kQ;
+  bool exI, exQ, near;
+};
+__device__ __forceinline__ Alt symbol_alt(float2 v, const AxisRegs& c, int lik) {
+  const Axes x = axes_fast(mul2(pack2(v), c.q), c);
+  const float2 e = x.e;
+  return Alt{__float_as_uint(x.kb.x) & 63u, __float_as_uint(x.kb.y) & 63u, fabsf(e.x) <= 256.0f, fabsf(e.y) <= 256.0f,
+             axis_dist(e.y, lik) < axis_dist(e.x, lik)};
 }
+
+// The full ordering key of one symbol (integer arithmetic with the int16
+// clamps of the fixed-point definition).
+__device__ __forceinline__ uint32_t symbol_key(float2 v, float q, int m, int lik) {
+  const AxisDemod I = demod_axis_q(v.x, q, 1 << m, lik), Q = demod_axis_q(v.y, q, 1 << m, lik);
+  return (uint32_t)(I.dq * I.dq) + (uint32_t)(Q.dq * Q.dq);
+}
+__device__ __forceinline__ bool finite2(float2 v) { return isfinite(v.x) && isfinite(v.y); }
 
 __device__ __forceinline__ uint32_t transform_word(uint32_t x) {  // superset sums inside a word
   x ^= (x >> 1) & 0x55555555u;
@@ -117,45 +195,25 @@ __device__ __forceinline__ uint32_t subset_pattern(uint32_t t) {
 // Where a symbol's demodulation comes from.
 enum { kFromUniform = 0, kFromMixed = 1, kFromArrays = 2 };
 
-struct Sym {
-  uint32_t key;    // full ordering key
-  uint32_t rec;    // record bits without the index
-  uint32_t label;  // Gray label bits in transmission order (bit k = label bit 2m-1-k)
-  bool nf;         // a coordinate is not finite (read as 0)
-};
-
-__device__ __forceinline__ Sym demod_symbol(float2 v, float q, int m, int lik) {
-  Sym s;
-  const int side = 1 << m;
-  s.nf = !(isfinite(v.x) && isfinite(v.y));
-  if (s.nf) v = make_float2(0.0f, 0.0f);
-  const Axis I = axis_at(v.x, q, side), Q = axis_at(v.y, q, side);
-  const int dI = axis_dist(I.e, lik), dQ = axis_dist(Q.e, lik);
-  s.key = (uint32_t)(dI * dI) + (uint32_t)(dQ * dQ);
-  s.rec = pack_rec(0, I.k, Q.k, I.e >= -256 && I.e <= 256, Q.e >= -256 && Q.e <= 256, dQ < dI);
-  const uint32_t lv = ((uint32_t)(I.k + (I.e >> 31)) << m) | (uint32_t)(Q.k + (Q.e >> 31));
-  const uint32_t gray = lv ^ ((lv >> 1) & ~(1u << (m - 1)));
-  s.label = __brev(gray) >> (32 - 2 * m);
-  return s;
-}
-
-// One symbol of a call on demodulated arrays (its hard word is an input).
-__device__ __forceinline__ Sym array_symbol(const DecodeArgs& a, int64_t o) {
-  Sym s;
+__device__ __forceinline__ Alt array_alt(const DecodeArgs& a, int64_t o) {
   const uint32_t h = a.hard_idx[o], nm = a.nmask[o];
-  s.key = a.key[o];
-  s.nf = (nm & 128u) != 0;
-  // the threshold toward the neighbour (0 or 2^m: none there, and no alternative)
-  const int kI = ((int)(h >> 8) + (int)((nm >> 3) & 1u)) & 63, kQ = ((int)(h & 0xFFu) + (int)((nm >> 4) & 1u)) & 63;
-  s.rec = pack_rec(0, kI, kQ, nm & 1u, nm & 2u, nm & 32u);
-  s.label = 0;
-  return s;
+  // the threshold toward the neighbour (where there is none the value is not used)
+  return Alt{((h >> 8) + ((nm >> 3) & 1u) - 1u) & 63u, ((h & 0xFFu) + ((nm >> 4) & 1u) - 1u) & 63u, (nm & 1u) != 0,
+             (nm & 2u) != 0, (nm & 32u) != 0};
 }
 
-template <int kFrom>
-__device__ __forceinline__ Sym symbol_at(const DecodeArgs& a, int64_t base, int i, float q, int m) {
-  if constexpr (kFrom == kFromArrays) return array_symbol(a, base + i);
-  else return demod_symbol(a.symbols[base + i], q, m, a.lik);
+// How lane `lane` takes part in packing the labels of 32 symbols into bytes
+// (m = 1..4): a group of 4, 2, 4, 1 symbols fills 1, 1, 3, 1 bytes; the group
+// ORs its labels, each shifted to its place, and some of its lanes store a
+// byte. Fields: shift to the place (bits 0..4), shift of the stored byte
+// (5..9), partner distances (10: 1, 11: 2), storing lane (12), first byte (13..).
+__device__ __forceinline__ uint32_t pack_plan(int m, int lane) {
+  if (m == 1) return (2u * (~lane & 3)) | (3u << 10) | ((lane & 3) == 0 ? 1u << 12 : 0u) | ((uint32_t)(lane >> 2) << 13);
+  if (m == 2) return (4u * (~lane & 1)) | (1u << 10) | ((lane & 1) == 0 ? 1u << 12 : 0u) | ((uint32_t)(lane >> 1) << 13);
+  if (m == 3)
+    return (6u * (~lane & 3)) | ((uint32_t)((16 - 8 * (lane & 3)) & 31) << 5) | (3u << 10) |
+           ((lane & 3) != 3 ? 1u << 12 : 0u) | ((uint32_t)((lane >> 2) * 3 + (lane & 3)) << 13);
+  return (1u << 12) | ((uint32_t)lane << 13);
 }
 
 // Exact selection of the S' smallest (key, index) pairs, S' scans of the
@@ -163,14 +221,16 @@ __device__ __forceinline__ Sym symbol_at(const DecodeArgs& a, int64_t base, int 
 // key saturates, or one lane of a long frame ran out of kept keys). Lane r
 // returns the index of rank r.
 template <int kFrom>
-__device__ __noinline__ int select_exact(const DecodeArgs& a, int64_t base, int L, int Sp, float q, int m) {
+__device__ __noinline__ int select_exact(const DecodeArgs& a, int64_t base, int L, int Sp, int m) {
   const int lane = threadIdx.x & 31;
   uint32_t last_k = 0;
   int last_i = -1, sel = 0;
   for (int r = 0; r < Sp; ++r) {
     uint32_t bk = kNone, bi = kNone;
     for (int i = lane; i < L; i += 32) {
-      const uint32_t k = symbol_at<kFrom>(a, base, i, q, m).key;
+      uint32_t k;
+      if constexpr (kFrom == kFromArrays) k = a.key[base + i];
+      else k = symbol_key(a.symbols[base + i], a.ax[m].q.x, m, a.lik);
       const bool after = k > last_k || (k == last_k && i > last_i);
       if (after && k < bk) { bk = k; bi = (uint32_t)i; }
     }
@@ -186,6 +246,17 @@ __device__ __noinline__ int select_exact(const DecodeArgs& a, int64_t base, int 
 // ---------------------------------------------------------------------------
 // Solve helpers (one thread per frame)
 // ---------------------------------------------------------------------------
+
+// c ^= v when c has a bit of p: a test and a predicated XOR (left to itself the
+// compiler selects between both values, twice the instructions).
+__device__ __forceinline__ void xor_if(uint32_t& c, uint32_t p, uint32_t v) {
+  asm("{\n\t.reg .pred q;\n\t.reg .b32 t;\n\t"
+      "and.b32 t, %0, %1;\n\t"
+      "setp.ne.b32 q, t, 0;\n\t"
+      "@q xor.b32 %0, %0, %2;\n\t}"
+      : "+r"(c)
+      : "r"(p), "r"(v));
+}
 
 // What a thread needs to look at its frame: its column of the shared words
 // (masked transform of y for polar-form H, else the compact syndrome), the
@@ -285,12 +356,13 @@ struct Proj {
 // and which passes the full test, or kNone.
 __device__ __noinline__ uint32_t light_hit(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
                                            bool exact, int wmax) {
-  auto delta = [&](int r, int c) {
-    uint32_t d = 0;
-    if (c & 1) d ^= proj(slot_pos(f, 2 * r));
-    if (c & 2) d ^= proj(slot_pos(f, 2 * r + 1));
-    return d;
-  };
+  uint32_t dl[3 * kSMax];  // thread-local: the loads of a warp are consecutive
+  for (int r = 0; r < Sp; ++r) {
+    dl[3 * r] = proj(slot_pos(f, 2 * r));
+    dl[3 * r + 1] = proj(slot_pos(f, 2 * r + 1));
+    dl[3 * r + 2] = dl[3 * r] ^ dl[3 * r + 1];
+  }
+  auto delta = [&](int r, int c) { return dl[3 * r + c - 1]; };
   auto valid = [&](int r, int c) { return ((ex >> (2 * r)) & (uint32_t)c) == (uint32_t)c; };
   auto full = [&](uint32_t x) { return exact || sum_zero(f, x, true); };
   if (f0 == 0 && full(0u)) return 0u;
@@ -363,10 +435,86 @@ __device__ __noinline__ uint32_t first_solution(const Frame f, const Proj proj, 
 }
 
 // ---------------------------------------------------------------------------
+// Front helpers (one warp per frame, one symbol per lane and step)
+// ---------------------------------------------------------------------------
+struct Step {
+  uint32_t kp;     // packed (reliability, index) key
+  uint32_t label;  // Gray labels, I then Q, most significant bit first
+};
+
+// Demodulation of 32 symbols (lane i: symbol i0 + i; off lanes give label 0).
+// nf: set when a symbol is not finite (its coordinates are read as 0).
+__device__ __forceinline__ Step demod_step(const DecodeArgs& a, const AxisRegs& ax, float2 cur, int m, uint32_t index,
+                                           bool on, bool& nf) {
+  F2 x = mul2(pack2(cur), ax.q);
+  const float2 xs = unpack2(x);
+  const bool plain = fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim;
+  uint32_t big = 0;  // key of a symbol outside the plain range
+  if (__any_sync(kAll, !plain)) {
+    float2 v = cur;
+    const bool bad = on && !finite2(v);
+    if (__any_sync(kAll, bad)) nf = true;
+    if (bad) {
+      v = make_float2(0.0f, 0.0f);
+      x = pack2(0.0f, 0.0f);
+    }
+    big = min(symbol_key(v, unpack2(ax.q).x, m, a.lik), kKeySat);
+  }
+  const Axes t = axes_fast(x, ax);
+  float2 d = t.e;
+  if (a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
+  Step s;
+  // key < 2^23 in the plain range: 2^23 + key has the key in its mantissa
+  const uint32_t key = __float_as_uint(__fadd_rn(__fmaf_rn(d.x, d.x, __fmul_rn(d.y, d.y)), 8388608.0f));
+  s.kp = (plain ? key : big) * 512u + index;
+  // hard levels: threshold index plus one above it (e >= 0; e is an integer),
+  // both axes' in one number on top of 1.5 * 2^23
+  const float lI = __fadd_rn(t.k.x, __saturatef(__fadd_rn(t.e.x, 1.0f)));
+  const float lQ = __fadd_rn(t.kb.y, __saturatef(__fadd_rn(t.e.y, 1.0f)));
+  const uint32_t lv = __float_as_uint(__fmaf_rn(lI, ax.side, lQ)) & (on ? (1u << (2 * m)) - 1u : 0u);
+  s.label = lv ^ ((lv >> 1) & ~(1u << (m - 1)));
+  return s;
+}
+
+// Labels of 32 symbols into the frame's bytes by the lane's plan (m <= 4);
+// room: bytes of the frame from the lane's byte of this step on (<= 0: none to
+// store). Every lane takes part.
+__device__ __forceinline__ void pack_labels(uint32_t label, uint32_t plan, uint8_t* yb, int room) {
+  uint32_t v = label << (plan & 31u);
+  v |= __shfl_xor_sync(kAll, v, (plan >> 10) & 1u);
+  v |= __shfl_xor_sync(kAll, v, (plan >> 10) & 2u);
+  if (room > 0) *yb = (uint8_t)(v >> ((plan >> 5) & 31u));
+}
+
+// 5 or 6 bits an axis: OR into the words.
+__device__ __forceinline__ void or_label(uint32_t label, int i, int m, uint32_t* y, int stride, int NW) {
+  const int p0 = 2 * m * i, wd = p0 >> 5, room = 32 - (p0 & 31) - 2 * m;
+  if (wd < NW) atomicOr(y + wd * stride, room >= 0 ? label << room : label >> -room);
+  if (room < 0 && wd + 1 < NW) atomicOr(y + (wd + 1) * stride, label << (32 + room));
+}
+
+// The kRanks smallest of one key per lane, by warp minima: returns the lane's
+// rank, 31 or more for none. Always kRanks rounds (straight-line code: a round
+// is four instructions); ranks beyond the frame's S' mean nothing.
+template <int kRanks>
+__device__ __forceinline__ uint32_t pick_ranks(uint32_t kp) {
+#pragma unroll
+  for (int r = 0; r < kRanks; ++r) {
+    const uint32_t kmin = __reduce_min_sync(kAll, kp);
+    kp = kp == kmin ? kPicked | (uint32_t)r : kp;
+  }
+  return kp >= kPicked ? kp & 31u : 32u;
+}
+
+// ---------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------
 // kOne: every frame has at most 32 symbols (one per lane). kSlots: 2 x the
 // largest S' (16, 20 or 24: the elimination is unrolled over it).
+//
+// Words of a hard word are kept bit-reversed in shared memory (the label bits
+// of a symbol arrive most significant first) until they are written out or
+// transformed.
 template <int kFrom, bool kOne, int kSlots>
 __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
@@ -376,11 +524,14 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   constexpr int kRanks = kSlots / 2;
   int64_t* s_off = reinterpret_cast<int64_t*>(smem_raw);             // [FT] mixed: first symbol
   int64_t* s_cw = s_off + (kFrom == kFromMixed ? FT : 0);            // [FT] mixed: first output word
-  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_cw + (kFrom == kFromMixed ? FT : 0));  // [FT] mixed: L | m | code
-  uint32_t* pat = s_par + (kFrom == kFromMixed ? FT : 0);            // [32]
+  float2* s_sym = reinterpret_cast<float2*>(s_cw + (kFrom == kFromMixed ? FT : 0));  // [kRanks][FT] kOne: the symbol of each rank
+  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_sym + (kOne ? kRanks * FT : 0));   // [FT] mixed: L | m | words | polar
+  uint32_t* s_code = s_par + (kFrom == kFromMixed ? FT : 0);         // [FT] mixed: index of the code
+  uint32_t* s_plan = s_code + (kFrom == kFromMixed ? FT : 0);        // [4][32] mixed: pack_plan
+  uint32_t* pat = s_plan + (kFrom == kFromMixed ? 128 : 0);          // [32]
   uint32_t* s_f0 = pat + 32;                                         // [FT] projection of s(y) (H not of polar form)
   uint32_t* s_flag = s_f0 + FT;                                      // [FT] 0, or the abandon flag of an undecodable frame
-  uint32_t* rec = s_flag + FT;                                       // [kRanks][FT]
+  uint32_t* rec = s_flag + FT;                                       // [kRanks][FT] symbol index, later slot positions
   uint32_t* buf = rec + kRanks * FT;                                 // [NWmax][stride]
   const int64_t tile = (int64_t)blockIdx.x * FT;
   const int n_here = (int)min((int64_t)FT, a.n_frames - tile);
@@ -389,192 +540,227 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   for (int t = threadIdx.x; t < a.NWmax * stride; t += 32 * kWarps) buf[t] = 0u;
   for (int t = threadIdx.x; t < FT; t += 32 * kWarps) s_flag[t] = 0u;
   if constexpr (kFrom == kFromMixed) {
+    s_plan[threadIdx.x] = pack_plan(warp + 1, lane);
     for (int t = threadIdx.x; t < n_here; t += 32 * kWarps) {
       const grand_frame_desc d = a.desc[tile + t];
       const int m = (31 - __clz(d.M)) >> 1;
       bool ok = d.code >= 0 && d.code < a.n_codes && m >= 1 && m <= 6 && d.M == 1 << (2 * m) && d.sym_offset >= 0 &&
                 d.cw_offset >= 0;
-      int L = 0;
+      uint32_t par = 1u << 10;  // L = 0: not decoded
       if (ok) {
-        const int N = a.codes[d.code].N;
-        L = (N + 2 * m - 1) / (2 * m);
+        const CodeDev* code = a.codes + d.code;
+        const int N = code->N, L = (N + 2 * m - 1) / (2 * m);
         ok = d.sym_offset + L <= a.n_symbols && d.cw_offset + (N >> 5) <= a.n_cw_words;
+        if (ok) par = (uint32_t)L | ((uint32_t)m << 10) | ((uint32_t)(N >> 5) << 13) | (code->polar ? 1u << 19 : 0u);
       }
       s_off[t] = d.sym_offset;
       s_cw[t] = d.cw_offset;
-      s_par[t] = ok ? (uint32_t)L | ((uint32_t)m << 10) | ((uint32_t)d.code << 13) : 1u << 10;  // L = 0: not decoded
+      s_par[t] = par;
+      s_code[t] = ok ? (uint32_t)d.code : 0u;
     }
   }
   __syncthreads();
 
   // --- front: one warp per frame ---------------------------------------------
-  int um = 0, uL = 0;
-  if constexpr (kFrom != kFromMixed) {
-    um = (31 - __clz(a.M)) >> 1;
-    uL = a.L;
-  }
-  const int fr_end = min(n_here, (warp + 1) * a.T);
+  const int um = kFrom == kFromMixed ? 0 : a.m, uL = kFrom == kFromMixed ? 0 : a.L;
+  const bool u_polar = kFrom == kFromMixed ? false : a.codes->polar != 0;
+  const int fr_begin = warp * a.T, fr_end = min(n_here, fr_begin + a.T);
   auto frame_base = [&](int fr) { return kFrom == kFromMixed ? s_off[fr] : (tile + fr) * (int64_t)uL; };
   auto frame_len = [&](int fr) { return kFrom == kFromMixed ? (int)(s_par[fr] & 1023u) : uL; };
-  float2 nxt = make_float2(0.0f, 0.0f);
-  if constexpr (kFrom != kFromArrays) {
-    const int fr = warp * a.T;
-    if (fr < fr_end && lane < frame_len(fr)) nxt = a.symbols[frame_base(fr) + lane];
-  }
-  for (int fr = warp * a.T; fr < fr_end; ++fr) {
-    const int64_t base = frame_base(fr);
-    const int L = frame_len(fr);
-    const int m = kFrom == kFromMixed ? (int)((s_par[fr] >> 10) & 7u) : um;
-    const CodeDev* code = kFrom == kFromMixed ? a.codes + (s_par[fr] >> 13) : a.codes;
-    const float q = a.qc.q[m];
-    const int Sp = a.S < L ? a.S : L;
-    const int b2 = 2 * m;
-    uint32_t* y = buf + fr;
-    uint32_t best[kOne ? 1 : kLanePick];
-#pragma unroll
-    for (int j = 0; j < (kOne ? 1 : kLanePick); ++j) best[j] = kNone;
-    uint32_t info = 0;
-    bool nf = false;
-    const int nch = kOne ? 1 : max(1, (L + 31) >> 5);
-    const int nbytes = kFrom == kFromMixed ? code->N >> 3 : a.NWmax * 4;
-    for (int c = 0; c < nch; ++c) {
-      const int i = 32 * c + lane;
-      const bool on = i < L;
-      const float2 cur = nxt;
-      if constexpr (kFrom != kFromArrays) {  // the next 32 symbols, of this frame or the next one
-        if (!kOne && c + 1 < nch) {
-          if (i + 32 < L) nxt = a.symbols[base + i + 32];
-        } else if (fr + 1 < fr_end) {
-          if (lane < frame_len(fr + 1)) nxt = a.symbols[frame_base(fr + 1) + lane];
-        }
-      }
-      Sym s{kNone, 0u, 0u, false};
-      if constexpr (kFrom == kFromArrays) {
-        if (on) s = array_symbol(a, base + i);
-      } else {
-        s = demod_symbol(cur, q, m, a.lik);
-        if (!on) { s.label = 0u; s.nf = false; }
-        // the group of symbols that fills whole bytes ORs its labels together
-        // and stores them (4, 2, 1 symbols a byte for m = 1, 2, 4; 4 symbols
-        // in 3 bytes for m = 3); m = 5, 6 OR into the word
-        uint8_t* yb = reinterpret_cast<uint8_t*>(y);
-        auto put = [&](int byte, uint32_t v) {
-          if (byte < nbytes) yb[(byte >> 2) * (4 * stride) + (byte & 3)] = (uint8_t)v;
-        };
-        if (m == 1) {
-          uint32_t v = s.label << (2 * (lane & 3));
-          v |= __shfl_xor_sync(kAll, v, 1);
-          v |= __shfl_xor_sync(kAll, v, 2);
-          if ((lane & 3) == 0) put(i >> 2, v);
-        } else if (m == 2) {
-          uint32_t v = s.label << (4 * (lane & 1));
-          v |= __shfl_xor_sync(kAll, v, 1);
-          if ((lane & 1) == 0) put(i >> 1, v);
-        } else if (m == 4) {
-          put(i, s.label);
-        } else if (m == 3) {
-          uint32_t v = s.label << (6 * (lane & 3));
-          v |= __shfl_xor_sync(kAll, v, 1);
-          v |= __shfl_xor_sync(kAll, v, 2);
-          if ((lane & 3) != 3) put((i >> 2) * 3 + (lane & 3), v >> (8 * (lane & 3)));
-        } else if (on) {
-          const int p0 = b2 * i, wd = p0 >> 5, sh = p0 & 31;
-          if (4 * wd < nbytes) atomicOr(y + wd * stride, s.label << sh);
-          if (sh + b2 > 32 && 4 * (wd + 1) < nbytes) atomicOr(y + (wd + 1) * stride, s.label >> (32 - sh));
-        }
-      }
-      nf |= s.nf;
-      const uint32_t kp = on ? (min(s.key, kKeySat) << 9) | (uint32_t)i : kNone;
-      if constexpr (kOne) {
-        best[0] = kp;
-        info = s.rec;
-      } else {
-        const uint32_t t0 = max(best[0], kp);
-        best[0] = min(best[0], kp);
-        const uint32_t t1 = max(best[1], t0);
-        best[1] = min(best[1], t0);
-        best[2] = min(best[2], t1);
-      }
-    }
-    if (L == 0) {  // not a decodable descriptor
-      if (lane == 0) s_flag[fr] = 3u;
-      continue;
-    }
-    if constexpr (kFrom == kFromArrays) {
-      const int NW = a.NWmax;
-      if (lane < NW) y[lane * stride] = a.y_in[(tile + fr) * NW + lane];
-    }
-    if (__any_sync(kAll, nf)) {
-      if (lane == 0) s_flag[fr] = 2u;
-      continue;
-    }
-    // Steps 2-3: the S' least reliable symbols by warp minima of the packed
-    // (reliability, index) keys
-    uint32_t sel = 0, kmin = 0;
-    int pops = 0;
-    for (int r = 0; r < Sp; ++r) {
-      kmin = __reduce_min_sync(kAll, best[0]);
-      if (lane == r) sel = kmin;
-      if (best[0] == kmin) {
-        if constexpr (kOne) {
-          best[0] = kNone;
-        } else {
-          best[0] = best[1];
-          best[1] = best[2];
-          best[2] = kNone;
-          ++pops;
-        }
-      }
-    }
-    bool redo = Sp > 0 && (kmin >> 9) >= kKeySat;
-    if constexpr (!kOne) redo |= __any_sync(kAll, pops >= kLanePick && L > 32 * kLanePick + lane);
-    sel &= 511u;
-    if (redo) sel = (uint32_t)select_exact<kFrom>(a, base, L, Sp, q, m);
+  // the rare rest of a frame: exact selection, and for H not of polar form
+  // the base syndrome by the columns of y's one-bits
+  auto reselect = [&](int fr, int L, int m, int Sp, float2 cur) {
+    const int sel = select_exact<kFrom>(a, frame_base(fr), L, Sp, m);
     if constexpr (kOne) {
-      const uint32_t v = __shfl_sync(kAll, info, (int)(sel & 31u));
-      if (lane < Sp) rec[lane * FT + fr] = v | sel;
-    } else {
-      if (lane < Sp) rec[lane * FT + fr] = sel;  // its alternatives are worked out in the solve
+      const float2 v = make_float2(__shfl_sync(kAll, cur.x, sel), __shfl_sync(kAll, cur.y, sel));
+      if (lane < Sp) s_sym[lane * FT + fr] = v;
     }
-    // H not of polar form: the base syndrome by the columns of y's one-bits
-    if (!code->polar) {
-      __syncwarp();
-      const int W = code->W, NW = code->N >> 5;
-      uint32_t yw = lane < NW ? y[lane * stride] : 0u;
-      const int64_t co = kFrom == kFromMixed ? s_cw[fr] : (tile + fr) * (int64_t)NW;
-      if (lane < NW) a.cw[co + lane] = yw;
-      uint32_t f0 = 0;
+    __syncwarp();
+    if (lane < Sp) rec[lane * FT + fr] = (uint32_t)sel;
+  };
+  auto general_syndrome = [&](int fr, int NW) {
+    __syncwarp();
+    uint32_t* y = buf + fr;
+    const CodeDev* code = a.codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
+    const int W = code->W;
+    const uint32_t yw = lane < NW ? __brev(y[lane * stride]) : 0u;
+    const int64_t co = kFrom == kFromMixed ? s_cw[fr] : (tile + fr) * (int64_t)NW;
+    if (lane < NW) a.cw[co + lane] = yw;
+    uint32_t f0 = 0;
+    for (int w = 0; w < NW; ++w)
+      if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) f0 ^= __ldg(code->hf + 32 * w + lane);
+    f0 = __reduce_xor_sync(kAll, f0);
+    for (int v = 0; v < W; ++v) {
+      uint32_t acc = 0;
       for (int w = 0; w < NW; ++w)
-        if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) f0 ^= __ldg(code->hf + 32 * w + lane);
-      f0 = __reduce_xor_sync(kAll, f0);
-      for (int v = 0; v < W; ++v) {
-        uint32_t acc = 0;
-        for (int w = 0; w < NW; ++w)
-          if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) acc ^= __ldg(code->hcol + (size_t)(32 * w + lane) * W + v);
-        acc = __reduce_xor_sync(kAll, acc);
-        if (lane == 0) y[v * stride] = acc;  // the hard word is no longer needed here
-        if (W == 1) f0 = acc;
-      }
-      if (lane == 0) s_f0[fr] = f0;
+        if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) acc ^= __ldg(code->hcol + (size_t)(32 * w + lane) * W + v);
+      acc = __reduce_xor_sync(kAll, acc);
+      if (lane == 0) y[v * stride] = acc;  // the hard word is no longer needed here
+      if (W == 1) f0 = acc;
     }
-  }
-  __syncthreads();
+    if (lane == 0) s_f0[fr] = f0;
+  };
 
-  // --- hard words out (decoded bits are flipped in place later) ---------------
-  if constexpr (kFrom == kFromMixed) {
-    for (int fr = warp; fr < n_here; fr += kWarps) {
-      if (s_flag[fr] == 3u) continue;
-      const CodeDev* code = a.codes + (s_par[fr] >> 13);
-      if ((code->polar || s_flag[fr]) && lane < (code->N >> 5)) a.cw[s_cw[fr] + lane] = buf[lane * stride + fr];
+  if constexpr (kOne) {
+    const AxisRegs ax = axis_regs(a.ax[um]);
+    const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
+    const bool on = lane < uL;
+    const uint32_t plan = pack_plan(um, lane);
+    const int byte0 = (int)(plan >> 13), room = (plan >> 12) & 1u ? 4 * NW - byte0 : 0;
+    uint8_t* yb = reinterpret_cast<uint8_t*>(buf + fr_begin) + (byte0 >> 2) * (4 * stride) + (~byte0 & 3);
+    const float2* sym = a.symbols + (tile + fr_begin) * (int64_t)uL + lane;
+    float2 nxt = make_float2(0.0f, 0.0f);
+    if (on && fr_begin < fr_end) nxt = *sym;
+    for (int fr = fr_begin; fr < fr_end; ++fr, yb += 4) {
+      const float2 cur = nxt;
+      sym += uL;
+      if (on && fr + 1 < fr_end) nxt = *sym;  // the next frame's symbols are on their way meanwhile
+      bool nf = false;
+      const Step st = demod_step(a, ax, cur, um, (uint32_t)lane, on, nf);
+      if (um <= 4) pack_labels(st.label, plan, yb, room);
+      else if (on) or_label(st.label, lane, um, buf + fr, stride, NW);
+      if (nf) {
+        if (lane == 0) s_flag[fr] = 2u;
+        continue;
+      }
+      const uint32_t r = pick_ranks<kRanks>(on ? st.kp : kOff + (uint32_t)lane);
+      const bool mine = r < (uint32_t)Sp;
+      if (mine) {
+        s_sym[r * FT + fr] = cur;
+        rec[r * FT + fr] = (uint32_t)lane;
+      }
+      if (__any_sync(kAll, mine && st.kp >= kKeySat << 9)) reselect(fr, uL, um, Sp, cur);
+      if (!u_polar) general_syndrome(fr, NW);
     }
   } else {
-    const int NW = a.NWmax, lg = 31 - __clz(NW), polar = a.codes->polar;
-    for (int t = threadIdx.x; t < n_here * NW; t += 32 * kWarps) {
-      const int fr = t >> lg, w = t & (NW - 1);
-      if (polar || s_flag[fr]) a.cw[tile * NW + t] = buf[w * stride + fr];
+    float2 nxt = make_float2(0.0f, 0.0f);
+    if constexpr (kFrom != kFromArrays) {
+      if (fr_begin < fr_end && lane < frame_len(fr_begin)) nxt = a.symbols[frame_base(fr_begin) + lane];
+    }
+    for (int fr = fr_begin; fr < fr_end; ++fr) {
+      const uint32_t par = kFrom == kFromMixed ? s_par[fr] : 0u;
+      const int L = kFrom == kFromMixed ? (int)(par & 1023u) : uL;
+      const int m = kFrom == kFromMixed ? (int)((par >> 10) & 7u) : um;
+      const int NW = kFrom == kFromMixed ? (int)((par >> 13) & 63u) : a.NWmax;
+      const bool polar = kFrom == kFromMixed ? (par >> 19) != 0u : u_polar;
+      const int Sp = a.S < L ? a.S : L;
+      uint32_t* y = buf + fr;
+      // this lane's smallest keys, ascending
+      uint32_t b0 = kNone, b1 = kNone, b2 = kNone;
+      static_assert(kLanePick == 3, "kept keys");
+      auto keep = [&](uint32_t kp) {
+        const uint32_t t0 = max(b0, kp);
+        b0 = min(b0, kp);
+        const uint32_t t1 = max(b1, t0);
+        b1 = min(b1, t0);
+        b2 = min(b2, t1);
+      };
+      bool nf = false;  // uniform
+      if constexpr (kFrom == kFromArrays) {
+        const int64_t base = frame_base(fr);
+        bool mine = false;
+        for (int i = lane; i < L; i += 32) {
+          mine |= (a.nmask[base + i] & 128u) != 0;
+          keep((min(a.key[base + i], kKeySat) << 9) | (uint32_t)i);
+        }
+        nf = __any_sync(kAll, mine);
+        if (lane < NW) y[lane * stride] = __brev(a.y_in[(tile + fr) * NW + lane]);
+      } else {
+        const AxisRegs ax = axis_regs(a.ax[m]);
+        const uint32_t plan = kFrom == kFromMixed ? s_plan[32 * ((m - 1) & 3) + lane] : pack_plan(um, lane);
+        const int byte0 = (int)(plan >> 13);
+        uint8_t* yb = reinterpret_cast<uint8_t*>(y) + (byte0 >> 2) * (4 * stride) + (~byte0 & 3);
+        int room = (plan >> 12) & 1u ? 4 * NW - byte0 : 0;
+        const float2* sym = a.symbols + frame_base(fr) + lane;
+        int left = L - lane;  // symbols of this lane's stride from here on: on while positive
+        uint32_t index = (uint32_t)lane;
+        for (int i0 = 0;;) {
+          const float2 cur = nxt;
+          const bool on = left > 0, more = i0 + 32 < L;
+          // the next 32 symbols, of this frame or the next one, are on their way meanwhile
+          if (more) {
+            sym += 32;
+            if (left > 32) nxt = *sym;
+          } else if (fr + 1 < fr_end) {
+            if (lane < frame_len(fr + 1)) nxt = a.symbols[frame_base(fr + 1) + lane];
+          }
+          const Step st = demod_step(a, ax, cur, m, index, on, nf);
+          if (m <= 4) {
+            pack_labels(st.label, plan, yb, room);
+            yb += 8 * m * stride;  // 2 m words on
+            room -= 8 * m;
+          } else if (on) {
+            or_label(st.label, (int)index, m, y, stride, NW);
+          }
+          keep(on ? st.kp : kNone);
+          if (!more) break;
+          i0 += 32;
+          left -= 32;
+          index += 32u;
+        }
+      }
+      if (nf || (kFrom == kFromMixed && L == 0)) {  // not searched, or not a decodable descriptor
+        if (lane == 0) s_flag[fr] = L == 0 ? 3u : 2u;
+        continue;
+      }
+      // Steps 2-3: the S' least reliable symbols; the lane that holds a
+      // minimum records it
+      uint32_t* recf = rec + fr;
+      bool redo;
+      if (L <= 32) {
+        const uint32_t r = pick_ranks<kRanks>(lane < L ? b0 : kOff + (uint32_t)lane);
+        const bool mine = r < (uint32_t)Sp;
+        if (mine) recf[r * FT] = (uint32_t)lane;
+        redo = mine && b0 >= kKeySat << 9;
+      } else {
+        uint32_t pick = 0;
+#pragma unroll
+        for (int r = 0; r < kRanks; ++r) {
+          const uint32_t kmin = __reduce_min_sync(kAll, b0);
+          const bool w = b0 == kmin;
+          if (lane == r) pick = kmin;
+          b0 = w ? b1 : b0;
+          b1 = w ? b2 : b1;
+          b2 = w ? kNone : b2;
+        }
+        const bool mine = lane < Sp;
+        if (mine) recf[lane * FT] = pick & 511u;
+        // a saturated key was taken, or a lane ran out of kept keys
+        redo = (mine && pick >= kKeySat << 9) || (b0 == kNone && L > 32 * kLanePick + lane);
+      }
+      if (__any_sync(kAll, redo)) reselect(fr, L, m, Sp, make_float2(0.0f, 0.0f));
+      if (!polar) general_syndrome(fr, NW);
     }
   }
-  __syncthreads();
+  // A full tile (32 frames a warp) is solved by the warps that prepared it,
+  // each on its own; smaller ones by the first 4 T threads of the CTA. (Long
+  // and uneven frames wait for one another in any case: warps of a CTA in
+  // different parts of the kernel evict each other's instructions, which cost
+  // more than the barrier: 306 against 281 us for 200,000 mixed frames.)
+  const bool own = kOne && a.T == 32;
+  auto tile_sync = [&]() {
+    if (own) __syncwarp(); else __syncthreads();
+  };
+  tile_sync();
+
+  // --- hard words out (decoded bits are flipped in place later) ---------------
+  {
+    const int first = own ? 32 * warp : 0, last = own ? min(n_here, first + 32) : n_here;
+    if constexpr (kFrom == kFromMixed) {
+      for (int fr = own ? first : warp; fr < last; fr += own ? 1 : kWarps) {
+        const uint32_t par = s_par[fr];
+        const bool out = (par & 1023u) && ((par >> 19) || s_flag[fr]);  // a general matrix's word is out already
+        if (out && lane < (int)((par >> 13) & 63u)) a.cw[s_cw[fr] + lane] = __brev(buf[lane * stride + fr]);
+      }
+    } else {
+      const int NW = a.NWmax, lg = 31 - __clz(NW);
+      for (int t = first * NW + (own ? lane : (int)threadIdx.x); t < last * NW; t += own ? 32 : 32 * kWarps) {
+        const int fr = t >> lg, w = t & (NW - 1);
+        if (u_polar || s_flag[fr]) a.cw[tile * NW + t] = __brev(buf[w * stride + fr]);
+      }
+    }
+  }
+  tile_sync();
 
   // --- solve: one thread per frame ---------------------------------------------
   unsigned long long evaluated = 0, useful = 0;
@@ -589,7 +775,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
     } else {
       const int L = frame_len(fr);
       const int m = kFrom == kFromMixed ? (int)((s_par[fr] >> 10) & 7u) : um;
-      const CodeDev* code = kFrom == kFromMixed ? a.codes + (s_par[fr] >> 13) : a.codes;
+      const CodeDev* code = kFrom == kFromMixed ? a.codes + s_code[fr] : a.codes;
       const int N = code->N, NW = N >> 5;
       const int64_t cw_off = kFrom == kFromMixed ? s_cw[fr] : f * (int64_t)NW;
       const int Sp = a.S < L ? a.S : L;
@@ -604,29 +790,49 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       F.pat = pat;
       F.polar = code->polar;
       F.nw = F.polar ? NW : code->W;
-      const bool exact = F.polar ? NW == 1 : code->W == 1;
+      // one syndrome word: the columns themselves, and the elimination is the full test
+      const bool exact = code->W == 1;
+      const Proj proj{exact && !(F.polar && NW == 1) ? code->hcol : (F.polar ? code->hx : code->hf)};
 
-      // the alternatives of each rank: flip positions, existing slots
-      uint32_t ex = 0;
+      // the alternatives of each rank: flip positions, existing slots, and
+      // the slots' columns
+      uint32_t c[kSlots];
+      uint32_t ex = 0, real = 0;  // existing slots; those whose flip lies inside the word
       {
-        const float q = a.qc.q[m];
+        const AxisRegs ax = axis_regs(a.ax[m]);
         const int64_t base = frame_base(fr);
-        for (int r = 0; r < Sp; ++r) {
-          uint32_t v = rec[r * FT + fr];
-          if constexpr (!kOne) v |= symbol_at<kFrom>(a, base, (int)v, q, m).rec;
-          const int i = (int)(v & 511u);
-          bool eI = (v >> 21) & 1u, eQ = (v >> 22) & 1u;
-          // the neighbour differs from the hard level in the Gray label's bit ctz(threshold)
-          int pI = 2 * m * i + m - __ffs((int)((v >> 9) & 63u));
-          int pQ = 2 * m * i + 2 * m - __ffs((int)((v >> 15) & 63u));
-          if (!eI || pI >= N) pI = kNoPos;
-          if (!eQ || pQ >= N) pQ = kNoPos;
-          if (a.nearer && ((v >> 23) & 1u)) {  // the nearer (vertical) alternative takes the first slot
-            const int tp = pI; pI = pQ; pQ = tp;
-            const bool te = eI; eI = eQ; eQ = te;
+        float2 v[kRanks];
+        uint32_t idx[kRanks];
+#pragma unroll
+        for (int r = 0; r < kRanks; ++r) {
+          v[r] = make_float2(0.0f, 0.0f);
+          idx[r] = r < Sp ? rec[r * FT + fr] : 0u;
+          if constexpr (kOne) v[r] = s_sym[r * FT + fr];
+          else if constexpr (kFrom != kFromArrays) {
+            if (r < Sp) v[r] = a.symbols[base + idx[r]];
           }
-          rec[r * FT + fr] = (uint32_t)pI | ((uint32_t)pQ << 16);
-          ex |= ((eI ? 1u : 0u) | (eQ ? 2u : 0u)) << (2 * r);
+        }
+#pragma unroll
+        for (int r = 0; r < kRanks; ++r) {
+          Alt t;
+          if constexpr (kFrom == kFromArrays) t = array_alt(a, base + idx[r]);
+          else t = symbol_alt(v[r], ax, a.lik);
+          // the neighbour across threshold k differs from the hard level in
+          // the Gray label's bit ctz(k + 1)
+          const int pI = 2 * m * (int)idx[r] + m - __ffs((int)t.kI + 1);
+          const int pQ = 2 * m * (int)idx[r] + 2 * m - __ffs((int)t.kQ + 1);
+          uint32_t e0 = r < Sp && t.exI, e1 = r < Sp && t.exQ;
+          uint32_t p0 = e0 && pI < N ? (uint32_t)pI : kNoPos, p1 = e1 && pQ < N ? (uint32_t)pQ : kNoPos;
+          if (a.nearer && t.near) {  // the nearer (vertical) alternative takes the first slot
+            const uint32_t tp = p0, te = e0;
+            p0 = p1; p1 = tp;
+            e0 = e1; e1 = te;
+          }
+          if (r < Sp) rec[r * FT + fr] = p0 | (p1 << 16);
+          ex |= (e0 | (e1 << 1)) << (2 * r);
+          real |= ((p0 != kNoPos ? 1u : 0u) | (p1 != kNoPos ? 2u : 0u)) << (2 * r);
+          c[2 * r] = proj(p0);
+          c[2 * r + 1] = proj(p1);
         }
       }
 
@@ -634,10 +840,10 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       uint32_t f0;
       if (F.polar) {
         uint32_t* b = F.buf;
+        auto word = [&](int w) { return transform_word(__brev(b[w * stride])); };
         if (NW >= 4) {
           for (int w = 0; w < NW; w += 4) {
-            uint32_t x0 = transform_word(b[w * stride]), x1 = transform_word(b[(w + 1) * stride]);
-            uint32_t x2 = transform_word(b[(w + 2) * stride]), x3 = transform_word(b[(w + 3) * stride]);
+            uint32_t x0 = word(w), x1 = word(w + 1), x2 = word(w + 2), x3 = word(w + 3);
             x0 ^= x1; x2 ^= x3;
             x0 ^= x2; x1 ^= x3;
             b[w * stride] = x0; b[(w + 1) * stride] = x1; b[(w + 2) * stride] = x2; b[(w + 3) * stride] = x3;
@@ -648,65 +854,74 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
               b[w * stride] ^= b[(w + dw) * stride];
             }
         } else {
-          const uint32_t x0 = transform_word(b[0]);
+          const uint32_t x0 = word(0);
           b[0] = x0;
           if (NW == 2) {
-            const uint32_t x1 = transform_word(b[stride]);
+            const uint32_t x1 = word(1);
             b[stride] = x1;
             b[0] = x0 ^ x1;
           }
         }
         f0 = 0;
-        for (int w = 0; w < NW; ++w) {
-          const uint32_t s = b[w * stride] & __ldg(F.fmask + w);
-          b[w * stride] = s;
-          f0 = syndrome_fold(f0, s);
+        if (exact && NW > 1) {  // at most 32 frozen bits: packed as the columns are
+          for (int r = 0; r < code->R; ++r) {
+            const uint32_t i = __ldg(code->frozen + r);
+            f0 |= ((b[(i >> 5) * stride] >> (i & 31u)) & 1u) << r;
+          }
+        } else {
+          for (int w = 0; w < NW; ++w) {
+            const uint32_t s = b[w * stride] & __ldg(F.fmask + w);
+            b[w * stride] = s;
+            f0 = syndrome_fold(f0, s);
+          }
         }
       } else {
         f0 = s_f0[fr];
       }
 
-      // elimination: column b reduced by the earlier pivots, its combination
-      // of slots beside it; the base syndrome last
-      const Proj proj{F.polar ? code->hx : (exact ? code->hcol : code->hf)};
-      uint32_t c[kSlots], comb[kSlots];
-      uint32_t real = 0;  // existing slots whose flip lies inside the word
-#pragma unroll
-      for (int b = 0; b < kSlots; ++b) {
-        uint32_t p = kNoPos;
-        if ((ex >> b) & 1u) p = slot_pos(F, b);
-        c[b] = proj(p);
-        comb[b] = 1u << b;
-        real |= p != kNoPos ? 1u << b : 0u;
-      }
-      uint32_t s = f0, x0 = 0;
-      uint32_t kv[kSlots];
+      // Gauss-Jordan on the columns: the pivot of column j is its lowest row
+      // that no earlier pivot took; the rows of every later column and of the
+      // syndrome are reduced by it, so that a pivot row's bit is a coefficient:
+      // afterwards the syndrome's bits in the pivot rows are the solution,
+      // and a bit elsewhere says there is none. A column without a free row
+      // is the sum of the pivot columns named by its bits: a kernel vector.
+      uint32_t s = f0, used = 0, free_slots = 0;
+      uint32_t piv[kSlots], kv[kSlots];
       int d = 0;
 #pragma unroll
       for (int j = 0; j < kSlots; ++j) {
-        const uint32_t v = c[j], piv = v & (0u - v);
+        const uint32_t u = c[j] & ~used, p = u & (0u - u);
+        const uint32_t clear = c[j] ^ p;
+        piv[j] = p;
+        used |= p;
 #pragma unroll
         for (int k = j + 1; k < kSlots; ++k)
-          if (c[k] & piv) {
-            c[k] ^= v;
-            comb[k] ^= comb[j];
-          }
-        if (s & piv) {
-          s ^= v;
-          x0 ^= comb[j];
-        }
+          xor_if(c[k], p, clear);
+        xor_if(s, p, clear);
         // a slot that changes nothing (padding) is never part of the first
         // solution: leaving it out lowers the position
-        if (v == 0u && ((real >> j) & 1u)) kv[d++] = comb[j];
+        if (p == 0u && ((real >> j) & 1u)) {
+          free_slots |= 1u << j;
+          kv[d++] = c[j];
+        }
       }
       uint32_t x = kNone;
       unsigned long long ranked = 0;
-      if (s == 0u) {
-        if (d == 0) {
+      if (!(s & ~used)) {
+        auto pivots_of = [&](uint32_t v) {
+          uint32_t r = 0;
+#pragma unroll
+          for (int j = 0; j < kSlots; ++j) r |= (v & piv[j]) ? 1u << j : 0u;
+          return r;
+        };
+        const uint32_t x0 = pivots_of(s);
+        if (free_slots == 0) {
           const bool ok = exact || (F.polar ? consume_zero_polar(F, x0) : sum_zero(F, x0, true));
           if (ok) x = x0;
           ranked = ok ? 1 : 0;
         } else {
+          for (int t = 0; t < d; ++t, free_slots &= free_slots - 1u)
+            kv[t] = pivots_of(kv[t]) | (free_slots & (0u - free_slots));
           x = first_solution(F, proj, ex, Sp, f0, exact, x0, kv, d, &ranked);
         }
       }
@@ -751,9 +966,28 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   }
 }
 
-size_t decode_smem(bool mixed, int slots, int T, int NWmax) {
+size_t decode_smem(bool mixed, bool one, int slots, int T, int NWmax) {
   const size_t FT = (size_t)kWarps * T;
-  return (mixed ? FT * 20 : 0) + 4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
+  return (mixed ? FT * 24 + 512 : 0) + (one ? FT * 8 * (slots / 2) : 0) +
+         4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
+}
+
+// Constants of axes_fast for sqrt(M) = 2^m. t + 512 = round(a q) + 256 sqrt(M);
+// the nearest inner threshold (ties down) is k = floor((t + 255) / 512) =
+// round((t - 3/4) / 512) within [0, sqrt(M) - 2]; with one inner threshold
+// (QPSK) it is 0.
+AxisConst axis_const(int m, const QamConst& qc) {
+  const double side = (double)(1 << m), range = side - 2.0;
+  auto twice = [](double v) { return make_float2((float)v, (float)v); };
+  AxisConst c;
+  c.q = make_float2(qc.q[m], qc.q[m]);
+  c.t0 = twice(-(12582912.0 - 256.0 * side + 512.0));
+  c.g = twice(range);
+  c.s = m > 1 ? (float)(1.0 / (512.0 * range)) : 0.0f;
+  c.c = m > 1 ? (float)(-0.75 / (512.0 * range)) : 0.0f;
+  c.lim = (float)(256.0 * side + 1500.0);  // distances up to 2012: keys below 2^23
+  c.side = (float)side;
+  return c;
 }
 
 template <int kFrom, bool kOne>
@@ -779,19 +1013,21 @@ int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const int Smax = a.S < Lmax ? a.S : Lmax;
   const int slots = Smax <= 8 ? 16 : (Smax <= 10 ? 20 : 24);
   const bool mixed = a.desc != nullptr, arrays = !mixed && a.symbols == nullptr;
+  const bool one = !mixed && !arrays && Lmax <= 32;
+  const QamConst qc = make_qam_const();
+  for (int m = 1; m <= 6; ++m) a.ax[m] = axis_const(m, qc);
   // frames per warp: as many as keep every SM full (each CTA holds the tile's
-  // solve in its first warps, so larger tiles waste fewer lanes there), in
-  // equal waves
+  // solve in its first warps, so larger tiles waste fewer lanes there)
   const int64_t slots_cta = (int64_t)sm_count() * 7;
-  const int64_t waves = (a.n_frames + slots_cta * kWarps * 32 - 1) / (slots_cta * kWarps * 32);
-  const int64_t T = (a.n_frames + slots_cta * kWarps * waves - 1) / (slots_cta * kWarps * waves);
+  const int64_t T = (a.n_frames + slots_cta * kWarps - 1) / (slots_cta * kWarps);
+  a.m = m_of(a.M);
   a.T = (int)(T < 1 ? 1 : (T > 32 ? 32 : T));
   const int64_t grid = (a.n_frames + kWarps * a.T - 1) / (kWarps * a.T);
-  const size_t smem = decode_smem(mixed, slots, a.T, a.NWmax);
+  const size_t smem = decode_smem(mixed, one, slots, a.T, a.NWmax);
   const void* kern = mixed ? pick_slots<kFromMixed, false>(Smax)
                            : (arrays ? pick_slots<kFromArrays, false>(Smax)
-                                     : (Lmax <= 32 ? pick_slots<kFromUniform, true>(Smax)
-                                                   : pick_slots<kFromUniform, false>(Smax)));
+                                     : (one ? pick_slots<kFromUniform, true>(Smax)
+                                            : pick_slots<kFromUniform, false>(Smax)));
   if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB
   void* args[] = {&a};
   if (cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(32 * kWarps), args, smem, st) != cudaSuccess)

@@ -6,6 +6,17 @@
 
 namespace grand {
 
+// Demodulation constants of one constellation for the packed floating-point
+// arithmetic on both axes (axes_fast in fused.cu): each value twice.
+struct AxisConst {
+  float2 q;      // 256 / d
+  float2 t0;     // -(1.5 * 2^23 - 256 sqrt(M) + 512)
+  float2 g;      // sqrt(M) - 2: the range of the thresholds' indices
+  float s, c;    // t s + c: that range scaled to [0, 1]
+  float lim;     // |a q| up to which the ordering key is exact in 23 bits
+  float side;    // sqrt(M)
+};
+
 struct DecodeArgs {
   const float2* symbols;         // received symbols, or NULL: the demodulated arrays
   const uint16_t* hard_idx;
@@ -19,6 +30,7 @@ struct DecodeArgs {
   int n_codes;
   int64_t n_frames;
   int M, L;                      // uniform batch
+  int m;                         // log2(M) / 2 (set by launch_decode)
   int S;
   int lik;
   int nearer;                    // GRAND_ORDER_QAM_NEARER: swap h / v where d_Q < d_I
@@ -27,7 +39,7 @@ struct DecodeArgs {
   int NWmax;                     // words of the longest code (uniform batch: of the code)
   int T;                         // frames per warp (set by launch_decode)
   int64_t cap;
-  QamConst qc;
+  AxisConst ax[7];               // index m = log2(M) / 2
   uint32_t* cw;
   uint32_t* queries;
   uint8_t* abandon;
