@@ -95,7 +95,9 @@ typedef enum grand_order {
  *               (one kernel, no scratch memory). With an explicit tiles[0] or
  *               tiles[1], a deadline, or in the resumable search: syndrome
  *               deltas (Alg. 2 Step 4: s(y) xor the H columns a TEP flips)
- *               compared TEP by TEP in the split search. QAM_NNE5 runs DELTA.
+ *               compared TEP by TEP in the split search. QAM_NNE5: DELTA for
+ *               the lightest weights, then a hash join of the two halves of
+ *               the ranks (same outputs; stats count every TEP it decides).
  *   DELTA       syndrome deltas, one TEP per lane and step in canonical
  *               order (no split search); grand_decode_symbols only.
  *   ROW_PARITY  the candidate word y ^ e multiplied by H row by row, each
@@ -330,8 +332,8 @@ int grand_decode_batch(const grand_code* code, const grand_params* params, const
  * to memory. symbols as for grand_demod (M = params->M); outputs as for
  * grand_decode_batch. Every QAM order and membership test is accepted here;
  * QAM_NNE5 and membership DELTA / ROW_PARITY run the per-TEP kernel (one
- * warp per frame: demodulation, selection and the canonical walk), whose
- * stats report prep_ms = 0, the walk in search_ms, hard_frames = frames
+ * warp per frame: demodulation, selection and the canonical walk; with AUTO
+ * the join), whose stats report prep_ms = 0, the kernel in search_ms, hard_frames = frames
  * whose first query failed and search_useful = their queries. */
 int grand_decode_symbols(const grand_code* code, const grand_params* params, const void* symbols,
                          int64_t n_frames, float N0, uint32_t* cw, uint32_t* queries, uint8_t* abandon,

@@ -16,6 +16,16 @@
 //               odd row.
 // Results equal those of the split search (and of the CPU oracle) for every
 // order; only the work per TEP differs.
+//
+// The five-point order with the library's choice of the test (AUTO) walks only
+// the lightest weights and then joins the two halves of the ranks (k_per_tep<true>):
+// a CTA of four warps prepares four frames, and each frame they leave open is
+// decided by all of them -- the partial syndromes of the lower ranks (at most
+// 5^5 = 3,125) go into a hash table in shared memory and those of the upper
+// ranks are looked up. 6,250 table steps take the place of up to 5^10 =
+// 9,765,625 TEPs tested one by one: 6,000 frames (N=128 16-QAM, 6/8/10 dB,
+// S=10, cap 2^20) 32 ms -> 0.12 ms. What is left is latency (37 % issue): the
+// CTA's warps wait for one another between the preparation and the joins.
 
 #include <stdint.h>
 
@@ -28,12 +38,17 @@ namespace {
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr int kAltMax = 4;  // alternatives per symbol (five-point NNE)
 constexpr int kTepWarps = 4;
+constexpr int kSlotBits = 13;        // hash slots: 2.6 per entry of a full side
+constexpr int kSlots = 1 << kSlotBits;
+constexpr int kJoinStep = 5;         // table accesses a thread keeps in flight
+constexpr int kLowRanks = 3;         // ranks of a side spread over the threads (5^3 <= 128)
 
 struct TepArgs {
   CodeDev code;
   const float2* symbols;
   int64_t n_frames;
   int m, side, L, Sp;
+  int walk;                      // weights walked before the join
   int lik, order, rowparity;
   float q;
   uint32_t cap;
@@ -100,13 +115,176 @@ __device__ bool delta_zero(const CodeDev& code, const uint32_t* s0, const uint32
   return true;
 }
 
+// One frame's ranks as the join sees them.
+struct JoinFrame {
+  const uint32_t* s0;
+  const uint32_t* apos;
+  const uint32_t* aproj;
+  const uint8_t* kk;
+  uint32_t f0;
+  int Sp;
+};
+
+// A vector of digits (3 bits per rank: 0 unchanged, else alternative + 1) and
+// its projection.
+struct Part {
+  uint32_t code, z;
+};
+
+// The index-th digit vector of ranks [r0, r0 + n), rank r0 the fastest, radix
+// alternatives + 1; `over`: index beyond the last.
+__device__ __forceinline__ Part join_part(const JoinFrame& f, int r0, int n, uint32_t index, bool& over) {
+  Part p{0u, 0u};
+  for (int r = r0; r < r0 + n; ++r) {
+    const uint32_t radix = (uint32_t)f.kk[r] + 1u;
+    const uint32_t d = index % radix;
+    index /= radix;
+    p.code |= d << (3 * r);
+    if (d) p.z ^= f.aproj[r * kAltMax + d - 1];
+  }
+  over = index != 0;
+  return p;
+}
+
+// Order of the TEPs as an integer: weight, altered ranks in colex order (the
+// mask as a number), alternatives from the largest rank down (the code).
+__device__ __forceinline__ unsigned long long join_key(uint32_t code) {
+  uint32_t m = 0;
+  for (int r = 0; r < GRAND_S_MAX_NNE5; ++r) m |= (((code >> (3 * r)) & 7u) ? 1u : 0u) << r;
+  return ((unsigned long long)__popc(m) << 40) | ((unsigned long long)m << 30) | code;
+}
+
+// Ranks and alternative indices of a code, packed as delta_zero takes them.
+__device__ __forceinline__ int join_unpack(uint32_t code, uint64_t& pp, uint32_t& dg) {
+  int w = 0;
+  pp = 0;
+  dg = 0;
+  for (int r = 0; r < GRAND_S_MAX_NNE5; ++r) {
+    const uint32_t d = (code >> (3 * r)) & 7u;
+    if (!d) continue;
+    pp |= (uint64_t)r << (4 * w);
+    dg |= (d - 1u) << (2 * w);
+    ++w;
+  }
+  return w;
+}
+
+// Hash join of the lower ranks [0, S'/2) with the upper ones, by the whole
+// CTA. A thread holds one digit vector of a side's first three ranks and goes
+// through those of the other two (at most 25, kept in `high`), kJoinStep table
+// accesses in flight at a time. Slots hold 20 bits of the mixed key and the
+// entry's number + 1 (low index + 128 x high index); equal ones are confirmed
+// on every syndrome word. *best: the smallest join_key of a codeword
+// (initialised by the caller).
+__device__ void join_sides(const CodeDev& code, const JoinFrame& f, uint32_t* table, uint2 (*high)[32],
+                           unsigned long long* best) {
+  constexpr int kThreads = 32 * kTepWarps;
+  const int nA = f.Sp >> 1, nB = f.Sp - nA;
+  const int loA = min(nA, kLowRanks), loB = min(nB, kLowRanks);
+  const uint32_t t = threadIdx.x;
+  uint4* t4 = reinterpret_cast<uint4*>(table);
+  for (int i = (int)t; i < kSlots / 4; i += kThreads) t4[i] = make_uint4(0u, 0u, 0u, 0u);
+  uint32_t sizeA = 1, sizeB = 1;  // digit vectors of the ranks after the first three
+  for (int r = loA; r < nA; ++r) sizeA *= f.kk[r] + 1u;
+  for (int r = nA + loB; r < f.Sp; ++r) sizeB *= f.kk[r] + 1u;
+  bool over, none;
+  if (t < 64) {
+    const Part p = t < 32 ? join_part(f, loA, nA - loA, t, over) : join_part(f, nA + loB, nB - loB, t - 32u, over);
+    high[t >> 5][t & 31u] = make_uint2(p.code, p.z);
+  }
+  __syncthreads();
+  {
+    const Part lo = join_part(f, 0, loA, t, over);
+    const uint32_t z0 = f.f0 ^ lo.z;
+    for (uint32_t h0 = 0; !over && h0 < sizeA; h0 += kJoinStep) {
+      uint32_t k[kJoinStep], was[kJoinStep];
+#pragma unroll
+      for (int u = 0; u < kJoinStep; ++u) {
+        const uint32_t h = h0 + u;
+        k[u] = (z0 ^ high[0][h & 31u].y) * 0x9E3779B1u;
+        was[u] = h < sizeA ? atomicCAS(table + (k[u] >> (32 - kSlotBits)), 0u, (k[u] << 12) | (t + 128u * h + 1u)) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kJoinStep; ++u) {  // taken: the next free slot
+        uint32_t slot = k[u] >> (32 - kSlotBits);
+        while (was[u] != 0u) {
+          slot = (slot + 1u) & (kSlots - 1u);
+          was[u] = atomicCAS(table + slot, 0u, (k[u] << 12) | (t + 128u * (h0 + u) + 1u));
+        }
+      }
+    }
+  }
+  __syncthreads();
+  {
+    const Part lo = join_part(f, nA, loB, t, over);
+    for (uint32_t h0 = 0; !over && h0 < sizeB; h0 += kJoinStep) {
+      uint32_t k[kJoinStep], seen[kJoinStep];
+#pragma unroll
+      for (int u = 0; u < kJoinStep; ++u) {
+        const uint32_t h = h0 + u;
+        k[u] = (lo.z ^ high[1][h & 31u].y) * 0x9E3779B1u;
+        seen[u] = h < sizeB ? table[k[u] >> (32 - kSlotBits)] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kJoinStep; ++u) {
+        uint32_t slot = k[u] >> (32 - kSlotBits);
+        for (uint32_t e = seen[u]; e != 0u; e = table[slot]) {
+          slot = (slot + 1u) & (kSlots - 1u);
+          if ((e ^ (k[u] << 12)) >> 12) continue;
+          const uint32_t n = (e & 4095u) - 1u;
+          const uint32_t c = lo.code | high[1][h0 + u].x | join_part(f, 0, loA, n & 127u, none).code | high[0][n >> 7].x;
+          const unsigned long long key = join_key(c);
+          if (key >= *(volatile unsigned long long*)best) continue;
+          uint64_t pp;
+          uint32_t dg;
+          const int w = join_unpack(c, pp, dg);
+          if (delta_zero(code, f.s0, f.apos, pp, dg, w)) atomicMin(best, key);
+        }
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// Position of a TEP among the valid ones (1-based), by one warp: lane v holds
+// the number of valid TEPs altering exactly v of the ranks passed so far.
+__device__ uint32_t join_position(const JoinFrame& f, uint32_t code) {
+  const int v = threadIdx.x & 31;
+  uint32_t e = v == 0 ? 1u : 0u, acc = 0, alt = 0, low = 1;
+  int w = 0;
+  for (int r = 0; r < f.Sp; ++r) {
+    const uint32_t k = f.kk[r], d = (code >> (3 * r)) & 7u;
+    if (d) {
+      ++w;
+      acc = acc * k + __shfl_sync(kAll, e, w);
+      alt += (d - 1u) * low;
+      low *= k;
+    }
+    uint32_t up = __shfl_up_sync(kAll, e, 1);
+    if (v == 0) up = 0;
+    e += k * up;
+  }
+  return __reduce_add_sync(kAll, v < w ? e : 0u) + acc + alt + 1u;
+}
+
+// kJoin: the five-point order with the join (see the head of the file); the
+// CTA's warps then take four consecutive frames together.
+template <bool kJoin>
 __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
+  __shared__ unsigned s_first;
+  __shared__ uint2 s_high[2][32];
+  __shared__ uint32_t s_f0[kTepWarps];
+  __shared__ int s_open[kTepWarps];
+  __shared__ unsigned long long s_best[kTepWarps];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const CodeDev& code = a.code;
   const int N = code.N, NW = N >> 5, L = a.L, Sp = a.Sp, m = a.m;
-  char* base = smem_raw + (size_t)warp * tep_warp_bytes(L, NW, a.rowparity);
+  const size_t warp_bytes = tep_warp_bytes(L, NW, a.rowparity);
+  uint32_t* table = reinterpret_cast<uint32_t*>(smem_raw);  // [kSlots], join only
+  char* const bases = smem_raw + (kJoin ? sizeof(uint32_t) * kSlots : 0);
+  char* base = bases + (size_t)warp * warp_bytes;
   uint32_t* y = reinterpret_cast<uint32_t*>(base);
   uint32_t* s0 = y + 32;
   uint32_t* apos = s0 + kWMax;
@@ -120,10 +298,35 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
 
   for (;;) {
     unsigned int fi = 0;
-    if (lane == 0) fi = atomicAdd(a.next, 1u);
-    fi = __shfl_sync(kAll, fi, 0);
-    if ((int64_t)fi >= a.n_frames) break;
+    bool walk = true;  // this warp has a frame to search
+    if constexpr (kJoin) {
+      __syncthreads();  // the last round's shared words have been read
+      if (threadIdx.x == 0) s_first = atomicAdd(a.next, (unsigned)kTepWarps);
+      if (lane == 0) {
+        s_open[warp] = 0;
+        s_best[warp] = ~0ull;
+      }
+      __syncthreads();
+      if ((int64_t)s_first >= a.n_frames) break;
+      fi = s_first + (unsigned)warp;
+      walk = (int64_t)fi < a.n_frames;
+    } else {
+      if (lane == 0) fi = atomicAdd(a.next, 1u);
+      fi = __shfl_sync(kAll, fi, 0);
+      if ((int64_t)fi >= a.n_frames) break;
+    }
     const int64_t f = fi;
+    uint32_t f0 = 0;
+    const uint32_t cap = a.cap;
+    uint32_t cum = 0;  // valid TEPs of the batches already walked
+    bool found = false;
+    uint32_t hit_rank = 0;
+    int hit_lane = -1, w_hit = 0;
+    // the lane's TEP, packed: pp = ranks (4 bits per position, ascending),
+    // dg = alternative indices (2 bits), km = alternatives - 1 (2 bits)
+    uint64_t pp = 0;
+    uint32_t dg = 0, km = 0;
+    if (walk) {
 
     // --- Step 1: demodulation and the hard word --------------------------
     if (lane < NW) y[lane] = 0u;
@@ -156,9 +359,9 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
         a.abandon[f] = 2;
       }
       __syncwarp();
-      continue;
+      walk = false;
     }
-    if (a.deadline > 0) {
+    if (walk && a.deadline > 0) {
       int cut = 0;
       if (lane == 0) cut = past_deadline(a.t0, a.deadline);
       if (__shfl_sync(kAll, cut, 0)) {  // fetched after the deadline: the hard word, marked 5
@@ -169,12 +372,13 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
           atomicOr(code.status, 1u);
         }
         __syncwarp();
-        continue;
+        walk = false;
       }
     }
+    }
+    if (walk) {
 
     // --- base syndrome s0 = H y and its projection (delta test) ----------
-    uint32_t f0 = 0;
     if (!a.rowparity) {
       uint32_t s[kWMax];
 #pragma unroll
@@ -255,16 +459,8 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
     __syncwarp();
 
     // --- Step 5: the canonical walk ----------------------------------------
-    const uint32_t cap = a.cap;
-    uint32_t cum = 0;  // valid TEPs of the batches already walked
-    bool found = false;
-    uint32_t hit_rank = 0;
-    int hit_lane = -1, w_hit = 0;
-    // the lane's TEP, packed: pp = ranks (4 bits per position, ascending),
-    // dg = alternative indices (2 bits), km = alternatives - 1 (2 bits)
-    uint64_t pp = 0;
-    uint32_t dg = 0, km = 0;
-    for (int w = 0; w <= Sp && !found && cum < cap; ++w) {
+    const int w_end = kJoin ? min(Sp, a.walk) : Sp;
+    for (int w = 0; w <= w_end && !found && cum < cap; ++w) {
       const uint32_t nsets = binom16(Sp, w);
       for (uint32_t b0 = 0; b0 < nsets && !found && cum < cap;) {
         // m sets in this batch, P lanes per set: lane l takes part l % P of
@@ -375,6 +571,47 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
       }
     }
 
+    }
+
+    // --- Step 5, the rest of an open frame by the join -----------------------
+    if constexpr (kJoin) {
+      if (walk && lane == 0 && !found && cum < cap && Sp > a.walk) {
+        s_open[warp] = 1;
+        s_f0[warp] = f0;
+      }
+      __syncthreads();
+      for (int q = 0; q < kTepWarps; ++q) {
+        if (!s_open[q]) continue;
+        const uint32_t* b = reinterpret_cast<const uint32_t*>(bases + (size_t)q * warp_bytes);
+        JoinFrame fr;
+        fr.s0 = b + 32;
+        fr.apos = fr.s0 + kWMax;
+        fr.aproj = fr.apos + kSMax * kAltMax;
+        fr.kk = reinterpret_cast<const uint8_t*>(fr.aproj + kSMax * kAltMax + kSMax);
+        fr.f0 = s_f0[q];
+        fr.Sp = Sp;
+        join_sides(code, fr, table, s_high, &s_best[q]);
+        if (q == warp) {
+          uint32_t total = 1;  // valid TEPs: at most 5^10
+          for (int r = 0; r < Sp; ++r) total *= kk[r] + 1u;
+          if (lane == 0) n_eval += total - cum;
+          cum = total;
+          const unsigned long long best = s_best[q];
+          if (best != ~0ull) {
+            const uint32_t c = (uint32_t)best & 0x3FFFFFFFu;
+            const uint32_t pos = join_position(fr, c);
+            if (pos <= cap) {
+              found = true;
+              hit_rank = pos;
+              hit_lane = 0;
+              w_hit = join_unpack(c, pp, dg);
+            }
+          }
+        }
+      }
+    }
+    if (!walk) continue;
+
     // --- Return: x = y xor e of the first hit, else y ---------------------
     if (found && lane == hit_lane) {
       for (int j = 0; j < w_hit; ++j) {
@@ -433,6 +670,15 @@ int run_per_tep(const grand_code* c, const grand_params* p, const void* symbols,
   a.cw = cw;
   a.queries = queries;
   a.abandon = abandon;
+  // the join decides every TEP at once; DELTA and ROW_PARITY ask for the test
+  // of each
+  const bool join = p->order == GRAND_ORDER_QAM_NNE5 && p->membership == GRAND_MEMBERSHIP_AUTO;
+  // Weight 1 (41 TEPs) decides most frames that decode; walking weight 2 (720
+  // more) costs more than it saves the join (134 against 125 us for 6,000 N=128
+  // frames), except where it decides nearly every frame: with few parity bits,
+  // whose space is full of codewords for the join to compare.
+  a.walk = c->R <= 12 ? 2 : 1;
+  auto kern = join ? k_per_tep<true> : k_per_tep<false>;
   char* scratch = nullptr;
   if (scratch_alloc((void**)&scratch, 64, st) != cudaSuccess) return GRAND_E_NOMEM;
   a.next = reinterpret_cast<unsigned int*>(scratch);
@@ -443,14 +689,17 @@ int run_per_tep(const grand_code* c, const grand_params* p, const void* symbols,
   cudaEvent_t ev[2] = {nullptr, nullptr};
   do {
     if (cudaMemsetAsync(scratch, 0, 64, st) != cudaSuccess) { rc = GRAND_E_CUDA; break; }
-    const size_t smem = kTepWarps * tep_warp_bytes(a.L, c->N / 32, a.rowparity);
+    const size_t smem =
+        (join ? sizeof(uint32_t) * kSlots : 0) + kTepWarps * tep_warp_bytes(a.L, c->N / 32, a.rowparity);
+    // (a fixed limit for the join: a concurrent call's larger frames are never undercut)
+    const size_t limit = join ? 64 * 1024 : smem;
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_per_tep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess) {
       rc = GRAND_E_CUDA;
       break;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_per_tep, 32 * kTepWarps, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTepWarps, smem) != cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
     const int64_t want = (n_frames + kTepWarps - 1) / kTepWarps;
@@ -462,7 +711,7 @@ int run_per_tep(const grand_code* c, const grand_params* p, const void* symbols,
       if (rc) break;
       cudaEventRecord(ev[0], st);
     }
-    k_per_tep<<<grid, 32 * kTepWarps, smem, st>>>(a);
+    kern<<<grid, 32 * kTepWarps, smem, st>>>(a);
     if (cudaGetLastError() != cudaSuccess) { rc = GRAND_E_CUDA; break; }
     if (stats) {
       cudaEventRecord(ev[1], st);
