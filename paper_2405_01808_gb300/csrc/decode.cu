@@ -24,8 +24,8 @@
 //   k_search       the split with one CTA per frame (explicit split in the
 //                  launch shape): one projection compare per TEP.
 //   k_ab           bit-level GRAND-AB (Sec. I), one warp per frame.
-//   k_demod        the public demodulation call (per-symbol outputs).
-// The five-point NNE order and the per-TEP membership tests are in per_tep.cu.
+// The public demodulation call is in demod.cu,
+// the five-point NNE order and the per-TEP membership tests are in per_tep.cu.
 #include <stdio.h>
 
 #include <mutex>
@@ -2405,189 +2405,8 @@ __global__ void __launch_bounds__(128) k_ab_split(AbArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Public demodulation: one thread per symbol
-// ---------------------------------------------------------------------------
-struct DemodArgs {
-  const float2* symbols;
-  int64_t n_sym;
-  int L, m, side, N, NW, lik;
-  float q, inv_d;
-  uint16_t* hard_idx;
-  uint32_t* key;
-  uint8_t* nmask;
-  float* rel;
-  uint32_t* y;
-  uint64_t Lmagic;  // ceil(2^64 / L): frame of symbol s = high word of s * Lmagic (exact for s < 2^64 / L)
-};
-
-// One symbol of the public demodulation call (outputs that are NULL are
-// skipped); rl = the symbol's Gray label bits in transmission order (bit k =
-// label bit 2m-1-k), for the hard word. kM = log2(sqrt(M)) is a template
-// argument so that the level arithmetic folds into constants.
-// Square root by the SFU's approximate instruction (relative error about
-// 2^-22, far inside the 1e-5 tolerance of the reported likelihood).
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-template <int kM, int kLit>
-__device__ __forceinline__ void demod_one(const DemodArgs& a, float2 v, uint16_t& hidx, uint32_t& key, uint8_t& nmask,
-                                          float& rel, uint32_t& rl) {
-  const bool nf = !(isfinite(v.x) && isfinite(v.y));
-  if (nf) v = make_float2(0.0f, 0.0f);
-  const AxisDemod I = demod_axis_q(v.x, a.q, 1 << kM, kLit);
-  const AxisDemod Q = demod_axis_q(v.y, a.q, 1 << kM, kLit);
-  hidx = (uint16_t)((I.level << 8) | Q.level);
-  key = (uint32_t)I.dq * (uint32_t)I.dq + (uint32_t)Q.dq * (uint32_t)Q.dq;
-  nmask = (uint8_t)make_nmask(I, Q, nf);
-  if (a.rel) {
-    const float dI = axis_dist_f32(v.x, a.inv_d, I.amp, I.outside, kLit);
-    const float dQ = axis_dist_f32(v.y, a.inv_d, Q.amp, Q.outside, kLit);
-    rel = sqrt_approx(dI * dI + dQ * dQ);
-  }
-  const uint32_t label = ((uint32_t)gray_code(I.level) << kM) | (uint32_t)gray_code(Q.level);
-  rl = __brev(label) >> (32 - 2 * kM);
-}
-
-// OR `bits` (at most 24) into the packed hard word yf at bit position p0;
-// words at or beyond NW (bits >= N: padding) are dropped.
-__device__ __forceinline__ void or_bits(uint32_t* yf, int NW, int p0, uint32_t bits) {
-  const int wd = p0 >> 5, sh = p0 & 31;
-  const uint32_t lo = bits << sh, hi = sh ? (bits >> (32 - sh)) : 0u;
-  if (wd < NW && lo) atomicOr(yf + wd, lo);
-  if (hi && wd + 1 < NW) atomicOr(yf + wd + 1, hi);
-}
-
-// Two symbols per thread: 16-byte loads, paired stores (every pointer aligned
-// for its pair type, checked by the host); otherwise one symbol per thread.
-// The frame of a symbol is found once per thread and then advanced by the
-// grid stride (a quotient and remainder of the stride by L, no division per
-// step); the pair's label bits go into the hard word with one OR when both
-// symbols belong to the same frame. kLit: the likelihood reading (selects
-// fold into constants).
-template <bool kPaired, int kM, int kLit>
-__global__ void __launch_bounds__(256, 8) k_demod(DemodArgs a) {
-  constexpr int b2 = 2 * kM;
-  const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
-  if constexpr (!kPaired) {
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.n_sym; s += gstride) {
-      uint16_t h0;
-      uint32_t k0, rl0;
-      uint8_t m0;
-      float r0 = 0.0f;
-      demod_one<kM, kLit>(a, a.symbols[s], h0, k0, m0, r0, rl0);
-      if (a.hard_idx) a.hard_idx[s] = h0;
-      if (a.key) a.key[s] = k0;
-      if (a.nmask) a.nmask[s] = m0;
-      if (a.rel) a.rel[s] = r0;
-      if (a.y) {
-        const int64_t f = (int64_t)__umul64hi((uint64_t)s, a.Lmagic);
-        const int i = (int)(s - f * a.L);
-        or_bits(a.y + f * a.NW, a.NW, b2 * i, rl0);
-      }
-    }
-    return;
-  }
-  const int64_t n_pairs = a.n_sym >> 1;
-  const float4* sym4 = reinterpret_cast<const float4*>(a.symbols);
-  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  // frame f and symbol i of this thread's first pair, and the symbol stride
-  // 2 * gstride = dq frames + dr symbols
-  int64_t f = (int64_t)__umul64hi((uint64_t)(2 * t0), a.Lmagic);
-  int i = (int)(2 * t0 - f * a.L);
-  const int64_t dq = (int64_t)__umul64hi((uint64_t)(2 * gstride), a.Lmagic);
-  const int dr = (int)(2 * gstride - dq * a.L);
-  for (int64_t t = t0; t <= n_pairs; t += gstride) {
-    const int64_t s = 2 * t;
-    if (t < n_pairs) {
-      const float4 v = sym4[t];
-      uint16_t h0, h1;
-      uint32_t k0, k1, rl0, rl1;
-      uint8_t m0, m1;
-      float r0 = 0.0f, r1 = 0.0f;
-      demod_one<kM, kLit>(a, make_float2(v.x, v.y), h0, k0, m0, r0, rl0);
-      demod_one<kM, kLit>(a, make_float2(v.z, v.w), h1, k1, m1, r1, rl1);
-      if (a.hard_idx) reinterpret_cast<ushort2*>(a.hard_idx)[t] = make_ushort2(h0, h1);
-      if (a.key) reinterpret_cast<uint2*>(a.key)[t] = make_uint2(k0, k1);
-      if (a.nmask) reinterpret_cast<uchar2*>(a.nmask)[t] = make_uchar2(m0, m1);
-      if (a.rel) reinterpret_cast<float2*>(a.rel)[t] = make_float2(r0, r1);
-      if (a.y) {
-        uint32_t* yf = a.y + f * a.NW;
-        if (i + 1 < a.L) {
-          or_bits(yf, a.NW, b2 * i, rl0 | (rl1 << b2));
-        } else {  // the pair straddles two frames
-          or_bits(yf, a.NW, b2 * i, rl0);
-          or_bits(yf + a.NW, a.NW, 0, rl1);
-        }
-      }
-    } else if (s < a.n_sym) {  // odd count: the last symbol
-      uint16_t h0;
-      uint32_t k0, rl0;
-      uint8_t m0;
-      float r0 = 0.0f;
-      demod_one<kM, kLit>(a, a.symbols[s], h0, k0, m0, r0, rl0);
-      if (a.hard_idx) a.hard_idx[s] = h0;
-      if (a.key) a.key[s] = k0;
-      if (a.nmask) a.nmask[s] = m0;
-      if (a.rel) a.rel[s] = r0;
-      if (a.y) or_bits(a.y + f * a.NW, a.NW, b2 * i, rl0);
-    }
-    // advance to the next pair of this thread
-    f += dq;
-    i += dr;
-    if (i >= a.L) {
-      i -= a.L;
-      f += 1;
-    }
-  }
-}
-
-// BPSK hard decisions: one warp per 32 samples
-__global__ void __launch_bounds__(256) k_demod_bpsk(const float* r, int64_t n_words, uint32_t* y, uint8_t* nmask) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_words;
-       w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    float v = r[32 * w + lane];
-    const bool nf = !isfinite(v);
-    if (nf) v = 0.0f;
-    const unsigned b = __ballot_sync(kFull, v < 0.0f);
-    if (lane == 0 && y) y[w] = b;
-    if (nmask) nmask[32 * w + lane] = nf ? 128 : 0;
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-
-template <int kM>
-static void launch_demod_m(const DemodArgs& a, bool paired, int grid, cudaStream_t st) {
-  if (a.lik == GRAND_LIK_LITERAL) {
-    if (paired)
-      k_demod<true, kM, 1><<<grid, 256, 0, st>>>(a);
-    else
-      k_demod<false, kM, 1><<<grid, 256, 0, st>>>(a);
-  } else {
-    if (paired)
-      k_demod<true, kM, 0><<<grid, 256, 0, st>>>(a);
-    else
-      k_demod<false, kM, 0><<<grid, 256, 0, st>>>(a);
-  }
-}
-
-// m = log2(sqrt(M)) in 1..6 (validated by the caller).
-static void launch_demod(const DemodArgs& a, bool paired, int grid, cudaStream_t st) {
-  switch (a.m) {
-    case 1: launch_demod_m<1>(a, paired, grid, st); break;
-    case 2: launch_demod_m<2>(a, paired, grid, st); break;
-    case 3: launch_demod_m<3>(a, paired, grid, st); break;
-    case 4: launch_demod_m<4>(a, paired, grid, st); break;
-    case 5: launch_demod_m<5>(a, paired, grid, st); break;
-    default: launch_demod_m<6>(a, paired, grid, st); break;
-  }
-}
 
 typedef void (*PrepKernel)(PrepArgs);
 static PrepKernel prep_kernel_for(int Wmax) {
@@ -3045,55 +2864,6 @@ static int run_ab(const grand_code* c, const grand_params* p, const float* sampl
 }  // namespace grand
 
 using namespace grand;
-
-extern "C" int grand_demod(const void* symbols, int64_t n_frames, int L, int M, float N0, int lik_variant,
-                           uint16_t* hard_idx, uint32_t* key, uint8_t* nmask, float* rel, uint32_t* y, int N,
-                           void* stream) {
-  if ((!symbols && n_frames > 0) || n_frames < 0 || !(N0 > 0.0f) || !isfinite(N0)) return GRAND_E_INVALID;
-  if (N < GRAND_N_MIN || N > GRAND_N_MAX || (N & (N - 1))) return GRAND_E_INVALID;
-  if (lik_variant != GRAND_LIK_THRESHOLD && lik_variant != GRAND_LIK_LITERAL) return GRAND_E_INVALID;
-  cudaStream_t st = (cudaStream_t)stream;
-  if (M == 2) {
-    if (L != N) return GRAND_E_INVALID;
-    if (n_frames == 0) return GRAND_OK;
-    const int64_t n_words = n_frames * (N / 32);
-    const int64_t blocks = (n_words * 32 + 255) / 256;
-    k_demod_bpsk<<<(int)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, st>>>((const float*)symbols, n_words, y,
-                                                                                  nmask);
-    return cudaGetLastError() == cudaSuccess ? GRAND_OK : GRAND_E_CUDA;
-  }
-  const int m = m_of(M);
-  if (!m || L != (N + 2 * m - 1) / (2 * m)) return GRAND_E_INVALID;
-  if (n_frames == 0) return GRAND_OK;
-  const QamConst qc = make_qam_const();
-  DemodArgs a{};
-  a.symbols = (const float2*)symbols;
-  a.n_sym = n_frames * L;
-  a.L = L;
-  a.m = m;
-  a.side = 1 << m;
-  a.N = N;
-  a.NW = N / 32;
-  a.lik = lik_variant;
-  a.q = qc.q[m];
-  a.inv_d = qc.inv_d[m];
-  a.hard_idx = hard_idx;
-  a.key = key;
-  a.nmask = nmask;
-  a.rel = rel;
-  a.y = y;
-  a.Lmagic = UINT64_MAX / (uint64_t)L + 1;  // L >= 3 for the supported N and M
-  if (y && cudaMemsetAsync(y, 0, sizeof(uint32_t) * (size_t)n_frames * (N / 32), st) != cudaSuccess)
-    return GRAND_E_CUDA;
-  auto aligned = [](const void* p, uintptr_t b) { return ((uintptr_t)p % b) == 0; };
-  const bool paired = aligned(a.symbols, 16) && aligned(a.hard_idx, 4) && aligned(a.key, 8) &&
-                      aligned(a.nmask, 2) && aligned(a.rel, 8);
-  const int64_t per_thread = paired ? 2 : 1;
-  const int64_t blocks = ((a.n_sym + per_thread - 1) / per_thread + 255) / 256;
-  const int grid = (int)(blocks < (int64_t)sm_count() * 32 ? blocks : (int64_t)sm_count() * 32);
-  launch_demod(a, paired, grid, st);
-  return cudaGetLastError() == cudaSuccess ? GRAND_OK : GRAND_E_CUDA;
-}
 
 extern "C" int grand_decode_batch(const grand_code* c, const grand_params* p, const uint16_t* hard_idx,
                                   const uint32_t* key, const uint8_t* nmask, const uint32_t* y, int64_t n_frames,

@@ -25,6 +25,7 @@
 //          where a warp per frame spent a ballot and a shuffle per slot on one.
 #include <type_traits>
 
+#include "axis.cuh"
 #include "device_common.cuh"
 #include "fused.cuh"
 #include "host_util.cuh"
@@ -38,7 +39,6 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kKeySat = 0x7FFFFEu; // packed selection keys hold 23 bits of the reliability
 constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low bits) without a symbol
 constexpr uint32_t kPicked = 0xFFFFFFE0u;  // above those: a key taken as rank (low bits)
-constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to the nearest integer, ties to even
 constexpr int kLanePick = 3;            // smallest keys kept per lane of a long frame
 
 // e_v(n1, n3): valid TEPs altering exactly v of n1 ranks with one alternative
@@ -66,87 +66,6 @@ constexpr EspTable make_esp() {
 }
 __device__ const EspTable g_esp = make_esp();
 
-// Two floats in one 64-bit register pair, one instruction for both.
-typedef unsigned long long F2;
-__device__ __forceinline__ F2 pack2(float a, float b) {
-  F2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ F2 pack2(float2 v) { return pack2(v.x, v.y); }
-__device__ __forceinline__ float2 unpack2(F2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-  F2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ F2 add2(F2 a, F2 b) {
-  F2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-  F2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-// Both axes of a symbol on the Q8.8 grid (the reading of demod_axis_q) in
-// floating point: the integers involved are below 2^24, so every step is
-// exact, the FMA pipe takes what would crowd the integer ALU, and the packed
-// forms do I and Q in one instruction (about 10 instructions for what took
-// 50 in integer form). x = a q rounded to float. k = index of the inner
-// decision threshold nearest to the received value (threshold k separates the
-// levels k and k + 1), e = the signed distance to it. Ties between two
-// thresholds go to the lower one, so that the neighbour of a value on a level
-// is the lower level; |e| > 256 says the value lies beyond the outermost level,
-// where the far threshold has no neighbour level. For |x| up to 2^22; beyond,
-// k stays right and |e| stays above 256.
-struct Axes {
-  float2 kb;  // k plus 1.5 * 2^23: k in the low 6 bits of the representation
-  float2 k, e;
-};
-
-// The constants of one constellation in registers. The empty statements keep
-// the compiler from building the pairs anew for every symbol (packed
-// instructions take no immediates), which was 30 of 240 instructions a frame.
-struct AxisRegs {
-  F2 q, t0, g, magic, unmagic, m512;
-  float s, c, lim, side;
-};
-__device__ __forceinline__ AxisRegs axis_regs(const AxisConst& a) {
-  AxisRegs r;
-  r.q = pack2(a.q);
-  r.t0 = pack2(a.t0);
-  r.g = pack2(a.g);
-  r.magic = pack2(kMagic, kMagic);
-  r.unmagic = pack2(-kMagic, -kMagic);
-  r.m512 = pack2(-512.0f, -512.0f);
-  asm volatile("" : "+l"(r.q), "+l"(r.t0), "+l"(r.g), "+l"(r.magic), "+l"(r.unmagic), "+l"(r.m512));
-  r.s = a.s;
-  r.c = a.c;
-  r.lim = a.lim;
-  r.side = a.side;
-  return r;
-}
-__device__ __forceinline__ Axes axes_fast(F2 x, const AxisRegs& c) {
-  const F2 t = add2(add2(x, c.magic), c.t0);  // round(x) + 256 sqrt(M) - 512
-  const float2 ts = unpack2(t);
-  // threshold index: the nearest one, clamped to the inner thresholds by the
-  // saturation, rounded by the addition; no value lies on a tie (the offset is
-  // a quarter of the grid)
-  const float uI = __saturatef(__fmaf_rn(ts.x, c.s, c.c)), uQ = __saturatef(__fmaf_rn(ts.y, c.s, c.c));
-  const F2 kb = fma2(pack2(uI, uQ), c.g, c.magic);
-  const F2 k = add2(kb, c.unmagic);
-  Axes r;
-  r.kb = unpack2(kb);
-  r.k = unpack2(k);
-  r.e = unpack2(fma2(k, c.m512, t));
-  return r;
-}
 // Distance of the ordering key (threshold or literal reading), unclamped above.
 __device__ __forceinline__ float axis_dist(float e, int literal) {
   const float m = fabsf(e);
@@ -970,24 +889,6 @@ size_t decode_smem(bool mixed, bool one, int slots, int T, int NWmax) {
   const size_t FT = (size_t)kWarps * T;
   return (mixed ? FT * 24 + 512 : 0) + (one ? FT * 8 * (slots / 2) : 0) +
          4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
-}
-
-// Constants of axes_fast for sqrt(M) = 2^m. t + 512 = round(a q) + 256 sqrt(M);
-// the nearest inner threshold (ties down) is k = floor((t + 255) / 512) =
-// round((t - 3/4) / 512) within [0, sqrt(M) - 2]; with one inner threshold
-// (QPSK) it is 0.
-AxisConst axis_const(int m, const QamConst& qc) {
-  const double side = (double)(1 << m), range = side - 2.0;
-  auto twice = [](double v) { return make_float2((float)v, (float)v); };
-  AxisConst c;
-  c.q = make_float2(qc.q[m], qc.q[m]);
-  c.t0 = twice(-(12582912.0 - 256.0 * side + 512.0));
-  c.g = twice(range);
-  c.s = m > 1 ? (float)(1.0 / (512.0 * range)) : 0.0f;
-  c.c = m > 1 ? (float)(-0.75 / (512.0 * range)) : 0.0f;
-  c.lim = (float)(256.0 * side + 1500.0);  // distances up to 2012: keys below 2^23
-  c.side = (float)side;
-  return c;
 }
 
 template <int kFrom, bool kOne>

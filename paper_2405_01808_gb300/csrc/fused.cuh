@@ -1,21 +1,11 @@
 // Launch interface of the fused decode kernel (fused.cu).
 #pragma once
 
+#include "axis.cuh"
 #include "host_util.cuh"
 #include "internal.cuh"
 
 namespace grand {
-
-// Demodulation constants of one constellation for the packed floating-point
-// arithmetic on both axes (axes_fast in fused.cu): each value twice.
-struct AxisConst {
-  float2 q;      // 256 / d
-  float2 t0;     // -(1.5 * 2^23 - 256 sqrt(M) + 512)
-  float2 g;      // sqrt(M) - 2: the range of the thresholds' indices
-  float s, c;    // t s + c: that range scaled to [0, 1]
-  float lim;     // |a q| up to which the ordering key is exact in 23 bits
-  float side;    // sqrt(M)
-};
 
 struct DecodeArgs {
   const float2* symbols;         // received symbols, or NULL: the demodulated arrays
