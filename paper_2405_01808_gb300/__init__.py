@@ -8,6 +8,7 @@ there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -96,6 +97,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
 def lib() -> ctypes.CDLL:
     """Load libgrand.so (building it first if the sources are newer)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not _build.up_to_date():
@@ -221,21 +224,41 @@ def stream_status(code: Code, stream=None) -> int:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
+    """The stream's handle; the current stream's for None. (The raw handle is
+    asked for directly: building a torch stream object takes 3 us, as long as
+    the library call itself.)"""
     import torch
 
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
+
+
+def _interleaved(symbols):
+    """Address of the received symbols as float32 pairs (complex tensors hold
+    them so). A lazily conjugated tensor is refused, as torch.view_as_real
+    does: its memory holds the values before conjugation."""
+    if symbols.is_complex() and symbols.is_conj():
+        import torch
+
+        torch.view_as_real(symbols)
+    return symbols.data_ptr()
 
 
 def _require_cuda(*ts):
     for t in ts:
-        if t is not None and not t.is_cuda:
+        if t is None:
+            continue
+        if not t.is_cuda:
             raise GrandArgumentError("tensors must live on the CUDA device")
-        if t is not None and not t.is_contiguous():
+        if not t.is_contiguous():
             raise GrandArgumentError("tensors must be contiguous")
 
 
@@ -251,6 +274,7 @@ def _symbols_per_frame(N: int, M: int) -> int:
     return -(-N // (2 * m))
 
 
+@functools.lru_cache(maxsize=None)
 def _dtypes(*names):
     import torch
 
@@ -280,6 +304,8 @@ def _check_symbols(symbols, M: int, L: int):
 
 
 def _check_outputs(F, N, cw, queries, abandon):
+    if cw is None and queries is None and abandon is None:
+        return
     _need(cw, "cw", _dtypes("int32", "uint32"), F * (N // 32))
     _need(queries, "queries", _dtypes("int32", "uint32"), F)
     _need(abandon, "abandon", _dtypes("uint8"), F)
@@ -296,7 +322,7 @@ def demod(symbols, M: int, N: int, N0: float = 1.0, lik_variant: int = LIK_THRES
     L = _symbols_per_frame(N, M)
     F = _check_symbols(symbols, M, L)
     _require_cuda(symbols)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     dev = symbols.device
     if outputs is None:
         outputs = {"y": torch.empty((F, N // 32), dtype=torch.int32, device=dev)}
@@ -317,7 +343,7 @@ def demod(symbols, M: int, N: int, N0: float = 1.0, lik_variant: int = LIK_THRES
     _need(o.get("hard_idx"), "hard_idx", _dtypes("int16", "uint16"), F * L)
     _need(o.get("key"), "key", _dtypes("int32", "uint32"), F * L)
     _need(o.get("rel"), "rel", _dtypes("float32"), F * L)
-    rc = lib().grand_demod(_ptr(sym), F, L, M, float(N0), int(lik_variant), _ptr(o.get("hard_idx")), _ptr(o.get("key")),
+    rc = lib().grand_demod(sym, F, L, M, float(N0), int(lik_variant), _ptr(o.get("hard_idx")), _ptr(o.get("key")),
                            _ptr(o.get("nmask")), _ptr(o.get("rel")), _ptr(o.get("y")), N, _stream(stream))
     _check(rc, "grand_demod")
     return o
@@ -376,15 +402,13 @@ def decode_batch(code: Code, params: Params, y, hard_idx=None, key=None, nmask=N
 def decode_symbols(code: Code, params: Params, symbols, N0: float = 1.0, cw=None, queries=None, abandon=None,
                    stats: bool = False, stream=None):
     """grand_decode_symbols: demodulate and decode in one pass."""
-    import torch
-
     F = _check_symbols(symbols, _params_M(params), _symbols_per_frame(code.N, _params_M(params)))
     _check_outputs(F, code.N, cw, queries, abandon)
     _require_cuda(symbols, cw, queries, abandon)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     cw, queries, abandon = _outputs(F, code.N, symbols.device, cw, queries, abandon)
     st = Stats()
-    rc = lib().grand_decode_symbols(code.handle, ctypes.byref(params), _ptr(sym), F, float(N0), _ptr(cw),
+    rc = lib().grand_decode_symbols(code.handle, ctypes.byref(params), sym, F, float(N0), _ptr(cw),
                                     _ptr(queries), _ptr(abandon), ctypes.byref(st) if stats else None, _stream(stream))
     _check(rc, "grand_decode_symbols")
     return _result(cw, queries, abandon, st, stats)
@@ -406,9 +430,9 @@ def decode_symbols_resumable(code: Code, params: Params, symbols, weight_step: i
         cursors = torch.empty(max(1, F) * CURSOR_BYTES, dtype=torch.uint8, device=symbols.device)
     _need(cursors, "cursors", _dtypes("uint8"), F * CURSOR_BYTES)
     _require_cuda(symbols, cw, queries, abandon, cursors)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     cw, queries, abandon = _outputs(F, code.N, symbols.device, cw, queries, abandon)
-    rc = lib().grand_decode_symbols_resumable(code.handle, ctypes.byref(params), _ptr(sym), F, float(N0),
+    rc = lib().grand_decode_symbols_resumable(code.handle, ctypes.byref(params), sym, F, float(N0),
                                               int(weight_step), _ptr(cursors), _ptr(cw), _ptr(queries),
                                               _ptr(abandon), _stream(stream))
     _check(rc, "grand_decode_symbols_resumable")
@@ -463,7 +487,7 @@ def decode_mixed(codes, params: Params, desc, symbols, n_cw_words: int, N0: floa
     _need(queries, "queries", _dtypes("int32", "uint32"), F)
     _need(abandon, "abandon", _dtypes("uint8"), F)
     _require_cuda(desc, symbols, cw, queries, abandon)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     dev = symbols.device
     if cw is None:
         cw = torch.empty(n_cw_words, dtype=torch.int32, device=dev)
@@ -473,7 +497,7 @@ def decode_mixed(codes, params: Params, desc, symbols, n_cw_words: int, N0: floa
         abandon = torch.empty(F, dtype=torch.uint8, device=dev)
     arr = (ctypes.c_void_p * len(codes))(*[c.handle.value for c in codes])
     st = Stats()
-    rc = lib().grand_decode_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, _ptr(sym), n_sym, float(N0),
+    rc = lib().grand_decode_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, sym, n_sym, float(N0),
                                   _ptr(cw), n_cw_words, _ptr(queries), _ptr(abandon),
                                   ctypes.byref(st) if stats else None, _stream(stream))
     _check(rc, "grand_decode_mixed")
@@ -503,9 +527,9 @@ def decode_mixed_host(codes, params: Params, desc, symbols, n_cw_words: int, N0:
         queries = torch.empty(F, dtype=torch.int32, pin_memory=pin)
     if abandon is None:
         abandon = torch.empty(F, dtype=torch.uint8, pin_memory=pin)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     arr = (ctypes.c_void_p * len(codes))(*[c.handle.value for c in codes])
-    rc = lib().grand_decode_mixed_host(arr, len(codes), ctypes.byref(params), _ptr(desc), F, _ptr(sym), n_sym,
+    rc = lib().grand_decode_mixed_host(arr, len(codes), ctypes.byref(params), _ptr(desc), F, sym, n_sym,
                                        float(N0), _ptr(cw), n_cw_words, _ptr(queries), _ptr(abandon),
                                        int(chunk_frames), _stream(stream))
     _check(rc, "grand_decode_mixed_host")
@@ -535,8 +559,8 @@ def decode_symbols_host(code: Code, params: Params, symbols, N0: float = 1.0, cw
         queries = torch.empty(F, dtype=torch.int32, pin_memory=pin)
     if abandon is None:
         abandon = torch.empty(F, dtype=torch.uint8, pin_memory=pin)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
-    rc = lib().grand_decode_symbols_host(code.handle, ctypes.byref(params), _ptr(sym), F, float(N0), _ptr(cw),
+    sym = _interleaved(symbols)
+    rc = lib().grand_decode_symbols_host(code.handle, ctypes.byref(params), sym, F, float(N0), _ptr(cw),
                                          _ptr(queries), _ptr(abandon), int(chunk_frames), _stream(stream))
     _check(rc, "grand_decode_symbols_host")
     return {"cw": cw, "queries": queries, "abandon": abandon}
@@ -547,16 +571,14 @@ def decode_symbols_noalloc(code: Code, params: Params, symbols, cw, queries, aba
     that may not allocate device memory while running. The caller passes every
     output buffer; at most NOALLOC_MAX_FRAMES frames per call; calls on one
     device must not overlap in time (they share one fixed scratch array)."""
-    import torch
-
     F = _check_symbols(symbols, _params_M(params), _symbols_per_frame(code.N, _params_M(params)))
     for t, name in ((cw, "cw"), (queries, "queries"), (abandon, "abandon")):
         if t is None:
             raise GrandArgumentError(f"{name} is required")
     _check_outputs(F, code.N, cw, queries, abandon)
     _require_cuda(symbols, cw, queries, abandon)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
-    rc = lib().grand_decode_symbols_noalloc(code.handle, ctypes.byref(params), _ptr(sym), F, float(N0), _ptr(cw),
+    sym = _interleaved(symbols)
+    rc = lib().grand_decode_symbols_noalloc(code.handle, ctypes.byref(params), sym, F, float(N0), _ptr(cw),
                                             _ptr(queries), _ptr(abandon), _stream(stream))
     _check(rc, "grand_decode_symbols_noalloc")
     return {"cw": cw, "queries": queries, "abandon": abandon}
@@ -586,34 +608,30 @@ class Plan:
 
 
 def plan_symbols(code: Code, params: Params, symbols, cw, queries, abandon, N0: float = 1.0) -> Plan:
-    import torch
-
     F = _check_symbols(symbols, _params_M(params), _symbols_per_frame(code.N, _params_M(params)))
     for t, name in ((cw, "cw"), (queries, "queries"), (abandon, "abandon")):
         if t is None:
             raise GrandArgumentError(f"{name} is required")
     _check_outputs(F, code.N, cw, queries, abandon)
     _require_cuda(symbols, cw, queries, abandon)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     h = ctypes.c_void_p()
-    rc = lib().grand_plan_symbols(code.handle, ctypes.byref(params), _ptr(sym), symbols.shape[0], float(N0), _ptr(cw),
+    rc = lib().grand_plan_symbols(code.handle, ctypes.byref(params), sym, symbols.shape[0], float(N0), _ptr(cw),
                                   _ptr(queries), _ptr(abandon), ctypes.byref(h))
     _check(rc, "grand_plan_symbols")
     return Plan(h, (code, params, symbols, cw, queries, abandon))
 
 
 def plan_mixed(codes, params: Params, desc, symbols, cw, queries, abandon, N0: float = 1.0) -> Plan:
-    import torch
-
     F, n_sym = _check_mixed(desc, symbols)
     _need(cw, "cw", _dtypes("int32", "uint32"), 0)
     _need(queries, "queries", _dtypes("int32", "uint32"), F)
     _need(abandon, "abandon", _dtypes("uint8"), F)
     _require_cuda(desc, symbols, cw, queries, abandon)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     arr = (ctypes.c_void_p * len(codes))(*[c.handle.value for c in codes])
     h = ctypes.c_void_p()
-    rc = lib().grand_plan_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, _ptr(sym), n_sym, float(N0),
+    rc = lib().grand_plan_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, sym, n_sym, float(N0),
                                 _ptr(cw), cw.numel(), _ptr(queries), _ptr(abandon), ctypes.byref(h))
     _check(rc, "grand_plan_mixed")
     return Plan(h, (codes, params, desc, symbols, cw, queries, abandon))
@@ -631,13 +649,11 @@ def _tune_dict(p, r):
 
 def autotune(code: Code, params: Params, symbols, N0: float = 1.0, cache_path: str | None = None, stream=None):
     """grand_autotune: picks params.tiles on a sample batch (in place)."""
-    import torch
-
     _check_symbols(symbols, _params_M(params), _symbols_per_frame(code.N, _params_M(params)))
     _require_cuda(symbols)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     r = TuneResult()
-    rc = lib().grand_autotune(code.handle, ctypes.byref(params), _ptr(sym), symbols.shape[0], float(N0),
+    rc = lib().grand_autotune(code.handle, ctypes.byref(params), sym, symbols.shape[0], float(N0),
                               cache_path.encode() if cache_path else None, _stream(stream), ctypes.byref(r))
     _check(rc, "grand_autotune")
     return _tune_dict(params, r)
@@ -645,14 +661,12 @@ def autotune(code: Code, params: Params, symbols, N0: float = 1.0, cache_path: s
 
 def autotune_mixed(codes, params: Params, desc, symbols, n_cw_words: int, N0: float = 1.0,
                    cache_path: str | None = None, stream=None):
-    import torch
-
     F, n_sym = _check_mixed(desc, symbols)
     _require_cuda(desc, symbols)
-    sym = torch.view_as_real(symbols) if symbols.is_complex() else symbols
+    sym = _interleaved(symbols)
     arr = (ctypes.c_void_p * len(codes))(*[c.handle.value for c in codes])
     r = TuneResult()
-    rc = lib().grand_autotune_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, _ptr(sym), n_sym, float(N0),
+    rc = lib().grand_autotune_mixed(arr, len(codes), ctypes.byref(params), _ptr(desc), F, sym, n_sym, float(N0),
                                     n_cw_words, cache_path.encode() if cache_path else None, _stream(stream),
                                     ctypes.byref(r))
     _check(rc, "grand_autotune_mixed")

@@ -55,6 +55,7 @@ struct PrepArgs {
   int64_t n_symbols;             // mixed: length of the flat symbol array
   int64_t n_cw_words;            // mixed: length of the flat output array
   const CodeDev* codes;          // device table
+  const CodeDev* host_codes;     // the same table in host memory (one-kernel decode), or NULL
   int n_codes;
   int64_t n_frames;
   int M, L;                      // uniform batch
@@ -2624,6 +2625,10 @@ static DecodeArgs decode_args(const PrepArgs& a, const grand_params* p, int n_co
   d.n_symbols = a.n_symbols;
   d.n_cw_words = a.n_cw_words;
   d.codes = a.codes;
+  if (a.host_codes && n_codes <= kInlineCodes) {
+    d.codes = nullptr;
+    for (int i = 0; i < n_codes; ++i) d.code[i] = a.host_codes[i];
+  }
   d.n_codes = n_codes;
   d.n_frames = n_frames;
   d.M = a.M;
@@ -2887,6 +2892,7 @@ extern "C" int grand_decode_batch(const grand_code* c, const grand_params* p, co
   a.nmask = nmask;
   a.y_in = y;
   a.codes = c->d_dev;
+  a.host_codes = &c->dev;
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
@@ -2924,6 +2930,7 @@ extern "C" int grand_decode_symbols(const grand_code* c, const grand_params* p, 
   PrepArgs a{};
   a.symbols = (const float2*)symbols;
   a.codes = c->d_dev;
+  a.host_codes = &c->dev;
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
@@ -2971,6 +2978,7 @@ extern "C" int grand_decode_symbols_resumable(const grand_code* c, const grand_p
   PrepArgs a{};
   a.symbols = (const float2*)symbols;
   a.codes = c->d_dev;
+  a.host_codes = &c->dev;
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;
@@ -3040,8 +3048,9 @@ static int check_mixed_args(const grand_code* const* codes, int n_codes, const g
 static int mixed_impl(const CodeDev* d_table, int n_codes, int Lmax, int Wmax, const grand_params* p,
                       const grand_frame_desc* desc, int64_t n_frames, const void* symbols, int64_t n_symbols,
                       uint32_t* cw, int64_t n_cw_words, uint32_t* queries, uint8_t* abandon, grand_stats* stats,
-                      cudaStream_t st, const ResumeOpt& ro = ResumeOpt()) {
+                      cudaStream_t st, const ResumeOpt& ro = ResumeOpt(), const CodeDev* host_table = nullptr) {
   PrepArgs a{};
+  a.host_codes = host_table;
   a.symbols = (const float2*)symbols;
   a.desc = desc;
   a.n_symbols = n_symbols;
@@ -3114,6 +3123,11 @@ extern "C" int grand_decode_mixed(const grand_code* const* codes, int n_codes, c
   std::vector<CodeDev> table;
   rc = code_table(codes, n_codes, table, Lmax, Wmax);
   if (rc) return rc;
+  // a small table travels with the one-kernel decode's launch (the allocation,
+  // the staged copy and the free were 10 us of host time a call)
+  if (takes_fused(p, ResumeOpt()) && n_codes <= kInlineCodes)
+    return mixed_impl(nullptr, n_codes, Lmax, Wmax, p, desc, n_frames, symbols, n_symbols, cw, n_cw_words, queries,
+                      abandon, stats, st, ResumeOpt(), table.data());
   CodeDev* d_table = nullptr;
   if (scratch_alloc((void**)&d_table, sizeof(CodeDev) * n_codes, st) != cudaSuccess) return GRAND_E_NOMEM;
   // pageable source: the copy is staged before the call returns
@@ -3306,6 +3320,7 @@ extern "C" int grand_decode_symbols_noalloc(const grand_code* c, const grand_par
   PrepArgs a{};
   a.symbols = (const float2*)symbols;
   a.codes = c->d_dev;
+  a.host_codes = &c->dev;
   a.n_codes = 1;
   a.n_frames = n_frames;
   a.M = p->M;

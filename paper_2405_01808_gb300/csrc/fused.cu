@@ -452,6 +452,8 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   uint32_t* s_flag = s_f0 + FT;                                      // [FT] 0, or the abandon flag of an undecodable frame
   uint32_t* rec = s_flag + FT;                                       // [kRanks][FT] symbol index, later slot positions
   uint32_t* buf = rec + kRanks * FT;                                 // [NWmax][stride]
+  __shared__ CodeDev s_table[kFrom == kFromMixed ? kInlineCodes : 1];
+  const CodeDev* const codes = kFrom == kFromMixed ? (a.codes ? a.codes : s_table) : a.code;
   const int64_t tile = (int64_t)blockIdx.x * FT;
   const int n_here = (int)min((int64_t)FT, a.n_frames - tile);
 
@@ -459,6 +461,10 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   for (int t = threadIdx.x; t < a.NWmax * stride; t += 32 * kWarps) buf[t] = 0u;
   for (int t = threadIdx.x; t < FT; t += 32 * kWarps) s_flag[t] = 0u;
   if constexpr (kFrom == kFromMixed) {
+    if (!a.codes) {
+      if ((int)threadIdx.x < a.n_codes) s_table[threadIdx.x] = a.code[threadIdx.x];
+      __syncthreads();
+    }
     s_plan[threadIdx.x] = pack_plan(warp + 1, lane);
     for (int t = threadIdx.x; t < n_here; t += 32 * kWarps) {
       const grand_frame_desc d = a.desc[tile + t];
@@ -467,7 +473,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
                 d.cw_offset >= 0;
       uint32_t par = 1u << 10;  // L = 0: not decoded
       if (ok) {
-        const CodeDev* code = a.codes + d.code;
+        const CodeDev* code = codes + d.code;
         const int N = code->N, L = (N + 2 * m - 1) / (2 * m);
         ok = d.sym_offset + L <= a.n_symbols && d.cw_offset + (N >> 5) <= a.n_cw_words;
         if (ok) par = (uint32_t)L | ((uint32_t)m << 10) | ((uint32_t)(N >> 5) << 13) | (code->polar ? 1u << 19 : 0u);
@@ -482,7 +488,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
 
   // --- front: one warp per frame ---------------------------------------------
   const int um = kFrom == kFromMixed ? 0 : a.m, uL = kFrom == kFromMixed ? 0 : a.L;
-  const bool u_polar = kFrom == kFromMixed ? false : a.codes->polar != 0;
+  const bool u_polar = kFrom == kFromMixed ? false : a.code[0].polar != 0;
   const int fr_begin = warp * a.T, fr_end = min(n_here, fr_begin + a.T);
   auto frame_base = [&](int fr) { return kFrom == kFromMixed ? s_off[fr] : (tile + fr) * (int64_t)uL; };
   auto frame_len = [&](int fr) { return kFrom == kFromMixed ? (int)(s_par[fr] & 1023u) : uL; };
@@ -500,7 +506,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   auto general_syndrome = [&](int fr, int NW) {
     __syncwarp();
     uint32_t* y = buf + fr;
-    const CodeDev* code = a.codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
+    const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
     const int W = code->W;
     const uint32_t yw = lane < NW ? __brev(y[lane * stride]) : 0u;
     const int64_t co = kFrom == kFromMixed ? s_cw[fr] : (tile + fr) * (int64_t)NW;
@@ -694,7 +700,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
     } else {
       const int L = frame_len(fr);
       const int m = kFrom == kFromMixed ? (int)((s_par[fr] >> 10) & 7u) : um;
-      const CodeDev* code = kFrom == kFromMixed ? a.codes + s_code[fr] : a.codes;
+      const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
       const int N = code->N, NW = N >> 5;
       const int64_t cw_off = kFrom == kFromMixed ? s_cw[fr] : f * (int64_t)NW;
       const int Sp = a.S < L ? a.S : L;

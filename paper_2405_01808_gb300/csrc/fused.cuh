@@ -7,6 +7,10 @@
 
 namespace grand {
 
+// Codes passed by value with the launch: the code of a uniform batch, or a
+// small table of an uneven one, which then needs no table in device memory.
+constexpr int kInlineCodes = 8;
+
 struct DecodeArgs {
   const float2* symbols;         // received symbols, or NULL: the demodulated arrays
   const uint16_t* hard_idx;
@@ -16,7 +20,7 @@ struct DecodeArgs {
   const grand_frame_desc* desc;  // NULL: uniform batch
   int64_t n_symbols;             // mixed: length of the flat symbol array
   int64_t n_cw_words;            // mixed: length of the flat output array
-  const CodeDev* codes;          // device table
+  const CodeDev* codes;          // uneven batch: device table, or NULL: code[]
   int n_codes;
   int64_t n_frames;
   int M, L;                      // uniform batch
@@ -34,6 +38,7 @@ struct DecodeArgs {
   uint32_t* queries;
   uint8_t* abandon;
   Scratch* scr;                  // statistics, or NULL
+  CodeDev code[kInlineCodes];    // uniform batch: [0]
 };
 
 // One launch on `st`; Lmax: the largest frame of the batch in symbols.
