@@ -39,7 +39,8 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kKeySat = 0x7FFFFEu; // packed selection keys hold 23 bits of the reliability
 constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low bits) without a symbol
 constexpr uint32_t kPicked = 0xFFFFFFE0u;  // above those: a key taken as rank (low bits)
-constexpr int kLanePick = 3;            // smallest keys kept per lane of a long frame
+constexpr int kLanePick = 4;            // smallest keys kept per lane of a long frame
+constexpr int kOwnDim = 3;              // kernels of up to this dimension are walked by the frame's thread
 
 // e_v(n1, n3): valid TEPs altering exactly v of n1 ranks with one alternative
 // and n3 ranks with three = the coefficient of x^v in (1 + x)^n1 (1 + 3x)^n3;
@@ -271,75 +272,17 @@ struct Proj {
   __device__ __forceinline__ uint32_t operator()(uint32_t p) const { return p == kNoPos ? 0u : __ldg(tab + p); }
 };
 
-// First TEP of weight <= wmax in canonical order whose projection equals f0
-// and which passes the full test, or kNone.
-__device__ __noinline__ uint32_t light_hit(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
-                                           bool exact, int wmax) {
-  uint32_t dl[3 * kSMax];  // thread-local: the loads of a warp are consecutive
-  for (int r = 0; r < Sp; ++r) {
-    dl[3 * r] = proj(slot_pos(f, 2 * r));
-    dl[3 * r + 1] = proj(slot_pos(f, 2 * r + 1));
-    dl[3 * r + 2] = dl[3 * r] ^ dl[3 * r + 1];
-  }
-  auto delta = [&](int r, int c) { return dl[3 * r + c - 1]; };
-  auto valid = [&](int r, int c) { return ((ex >> (2 * r)) & (uint32_t)c) == (uint32_t)c; };
-  auto full = [&](uint32_t x) { return exact || sum_zero(f, x, true); };
-  if (f0 == 0 && full(0u)) return 0u;
-  for (int p = 0; wmax >= 1 && p < Sp; ++p)
-    for (int c = 1; c <= 3; ++c)
-      if (valid(p, c) && delta(p, c) == f0 && full((uint32_t)c << (2 * p))) return (uint32_t)c << (2 * p);
-  for (int p = 1; wmax >= 2 && p < Sp; ++p)
-    for (int o = 0; o < p; ++o)
-      for (int c = 1; c <= 3; ++c) {
-        if (!valid(p, c)) continue;
-        const uint32_t z = f0 ^ delta(p, c);
-        for (int d = 1; d <= 3; ++d) {
-          const uint32_t x = ((uint32_t)c << (2 * p)) | ((uint32_t)d << (2 * o));
-          if (valid(o, d) && delta(o, d) == z && full(x)) return x;
-        }
-      }
-  for (int p = 2; wmax >= 3 && p < Sp; ++p)
-    for (int o = 1; o < p; ++o)
-      for (int n = 0; n < o; ++n)
-        for (int c = 1; c <= 3; ++c) {
-          if (!valid(p, c)) continue;
-          const uint32_t z = f0 ^ delta(p, c);
-          for (int d = 1; d <= 3; ++d) {
-            if (!valid(o, d)) continue;
-            const uint32_t zz = z ^ delta(o, d);
-            for (int e = 1; e <= 3; ++e) {
-              const uint32_t x = ((uint32_t)c << (2 * p)) | ((uint32_t)d << (2 * o)) | ((uint32_t)e << (2 * n));
-              if (valid(n, e) && delta(n, e) == zz && full(x)) return x;
-            }
-          }
-        }
-  return kNone;
-}
-
-// First solution in canonical order among x0 + span(kv[0..d)), d >= 1 (a
-// Gray-code walk; every solution is a valid TEP). exact: the projection
-// decides. Else: when every kernel vector passes the full test the projected
-// kernel is the true one, and x0 decides for all; otherwise (the projection
-// lost rank on the columns) every candidate is tested.
-// The walk costs 2^d steps; codes with few parity bits have large kernels,
-// and then their first hit is light: weights <= 2 (630 TEPs at most), and
-// above 2^11 solutions weight 3 (5,940), are tested first.
-__device__ __noinline__ uint32_t first_solution(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
-                                                bool exact, uint32_t x0, const uint32_t* kv, int d,
-                                                unsigned long long* ranked) {
+// First solution in canonical order among x0 + span(kv[0..d)), d >= 1, by one
+// thread (a Gray-code walk; every solution is a valid TEP). exact: the
+// projection decides. Else: when every kernel vector passes the full test the
+// projected kernel is the true one, and x0 decides for all; otherwise (the
+// projection lost rank on the columns) every candidate is tested.
+__device__ __noinline__ uint32_t first_solution(const Frame f, bool exact, uint32_t x0, const uint32_t* kv, int d) {
   bool each = false;
   if (!exact) {
     for (int t = 0; t < d && !each; ++t) each = !sum_zero(f, kv[t], false);
     if (!each && !sum_zero(f, x0, true)) return kNone;
   }
-  if (d > 8) {
-    const uint32_t x = light_hit(f, proj, ex, Sp, f0, exact || !each, d > 11 ? 3 : 2);
-    if (x != kNone) {
-      *ranked += 1;
-      return x;
-    }
-  }
-  *ranked += 1ull << d;
   uint32_t x = x0, bk = kNone, bx = kNone;
   for (uint32_t i = 0;;) {
     const uint32_t k = order_key(x);
@@ -351,6 +294,95 @@ __device__ __noinline__ uint32_t first_solution(const Frame f, const Proj proj, 
     x ^= kv[__ffs(i) - 1];
   }
   return bx;
+}
+
+// First TEP of weight <= wmax (at most 3) in canonical order whose projection
+// equals f0 and which passes the full test, or kNone: by one warp, 32 TEPs of
+// the order at a time (all arguments the same in every lane). A weight's TEPs
+// are numbered by their rank set in colex order, then by their alternatives.
+__device__ __noinline__ uint32_t light_hit_warp(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
+                                                bool exact, int wmax) {
+  const int lane = threadIdx.x & 31;
+  uint32_t dl[3 * kSMax];
+  for (int r = 0; r < Sp; ++r) {
+    dl[3 * r] = proj(slot_pos(f, 2 * r));
+    dl[3 * r + 1] = proj(slot_pos(f, 2 * r + 1));
+    dl[3 * r + 2] = dl[3 * r] ^ dl[3 * r + 1];
+  }
+  if (f0 == 0 && (exact || sum_zero(f, 0u, true))) return 0u;
+  for (int w = 1; w <= min(wmax, Sp); ++w) {
+    const int alts = w == 1 ? 3 : (w == 2 ? 9 : 27);
+    const int n = alts * (w == 1 ? Sp : (w == 2 ? Sp * (Sp - 1) / 2 : Sp * (Sp - 1) * (Sp - 2) / 6));
+    for (int b = 0; b < n; b += 32) {
+      const int i = b + lane;
+      bool hit = false;
+      uint32_t x = 0;
+      if (i < n) {
+        int set = i / alts, alt = i % alts;  // the largest rank's alternative is the leading digit
+        uint32_t z = f0;
+        bool valid = true;
+        int lead = alts;
+        for (int j = w; j >= 1; --j) {  // colex: the largest rank first
+          int p = j - 1;
+          if (j == 1) p = set;
+          else if (j == 2) while ((p + 1) * p / 2 <= set) ++p;
+          else while ((p + 1) * p * (p - 1) / 6 <= set) ++p;
+          set -= j == 1 ? set : (j == 2 ? p * (p - 1) / 2 : p * (p - 1) * (p - 2) / 6);
+          lead /= 3;
+          const int c = alt / lead;
+          alt -= c * lead;
+          const uint32_t code = (uint32_t)c + 1u;
+          valid = valid && ((ex >> (2 * p)) & code) == code;
+          x |= code << (2 * p);
+          z ^= dl[3 * p + c];
+        }
+        hit = valid && z == 0u && (exact || sum_zero(f, x, true));
+      }
+      const unsigned m = __ballot_sync(kAll, hit);
+      if (m) return __shfl_sync(kAll, x, __ffs(m) - 1);
+    }
+  }
+  return kNone;
+}
+
+// first_solution by one warp (all arguments but kv the same in every lane; kv
+// is read in lane src). The walk over 2^d solutions takes 2^(d-5) steps; codes
+// with few parity bits have large kernels, and then their first hit is light:
+// above 2^10 solutions weights <= 2 (631 TEPs at most) are tested first, above
+// 2^13 weight 3 (5,940) as well.
+__device__ __noinline__ uint32_t first_solution_warp(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
+                                                     bool exact, uint32_t x0, const uint32_t* kv, int d, int src) {
+  const int lane = threadIdx.x & 31;
+  uint32_t k[2 * kSMax];
+  uint32_t mine = 0;
+  for (int t = 0; t < d; ++t) {
+    k[t] = __shfl_sync(kAll, kv[t], src);
+    if (lane == t) mine = k[t];
+  }
+  bool each = false;
+  if (!exact) {
+    each = __any_sync(kAll, lane < d && !sum_zero(f, mine, false));
+    if (!each && !sum_zero(f, x0, true)) return kNone;
+  }
+  if (d > 10) {
+    const uint32_t x = light_hit_warp(f, proj, ex, Sp, f0, exact || !each, d > 13 ? 3 : 2);
+    if (x != kNone) return x;
+  }
+  uint32_t x = x0, bk = kNone, bx = kNone;
+  for (int t = 0; t < 5 && t < d; ++t)
+    if ((lane >> t) & 1) x ^= k[t];
+  const bool on = d >= 5 || lane < 1 << d;
+  for (uint32_t i = 0; on;) {
+    const uint32_t key = order_key(x);
+    if (comes_before(key, x, bk, bx) && (!each || sum_zero(f, x, true))) {
+      bk = key;
+      bx = x;
+    }
+    if (d <= 5 || ++i >> (d - 5)) break;
+    x ^= k[5 + __ffs(i) - 1];
+  }
+  const uint32_t kmin = __reduce_min_sync(kAll, bk);
+  return __reduce_min_sync(kAll, bk == kmin ? bx : kNone);
 }
 
 // ---------------------------------------------------------------------------
@@ -571,14 +603,16 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       const int Sp = a.S < L ? a.S : L;
       uint32_t* y = buf + fr;
       // this lane's smallest keys, ascending
-      uint32_t b0 = kNone, b1 = kNone, b2 = kNone;
-      static_assert(kLanePick == 3, "kept keys");
+      uint32_t b0 = kNone, b1 = kNone, b2 = kNone, b3 = kNone;
+      static_assert(kLanePick == 4, "kept keys");
       auto keep = [&](uint32_t kp) {
         const uint32_t t0 = max(b0, kp);
         b0 = min(b0, kp);
         const uint32_t t1 = max(b1, t0);
         b1 = min(b1, t0);
+        const uint32_t t2 = max(b2, t1);
         b2 = min(b2, t1);
+        b3 = min(b3, t2);
       };
       bool nf = false;  // uniform
       if constexpr (kFrom == kFromArrays) {
@@ -646,7 +680,8 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
           if (lane == r) pick = kmin;
           b0 = w ? b1 : b0;
           b1 = w ? b2 : b1;
-          b2 = w ? kNone : b2;
+          b2 = w ? b3 : b2;
+          b3 = w ? kNone : b3;
         }
         const bool mine = lane < Sp;
         if (mine) recf[lane * FT] = pick & 511u;
@@ -690,39 +725,47 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   // --- solve: one thread per frame ---------------------------------------------
   unsigned long long evaluated = 0, useful = 0;
   unsigned hard = 0;
+  // what a thread needs to look at frame fr of the tile
+  auto frame_of = [&](int fr, Proj& proj) {
+    const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
+    Frame F;
+    F.buf = buf + fr;
+    F.pos = rec + fr;
+    F.stride = stride;
+    F.pstride = FT;
+    F.fmask = code->fmask;
+    F.hcol = code->hcol;
+    F.W = code->W;
+    F.pat = pat;
+    F.polar = code->polar;
+    F.nw = F.polar ? code->N >> 5 : code->W;
+    // one syndrome word: the columns themselves, and the elimination is the full test
+    proj.tab = code->W == 1 && !(F.polar && F.nw == 1) ? code->hcol : (F.polar ? code->hx : code->hf);
+    return F;
+  };
   const int fr = threadIdx.x;
-  if (fr < n_here) {
-    const int64_t f = tile + fr;
-    const uint32_t flag = s_flag[fr];
-    if (flag) {
-      a.queries[f] = 0;
-      a.abandon[f] = (uint8_t)flag;
-    } else {
+  const uint32_t flag = fr < n_here ? s_flag[fr] : 0u;
+  const bool active = fr < n_here && flag == 0u;
+  int Sp = 0, d = 0;
+  uint32_t ex = 0, f0 = 0, x0 = 0, x = kNone;
+  uint32_t kv[kSlots];
+  bool solvable = false;  // the projected system has solutions (2^d of them)
+  bool shared = false;  // its solutions are walked by the whole warp
+  {
+    if (active) {
       const int L = frame_len(fr);
       const int m = kFrom == kFromMixed ? (int)((s_par[fr] >> 10) & 7u) : um;
       const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
       const int N = code->N, NW = N >> 5;
-      const int64_t cw_off = kFrom == kFromMixed ? s_cw[fr] : f * (int64_t)NW;
-      const int Sp = a.S < L ? a.S : L;
-      Frame F;
-      F.buf = buf + fr;
-      F.pos = rec + fr;
-      F.stride = stride;
-      F.pstride = FT;
-      F.fmask = code->fmask;
-      F.hcol = code->hcol;
-      F.W = code->W;
-      F.pat = pat;
-      F.polar = code->polar;
-      F.nw = F.polar ? NW : code->W;
-      // one syndrome word: the columns themselves, and the elimination is the full test
+      Sp = a.S < L ? a.S : L;
+      Proj proj;
+      const Frame F = frame_of(fr, proj);
       const bool exact = code->W == 1;
-      const Proj proj{exact && !(F.polar && NW == 1) ? code->hcol : (F.polar ? code->hx : code->hf)};
 
       // the alternatives of each rank: flip positions, existing slots, and
       // the slots' columns
       uint32_t c[kSlots];
-      uint32_t ex = 0, real = 0;  // existing slots; those whose flip lies inside the word
+      uint32_t real = 0;  // ex: existing slots; real: those whose flip lies inside the word
       {
         const AxisRegs ax = axis_regs(a.ax[m]);
         const int64_t base = frame_base(fr);
@@ -762,7 +805,6 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       }
 
       // base syndrome (polar form: the transform of y on the frozen bits) and its projection
-      uint32_t f0;
       if (F.polar) {
         uint32_t* b = F.buf;
         auto word = [&](int w) { return transform_word(__brev(b[w * stride])); };
@@ -811,8 +853,7 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       // and a bit elsewhere says there is none. A column without a free row
       // is the sum of the pivot columns named by its bits: a kernel vector.
       uint32_t s = f0, used = 0, free_slots = 0;
-      uint32_t piv[kSlots], kv[kSlots];
-      int d = 0;
+      uint32_t piv[kSlots];
 #pragma unroll
       for (int j = 0; j < kSlots; ++j) {
         const uint32_t u = c[j] & ~used, p = u & (0u - u);
@@ -830,8 +871,6 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
           kv[d++] = c[j];
         }
       }
-      uint32_t x = kNone;
-      unsigned long long ranked = 0;
       if (!(s & ~used)) {
         auto pivots_of = [&](uint32_t v) {
           uint32_t r = 0;
@@ -839,18 +878,48 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
           for (int j = 0; j < kSlots; ++j) r |= (v & piv[j]) ? 1u << j : 0u;
           return r;
         };
-        const uint32_t x0 = pivots_of(s);
-        if (free_slots == 0) {
-          const bool ok = exact || (F.polar ? consume_zero_polar(F, x0) : sum_zero(F, x0, true));
-          if (ok) x = x0;
-          ranked = ok ? 1 : 0;
+        x0 = pivots_of(s);
+        solvable = true;
+        if (d == 0) {
+          if (exact || (F.polar ? consume_zero_polar(F, x0) : sum_zero(F, x0, true))) x = x0;
         } else {
           for (int t = 0; t < d; ++t, free_slots &= free_slots - 1u)
             kv[t] = pivots_of(kv[t]) | (free_slots & (0u - free_slots));
-          x = first_solution(F, proj, ex, Sp, f0, exact, x0, kv, d, &ranked);
+          shared = d > kOwnDim;
+          if (shared && exact && d > 10) {  // few parity bits: most first hits weigh at most 1
+            if (f0 == 0u) x = 0u;
+            for (int r = 0; r < Sp && x == kNone; ++r) {
+              const uint32_t e = (ex >> (2 * r)) & 3u;
+              const uint32_t d0 = proj(slot_pos(F, 2 * r)), d1 = proj(slot_pos(F, 2 * r + 1));
+              if ((e & 1u) && d0 == f0) x = 1u << (2 * r);
+              else if ((e & 2u) && d1 == f0) x = 2u << (2 * r);
+              else if (e == 3u && (d0 ^ d1) == f0) x = 3u << (2 * r);
+            }
+            shared = x == kNone;
+          }
+          if (!shared && x == kNone) x = first_solution(F, exact, x0, kv, d);
         }
       }
+    }
+  }
+  // frames with many solutions, one after the other
+  for (unsigned todo = __ballot_sync(kAll, shared); todo; todo &= todo - 1u) {
+    const int src = __ffs(todo) - 1, of = (int)(threadIdx.x & ~31u) + src;
+    Proj proj;
+    const Frame F = frame_of(of, proj);
+    const int sp = __shfl_sync(kAll, Sp, src), dim = __shfl_sync(kAll, d, src);
+    const uint32_t e = __shfl_sync(kAll, ex, src), p0 = __shfl_sync(kAll, f0, src), s0 = __shfl_sync(kAll, x0, src);
+    const uint32_t got = first_solution_warp(F, proj, e, sp, p0, F.W == 1, s0, kv, dim, src);
+    if (lane == src) x = got;
+  }
 
+  if (fr < n_here) {
+    const int64_t f = tile + fr;
+    if (flag) {
+      a.queries[f] = 0;
+      a.abandon[f] = (uint8_t)flag;
+    } else {
+      const int64_t cw_off = kFrom == kFromMixed ? s_cw[fr] : f * (int64_t)a.NWmax;
       // outputs
       const uint32_t exh = ex & 0x55555555u, exv = (ex >> 1) & 0x55555555u;
       const uint32_t one = exh ^ exv, both = exh & exv;
@@ -862,14 +931,15 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       a.abandon[f] = hit ? 0 : 1;
       if (hit) {
         for (uint32_t t = x; t; t &= t - 1u) {
-          const uint32_t p = slot_pos(F, __ffs(t) - 1);
+          const int b = __ffs(t) - 1;
+          const uint32_t p = (rec[(b >> 1) * FT + fr] >> (16 * (b & 1))) & 0xFFFFu;
           if (p != kNoPos) atomicXor(a.cw + cw_off + (p >> 5), 1u << (p & 31u));
         }
       }
       if (a.scr) {
         // searched: no codeword among the TEPs of the first w0 weights
         const uint32_t done = g_esp.cum[__popc(one)][__popc(both)][min(a.w0, Sp) + 1];
-        evaluated = a.solve ? ranked : (unsigned long long)total;
+        evaluated = !a.solve ? (unsigned long long)total : (solvable ? 1ull << d : 0ull);
         if (!a.solve && qn > done) {
           hard = 1;
           useful = qn - done;
