@@ -17,6 +17,7 @@ struct AxisConst {
   float s, c;    // t s + c: that range scaled to [0, 1]
   float lim;     // |a q| up to which the ordering key is exact in 23 bits
   float side;    // sqrt(M)
+  uint64_t below_top;  // labels of four symbols, m bits an axis: every bit but the top one of each axis
 };
 
 // Constants of axes_fast for sqrt(M) = 2^m. t + 512 = round(a q) + 256 sqrt(M);
@@ -34,6 +35,7 @@ inline AxisConst axis_const(int m, const QamConst& qc) {
   c.c = m > 1 ? (float)(-0.75 / (512.0 * range)) : 0.0f;
   c.lim = (float)(256.0 * side + 1500.0);  // distances up to 2012: keys below 2^23
   c.side = (float)side;
+  c.below_top = ((1ull << 8 * m) - 1ull) / ((1ull << m) - 1ull) * ((1ull << (m - 1)) - 1ull);
   return c;
 }
 

@@ -11,12 +11,23 @@
 // first hit is the solution of smallest canonical position (none: abandoned
 // after min(valid TEPs, cap) queries).
 //
-// k_decode works on tiles of 4 T frames per CTA in two mappings:
-//   front  one warp per frame, T frames one after the other: symbols are read
-//          coalesced (the next 32 are in flight while 32 are worked on), the
-//          hard word is packed by byte stores, the S' least reliable symbols
-//          are picked by warp minima. What is left of a frame is its hard
-//          word and S' symbol records in shared memory.
+// k_decode works on tiles of 4 T frames per CTA:
+//   front  (small, uneven and demodulated batches) one warp per frame, T frames
+//          one after the other: symbols are read coalesced (the next 32 are in
+//          flight while 32 are worked on), the hard word is packed by byte
+//          stores, the S' least reliable symbols are picked by warp minima.
+//          (large uniform batches) one thread per frame: 8 symbols of each of a
+//          warp's 32 frames at a time go through shared memory (asynchronous
+//          copies, 64 contiguous bytes a frame, the next 8 under way
+//          meanwhile); a thread packs its labels by multiplications and keeps
+//          its S' smallest keys sorted by comparator networks. Nothing crosses
+//          lanes, where the warp per frame spends 10 warp minima at a quarter
+//          of the issue rate and a label reduction a step: 416 warp
+//          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
+//          frames 137 -> 64 us, N=128 300,000 frames 91 -> 73 us, N=512 S=12
+//          80,000 frames 76 -> 44 us.
+//          What is left of a frame is its hard word and S' symbol records in
+//          shared memory.
 //   solve  one thread per frame: the base syndrome by the polar transform of
 //          the hard word, the slot columns' 32-bit projections, Gaussian
 //          elimination with the columns in registers, the check of the
@@ -458,16 +469,91 @@ __device__ __forceinline__ uint32_t pick_ranks(uint32_t kp) {
 }
 
 // ---------------------------------------------------------------------------
+// Front helpers (one thread per frame, kChunk symbols at a time)
+// ---------------------------------------------------------------------------
+constexpr int kChunk = 8;                      // symbols of a frame per step
+constexpr int kRowPad = kChunk + 1;            // odd: the rows' 8-byte reads of half a warp fall into different banks
+constexpr int kStageSyms = 32 * kRowPad;       // one chunk of a warp's 32 frames in shared memory
+constexpr int kStages = 2;
+// Resident CTAs of the thread-per-frame kernels (96 registers a thread): against
+// 6 (80 registers) 64 for 67 us on 250,000 frames of 43 symbols, 44 for 46 us
+// on 80,000 of 86, 73 for 72 us on 300,000 of 32; 8 spill and take 71, 50, 76.
+constexpr int kThreadCtas = 5;
+
+// 8 bytes global -> shared without passing the registers; off: zeros.
+__device__ __forceinline__ void fetch8(uint32_t dst, const void* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(on ? 8 : 0) : "memory");
+}
+
+// max(|a|, |b|, |c|), NaN when one is.
+__device__ __forceinline__ float max_abs(float a, float b, float c) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+__device__ __forceinline__ void order2(uint32_t& a, uint32_t& b) {
+  const uint32_t lo = min(a, b);
+  b = max(a, b);
+  a = lo;
+}
+
+// Ascending sort of eight keys (odd-even merge sort, 19 comparators).
+__device__ __forceinline__ void sort8(uint32_t (&k)[kChunk]) {
+  order2(k[0], k[1]); order2(k[2], k[3]); order2(k[4], k[5]); order2(k[6], k[7]);
+  order2(k[0], k[2]); order2(k[1], k[3]); order2(k[4], k[6]); order2(k[5], k[7]);
+  order2(k[1], k[2]); order2(k[5], k[6]);
+  order2(k[0], k[4]); order2(k[1], k[5]); order2(k[2], k[6]); order2(k[3], k[7]);
+  order2(k[2], k[4]); order2(k[3], k[5]);
+  order2(k[1], k[2]); order2(k[3], k[4]); order2(k[5], k[6]);
+}
+
+// The R smallest of best (ascending) and k (ascending), ascending: the minima
+// of best against k reversed rise and then fall, and a bitonic merge sorts
+// them (for R = 10 and 12 that of 16 numbers of which the first 6 or 4 are
+// below all others and stay where they are).
+template <int R>
+__device__ __forceinline__ void merge_smallest(uint32_t (&best)[R], const uint32_t (&k)[kChunk]) {
+  static_assert(R == 8 || R == 10 || R == 12, "ranks");
+#pragma unroll
+  for (int i = R - kChunk; i < R; ++i) best[i] = min(best[i], k[R - 1 - i]);
+#pragma unroll
+  for (int i = 0; i < R - 8; ++i) order2(best[i], best[i + 8]);
+  if constexpr (R == 12) {
+    order2(best[0], best[2]); order2(best[1], best[3]);
+    order2(best[2], best[3]);
+  }
+  if constexpr (R > 8) order2(best[0], best[1]);
+  constexpr int o = R - 8;
+#pragma unroll
+  for (int dist = 4; dist >= 1; dist >>= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (!(i & dist)) order2(best[o + i], best[o + i + dist]);
+}
+
+// Natural labels of four symbols (m bits an axis, I then Q, the first symbol
+// highest) to Gray labels.
+template <typename T>
+__device__ __forceinline__ T gray4(T v, T below_top) { return v ^ ((v >> 1) & below_top); }
+
+// ---------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------
-// kOne: every frame has at most 32 symbols (one per lane). kSlots: 2 x the
-// largest S' (16, 20 or 24: the elimination is unrolled over it).
+// kMap: how the front maps frames to threads. kSlots: 2 x the largest S' (16,
+// 20 or 24: the elimination is unrolled over it).
+enum {
+  kWarpShort = 0,  // a warp per frame of at most 32 symbols (one per lane)
+  kWarpLong = 1,   // a warp per frame, 32 symbols at a time
+  kThread = 2,     // a thread per frame, kChunk symbols at a time
+};
 //
 // Words of a hard word are kept bit-reversed in shared memory (the label bits
 // of a symbol arrive most significant first) until they are written out or
 // transformed.
-template <int kFrom, bool kOne, int kSlots>
-__global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant__ DecodeArgs a) {
+template <int kFrom, int kMap, int kSlots>
+__global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
+  constexpr bool kOne = kMap == kWarpShort;
   extern __shared__ __align__(16) char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int FT = kWarps * a.T;
@@ -476,7 +562,8 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   int64_t* s_off = reinterpret_cast<int64_t*>(smem_raw);             // [FT] mixed: first symbol
   int64_t* s_cw = s_off + (kFrom == kFromMixed ? FT : 0);            // [FT] mixed: first output word
   float2* s_sym = reinterpret_cast<float2*>(s_cw + (kFrom == kFromMixed ? FT : 0));  // [kRanks][FT] kOne: the symbol of each rank
-  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_sym + (kOne ? kRanks * FT : 0));   // [FT] mixed: L | m | words | polar
+  float2* s_stage = s_sym + (kOne ? kRanks * FT : 0);                // [kWarps][kStages][32][kRowPad] kThread: chunks in flight
+  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_stage + (kMap == kThread ? kWarps * kStages * kStageSyms : 0));  // [FT] mixed: L | m | words | polar
   uint32_t* s_code = s_par + (kFrom == kFromMixed ? FT : 0);         // [FT] mixed: index of the code
   uint32_t* s_plan = s_code + (kFrom == kFromMixed ? FT : 0);        // [4][32] mixed: pack_plan
   uint32_t* pat = s_plan + (kFrom == kFromMixed ? 128 : 0);          // [32]
@@ -558,7 +645,144 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
     if (lane == 0) s_f0[fr] = f0;
   };
 
-  if constexpr (kOne) {
+  if constexpr (kMap == kThread) {
+    const AxisRegs ax = axis_regs(a.ax[um]);
+    const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
+    const int rows = n_here - 32 * warp, mine = 32 * warp + lane;
+    const int n_chunks = rows > 0 ? (uL + kChunk - 1) / kChunk : 0;
+    const uint32_t side2 = 1u << (2 * um);
+    // what the fixed exponent bits of four packed labels add up to
+    const uint32_t fixed = __float_as_uint(kMagic) * (1u + side2 + side2 * side2 + side2 * side2 * side2);
+    const uint64_t below_top = a.ax[um].below_top;
+    float2* stage = s_stage + warp * (kStages * kStageSyms);
+    // a fetch takes 8 symbols of 4 frames: 64 contiguous bytes of each
+    const int frow = lane >> 3, fcol = lane & 7;
+    const float2* src = a.symbols + (tile + 32 * warp + frow) * (int64_t)uL + fcol;
+    const uint32_t fdst = (uint32_t)__cvta_generic_to_shared(stage + frow * kRowPad + fcol);
+    auto fetch = [&](int c) {
+      if (c < n_chunks) {
+        const bool in = c * kChunk + fcol < uL;
+        const uint32_t dst = fdst + (uint32_t)(c % kStages) * (kStageSyms * 8);
+        const float2* s = src + c * kChunk;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const bool on = in && frow + 4 * k < rows;
+          fetch8(dst + k * (4 * kRowPad * 8), on ? s + (int64_t)(4 * k) * uL : a.symbols, on);
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint32_t best[kRanks];
+#pragma unroll
+    for (int r = 0; r < kRanks; ++r) best[r] = kNone;
+    bool nf = false;
+    fetch(0);
+    for (int c = 0; c < n_chunks; ++c) {
+      fetch(c + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+      float2* row = stage + (c % kStages) * kStageSyms + lane * kRowPad;
+      F2 x[kChunk];
+      float top = 0.0f;
+#pragma unroll
+      for (int j = 0; j < kChunk; ++j) {
+        x[j] = mul2(pack2(row[j]), ax.q);
+        const float2 xs = unpack2(x[j]);
+        top = max_abs(top, xs.x, xs.y);
+      }
+      const bool wide = __any_sync(kAll, !(top <= ax.lim));
+      if (wide) {  // coordinates that are not finite are read as 0
+#pragma unroll
+        for (int j = 0; j < kChunk; ++j)
+          if (!finite2(row[j])) {
+            nf = true;
+            x[j] = pack2(0.0f, 0.0f);
+            row[j] = make_float2(0.0f, 0.0f);
+          }
+      }
+      uint32_t kp[kChunk], four[2] = {0u, 0u};
+      uint32_t pair[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int j = 0; j < kChunk; ++j) {
+        const Axes t = axes_fast(x[j], ax);
+        float2 d = t.e;
+        if (a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
+        const uint32_t key = __float_as_uint(__fadd_rn(__fmaf_rn(d.x, d.x, __fmul_rn(d.y, d.y)), 8388608.0f));
+        kp[j] = key * 512u + (uint32_t)(c * kChunk + j);
+        const float lI = __fadd_rn(t.k.x, __saturatef(__fadd_rn(t.e.x, 1.0f)));
+        const float lQ = __fadd_rn(t.kb.y, __saturatef(__fadd_rn(t.e.y, 1.0f)));
+        const uint32_t lv = __float_as_uint(__fmaf_rn(lI, ax.side, lQ));
+        if (um <= 4) four[j >> 2] = four[j >> 2] * side2 + lv;
+        else pair[j >> 1] = (pair[j >> 1] << (2 * um)) | (lv & (side2 - 1u));
+      }
+      if (wide) {
+#pragma unroll
+        for (int j = 0; j < kChunk; ++j) {
+          const float2 v = row[j], xs = unpack2(mul2(pack2(v), ax.q));
+          if (!(fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim))
+            kp[j] = (min(symbol_key(v, unpack2(ax.q).x, um, a.lik), kKeySat) << 9) | (uint32_t)(c * kChunk + j);
+        }
+      }
+      if ((c + 1) * kChunk > uL) {
+#pragma unroll
+        for (int j = 0; j < kChunk; ++j)
+          if (c * kChunk + j >= uL) kp[j] = kNone;
+      }
+      sort8(kp);
+      merge_smallest<kRanks>(best, kp);
+      // the labels' 16 m bits, most significant first (N ends with a word:
+      // what lies beyond it is not stored)
+      if (um <= 4) {
+        const uint32_t g0 = gray4(four[0] - fixed, (uint32_t)below_top), g1 = gray4(four[1] - fixed, (uint32_t)below_top);
+        uint32_t* y = buf + mine;
+        auto half = [&](int h, uint32_t v) {
+          if (h < 2 * NW)
+            *(reinterpret_cast<uint16_t*>(y + (h >> 1) * stride) + (~h & 1)) = (uint16_t)v;
+        };
+        if (um == 2) {
+          if (c < NW) y[c * stride] = (g0 << 16) | g1;
+        } else if (um == 4) {
+          if (2 * c < NW) y[2 * c * stride] = g0;
+          if (2 * c + 1 < NW) y[(2 * c + 1) * stride] = g1;
+        } else if (um == 3) {
+          half(3 * c, g0 >> 8);
+          half(3 * c + 1, (g0 << 8) | (g1 >> 16));
+          half(3 * c + 2, g1);
+        } else {
+          half(c, (g0 << 8) | g1);
+        }
+      } else {
+        uint8_t* yb = reinterpret_cast<uint8_t*>(buf + mine);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const uint64_t g = gray4(((uint64_t)pair[2 * i] << (4 * um)) | pair[2 * i + 1], below_top);
+          for (int t = 0; t < um; ++t) {
+            const int b = (2 * c + i) * um + t;
+            if (b < 4 * NW) yb[(b >> 2) * (4 * stride) + (~b & 3)] = (uint8_t)(g >> (8 * (um - 1 - t)));
+          }
+        }
+      }
+      __syncwarp();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const bool here = lane < rows;
+    if (here) {
+      if (nf) s_flag[mine] = 2u;
+#pragma unroll
+      for (int r = 0; r < kRanks; ++r) rec[r * FT + mine] = best[r] & 511u;
+    }
+    // a key that does not fit 23 bits was taken
+    bool redo = false;
+#pragma unroll
+    for (int r = 0; r < kRanks; ++r) redo = redo || (r < Sp && best[r] >= kKeySat << 9);
+    for (unsigned todo = __ballot_sync(kAll, here && !nf && redo); todo; todo &= todo - 1u)
+      reselect(32 * warp + __ffs(todo) - 1, uL, um, Sp, make_float2(0.0f, 0.0f));
+    if (!u_polar) {
+      __syncwarp();
+      for (int fr = 32 * warp; fr < min(n_here, 32 * warp + 32); ++fr)
+        if (!s_flag[fr]) general_syndrome(fr, NW);
+    }
+  } else if constexpr (kOne) {
     const AxisRegs ax = axis_regs(a.ax[um]);
     const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
     const bool on = lane < uL;
@@ -692,12 +916,9 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
       if (!polar) general_syndrome(fr, NW);
     }
   }
-  // A full tile (32 frames a warp) is solved by the warps that prepared it,
-  // each on its own; smaller ones by the first 4 T threads of the CTA. (Long
-  // and uneven frames wait for one another in any case: warps of a CTA in
-  // different parts of the kernel evict each other's instructions, which cost
-  // more than the barrier: 306 against 281 us for 200,000 mixed frames.)
-  const bool own = kOne && a.T == 32;
+  // Where a thread prepared each frame it also solves it; the frames of a warp
+  // per frame are solved by the first 4 T threads of the CTA.
+  constexpr bool own = kMap == kThread;
   auto tile_sync = [&]() {
     if (own) __syncwarp(); else __syncthreads();
   };
@@ -961,24 +1182,25 @@ __global__ void __launch_bounds__(32 * kWarps, 8) k_decode(const __grid_constant
   }
 }
 
-size_t decode_smem(bool mixed, bool one, int slots, int T, int NWmax) {
+size_t decode_smem(bool mixed, int map, int slots, int T, int NWmax) {
   const size_t FT = (size_t)kWarps * T;
-  return (mixed ? FT * 24 + 512 : 0) + (one ? FT * 8 * (slots / 2) : 0) +
+  return (mixed ? FT * 24 + 512 : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
+         (map == kThread ? (size_t)kWarps * kStages * kStageSyms * 8 : 0) +
          4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
 }
 
-template <int kFrom, bool kOne>
+template <int kFrom, int kMap>
 const void* pick_slots(int Smax) {
-  if (Smax <= 8) return (const void*)k_decode<kFrom, kOne, 16>;
-  if (Smax <= 10) return (const void*)k_decode<kFrom, kOne, 20>;
-  return (const void*)k_decode<kFrom, kOne, 24>;
+  if (Smax <= 8) return (const void*)k_decode<kFrom, kMap, 16>;
+  if (Smax <= 10) return (const void*)k_decode<kFrom, kMap, 20>;
+  return (const void*)k_decode<kFrom, kMap, 24>;
 }
 
 }  // namespace
 
 int preload_decode_kernels() {
-  const void* kernels[] = {(const void*)k_decode<kFromMixed, false, 16>, (const void*)k_decode<kFromMixed, false, 20>,
-                           (const void*)k_decode<kFromMixed, false, 24>};
+  const void* kernels[] = {(const void*)k_decode<kFromMixed, kWarpLong, 16>, (const void*)k_decode<kFromMixed, kWarpLong, 20>,
+                           (const void*)k_decode<kFromMixed, kWarpLong, 24>};
   for (const void* k : kernels) {
     cudaFuncAttributes attr;
     if (cudaFuncGetAttributes(&attr, k) != cudaSuccess) return GRAND_E_CUDA;
@@ -986,25 +1208,36 @@ int preload_decode_kernels() {
   return GRAND_OK;
 }
 
+// Uniform batches from here on are prepared by a thread per frame. Its time
+// hardly depends on the batch up to one wave (each lane works through its
+// frame's symbols one after the other), the warp's grows from 4,000 frames on:
+// both cross near 16,384 frames for every length. Thread against warp per
+// frame at 8,192 / 16,384 / 65,536 frames, us: 8 symbols 10.8 / 11.4 / 14.5
+// against 10.8 / 13.3 / 25.6; 32: 10.0 / 10.3 / 16.1 against 9.0 / 11.1 / 23.3;
+// 86: 22 / 23 / 36 against 18 / 25 / 61; 512: 57 / 57 / 125 against 42 / 60 / 219.
+constexpr int64_t kThreadFrames = 16384;
+
 int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const int Smax = a.S < Lmax ? a.S : Lmax;
   const int slots = Smax <= 8 ? 16 : (Smax <= 10 ? 20 : 24);
   const bool mixed = a.desc != nullptr, arrays = !mixed && a.symbols == nullptr;
-  const bool one = !mixed && !arrays && Lmax <= 32;
   const QamConst qc = make_qam_const();
   for (int m = 1; m <= 6; ++m) a.ax[m] = axis_const(m, qc);
-  // frames per warp: as many as keep every SM full (each CTA holds the tile's
-  // solve in its first warps, so larger tiles waste fewer lanes there)
+  const int map = !mixed && !arrays && a.n_frames >= kThreadFrames ? kThread : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
+  // frames per warp: a thread per frame takes 32; else as many as keep every
+  // SM full (each CTA holds the tile's solve in its first warps, so larger
+  // tiles waste fewer lanes there)
   const int64_t slots_cta = (int64_t)sm_count() * 7;
-  const int64_t T = (a.n_frames + slots_cta * kWarps - 1) / (slots_cta * kWarps);
+  const int64_t T = map == kThread ? 32 : (a.n_frames + slots_cta * kWarps - 1) / (slots_cta * kWarps);
   a.m = m_of(a.M);
   a.T = (int)(T < 1 ? 1 : (T > 32 ? 32 : T));
   const int64_t grid = (a.n_frames + kWarps * a.T - 1) / (kWarps * a.T);
-  const size_t smem = decode_smem(mixed, one, slots, a.T, a.NWmax);
-  const void* kern = mixed ? pick_slots<kFromMixed, false>(Smax)
-                           : (arrays ? pick_slots<kFromArrays, false>(Smax)
-                                     : (one ? pick_slots<kFromUniform, true>(Smax)
-                                            : pick_slots<kFromUniform, false>(Smax)));
+  const size_t smem = decode_smem(mixed, map, slots, a.T, a.NWmax);
+  const void* kern = nullptr;
+  if (mixed) kern = pick_slots<kFromMixed, kWarpLong>(Smax);
+  else if (arrays) kern = pick_slots<kFromArrays, kWarpLong>(Smax);
+  else if (map == kThread) kern = pick_slots<kFromUniform, kThread>(Smax);
+  else kern = map == kWarpShort ? pick_slots<kFromUniform, kWarpShort>(Smax) : pick_slots<kFromUniform, kWarpLong>(Smax);
   if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB
   void* args[] = {&a};
   if (cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(32 * kWarps), args, smem, st) != cudaSuccess)
