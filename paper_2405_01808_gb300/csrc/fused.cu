@@ -24,8 +24,8 @@
 //          lanes, where the warp per frame spends 10 warp minima at a quarter
 //          of the issue rate and a label reduction a step: 416 warp
 //          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
-//          frames 137 -> 64 us, N=128 300,000 frames 91 -> 73 us, N=512 S=12
-//          80,000 frames 76 -> 44 us.
+//          frames 137 -> 54 us, N=128 300,000 frames 91 -> 62 us, N=512 S=12
+//          80,000 frames 76 -> 38 us.
 //          What is left of a frame is its hard word and S' symbol records in
 //          shared memory.
 //   solve  one thread per frame: the base syndrome by the polar transform of
@@ -45,7 +45,7 @@ namespace grand {
 namespace {
 
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr int kWarps = 4;               // warps per CTA
+constexpr int kCtaWarps = 4;            // warps per CTA
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kKeySat = 0x7FFFFEu; // packed selection keys hold 23 bits of the reliability
 constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low bits) without a symbol
@@ -475,12 +475,19 @@ constexpr int kChunk = 8;                      // symbols of a frame per step
 constexpr int kRowPad = kChunk + 1;            // odd: the rows' 8-byte reads of half a warp fall into different banks
 constexpr int kStageSyms = 32 * kRowPad;       // one chunk of a warp's 32 frames in shared memory
 constexpr int kStages = 2;
-// Resident CTAs of the thread-per-frame kernels (96 registers a thread): against
-// 6 (80 registers) 64 for 67 us on 250,000 frames of 43 symbols, 44 for 46 us
-// on 80,000 of 86, 73 for 72 us on 300,000 of 32; 8 spill and take 71, 50, 76.
-constexpr int kThreadCtas = 5;
+// CTAs of the thread-per-frame kernels are single warps: nothing is shared
+// between warps, and the last wave is finer (against 4 warps: 20,000 frames of
+// 128 symbols 34 -> 30 us, 300,000 of 32 70 -> 68 us). 20 of them an SM leave 96
+// registers a thread: against 24 (80 registers) 64 for 67 us on 250,000 frames
+// of 43 symbols, 44 for 46 us on 80,000 of 86, 73 for 72 us on 300,000 of 32;
+// 32 spill and take 71, 50, 76.
+constexpr int kThreadCtas = 20;
+constexpr int kThreadWarps = 1;
 
-// 8 bytes global -> shared without passing the registers; off: zeros.
+// 4 or 8 bytes global -> shared without passing the registers; off: zeros.
+__device__ __forceinline__ void fetch4(uint32_t dst, const void* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0) : "memory");
+}
 __device__ __forceinline__ void fetch8(uint32_t dst, const void* src, bool on) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(on ? 8 : 0) : "memory");
 }
@@ -546,14 +553,18 @@ enum {
   kWarpShort = 0,  // a warp per frame of at most 32 symbols (one per lane)
   kWarpLong = 1,   // a warp per frame, 32 symbols at a time
   kThread = 2,     // a thread per frame, kChunk symbols at a time
+  kThreadQam = 3,  // the same for at most 8 bits a symbol and the threshold likelihood (no other case in its inner loop)
 };
 //
 // Words of a hard word are kept bit-reversed in shared memory (the label bits
 // of a symbol arrive most significant first) until they are written out or
 // transformed.
+constexpr int warps_of(int map) { return map >= kThread ? kThreadWarps : kCtaWarps; }
+
 template <int kFrom, int kMap, int kSlots>
-__global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
-  constexpr bool kOne = kMap == kWarpShort;
+__global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWarps), kMap >= kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
+  constexpr int kWarps = kMap >= kThread ? kThreadWarps : kCtaWarps;
+  constexpr bool kOne = kMap == kWarpShort, kRows = kMap >= kThread;
   extern __shared__ __align__(16) char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int FT = kWarps * a.T;
@@ -563,7 +574,7 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
   int64_t* s_cw = s_off + (kFrom == kFromMixed ? FT : 0);            // [FT] mixed: first output word
   float2* s_sym = reinterpret_cast<float2*>(s_cw + (kFrom == kFromMixed ? FT : 0));  // [kRanks][FT] kOne: the symbol of each rank
   float2* s_stage = s_sym + (kOne ? kRanks * FT : 0);                // [kWarps][kStages][32][kRowPad] kThread: chunks in flight
-  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_stage + (kMap == kThread ? kWarps * kStages * kStageSyms : 0));  // [FT] mixed: L | m | words | polar
+  uint32_t* s_par = reinterpret_cast<uint32_t*>(s_stage + (kRows ? kWarps * kStages * kStageSyms : 0));  // [FT] mixed: L | m | words | polar
   uint32_t* s_code = s_par + (kFrom == kFromMixed ? FT : 0);         // [FT] mixed: index of the code
   uint32_t* s_plan = s_code + (kFrom == kFromMixed ? FT : 0);        // [4][32] mixed: pack_plan
   uint32_t* pat = s_plan + (kFrom == kFromMixed ? 128 : 0);          // [32]
@@ -645,7 +656,8 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
     if (lane == 0) s_f0[fr] = f0;
   };
 
-  if constexpr (kMap == kThread) {
+  if constexpr (kRows) {
+    constexpr bool kQam = kMap == kThreadQam;
     const AxisRegs ax = axis_regs(a.ax[um]);
     const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
     const int rows = n_here - 32 * warp, mine = 32 * warp + lane;
@@ -663,11 +675,16 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
       if (c < n_chunks) {
         const bool in = c * kChunk + fcol < uL;
         const uint32_t dst = fdst + (uint32_t)(c % kStages) * (kStageSyms * 8);
-        const float2* s = src + c * kChunk;
+        const float2* s = in ? src + c * kChunk : a.symbols;  // (a fetch of no bytes reads nothing)
+        if (rows >= 32) {
+          const int64_t step = in ? 4 * uL : 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const bool on = in && frow + 4 * k < rows;
-          fetch8(dst + k * (4 * kRowPad * 8), on ? s + (int64_t)(4 * k) * uL : a.symbols, on);
+          for (int k = 0; k < 8; ++k, s += step) fetch8(dst + k * (4 * kRowPad * 8), s, in);
+        } else {
+          for (int k = 0; k < 8; ++k) {
+            const bool on = in && frow + 4 * k < rows;
+            fetch8(dst + k * (4 * kRowPad * 8), on ? s + (int64_t)(4 * k) * uL : a.symbols, on);
+          }
         }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -706,13 +723,13 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
       for (int j = 0; j < kChunk; ++j) {
         const Axes t = axes_fast(x[j], ax);
         float2 d = t.e;
-        if (a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
+        if (!kQam && a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
         const uint32_t key = __float_as_uint(__fadd_rn(__fmaf_rn(d.x, d.x, __fmul_rn(d.y, d.y)), 8388608.0f));
         kp[j] = key * 512u + (uint32_t)(c * kChunk + j);
         const float lI = __fadd_rn(t.k.x, __saturatef(__fadd_rn(t.e.x, 1.0f)));
         const float lQ = __fadd_rn(t.kb.y, __saturatef(__fadd_rn(t.e.y, 1.0f)));
         const uint32_t lv = __float_as_uint(__fmaf_rn(lI, ax.side, lQ));
-        if (um <= 4) four[j >> 2] = four[j >> 2] * side2 + lv;
+        if (kQam || um <= 4) four[j >> 2] = four[j >> 2] * side2 + lv;
         else pair[j >> 1] = (pair[j >> 1] << (2 * um)) | (lv & (side2 - 1u));
       }
       if (wide) {
@@ -732,7 +749,7 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
       merge_smallest<kRanks>(best, kp);
       // the labels' 16 m bits, most significant first (N ends with a word:
       // what lies beyond it is not stored)
-      if (um <= 4) {
+      if (kQam || um <= 4) {
         const uint32_t g0 = gray4(four[0] - fixed, (uint32_t)below_top), g1 = gray4(four[1] - fixed, (uint32_t)below_top);
         uint32_t* y = buf + mine;
         auto half = [&](int h, uint32_t v) {
@@ -782,6 +799,16 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
       for (int fr = 32 * warp; fr < min(n_here, 32 * warp + 32); ++fr)
         if (!s_flag[fr]) general_syndrome(fr, NW);
     }
+    // the selected symbols, rank by rank, on their way to where the chunks were
+    __syncwarp();
+    if (here && !nf) {
+      const float2* own_sym = a.symbols + (tile + mine) * (int64_t)uL;
+      const uint32_t sel = (uint32_t)__cvta_generic_to_shared(stage + lane);
+#pragma unroll
+      for (int r = 0; r < kRanks; ++r)
+        if (r < Sp) fetch8(sel + r * 256, own_sym + rec[r * FT + mine], true);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   } else if constexpr (kOne) {
     const AxisRegs ax = axis_regs(a.ax[um]);
     const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
@@ -918,7 +945,7 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
   }
   // Where a thread prepared each frame it also solves it; the frames of a warp
   // per frame are solved by the first 4 T threads of the CTA.
-  constexpr bool own = kMap == kThread;
+  constexpr bool own = kRows;
   auto tile_sync = [&]() {
     if (own) __syncwarp(); else __syncthreads();
   };
@@ -989,29 +1016,16 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
       uint32_t real = 0;  // ex: existing slots; real: those whose flip lies inside the word
       {
         const AxisRegs ax = axis_regs(a.ax[m]);
-        const int64_t base = frame_base(fr);
-        float2 v[kRanks];
-        uint32_t idx[kRanks];
-#pragma unroll
-        for (int r = 0; r < kRanks; ++r) {
-          v[r] = make_float2(0.0f, 0.0f);
-          idx[r] = r < Sp ? rec[r * FT + fr] : 0u;
-          if constexpr (kOne) v[r] = s_sym[r * FT + fr];
-          else if constexpr (kFrom != kFromArrays) {
-            if (r < Sp) v[r] = a.symbols[base + idx[r]];
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < kRanks; ++r) {
-          Alt t;
-          if constexpr (kFrom == kFromArrays) t = array_alt(a, base + idx[r]);
-          else t = symbol_alt(v[r], ax, a.lik);
+        // slots of rank r (symbol idx) from its alternatives: their positions,
+        // entered in rec, ex and real
+        auto enter = [&](int r, uint32_t idx, const Alt& t, uint32_t& p0, uint32_t& p1) {
           // the neighbour across threshold k differs from the hard level in
           // the Gray label's bit ctz(k + 1)
-          const int pI = 2 * m * (int)idx[r] + m - __ffs((int)t.kI + 1);
-          const int pQ = 2 * m * (int)idx[r] + 2 * m - __ffs((int)t.kQ + 1);
+          const int pI = 2 * m * (int)idx + m - __ffs((int)t.kI + 1);
+          const int pQ = 2 * m * (int)idx + 2 * m - __ffs((int)t.kQ + 1);
           uint32_t e0 = r < Sp && t.exI, e1 = r < Sp && t.exQ;
-          uint32_t p0 = e0 && pI < N ? (uint32_t)pI : kNoPos, p1 = e1 && pQ < N ? (uint32_t)pQ : kNoPos;
+          p0 = e0 && pI < N ? (uint32_t)pI : kNoPos;
+          p1 = e1 && pQ < N ? (uint32_t)pQ : kNoPos;
           if (a.nearer && t.near) {  // the nearer (vertical) alternative takes the first slot
             const uint32_t tp = p0, te = e0;
             p0 = p1; p1 = tp;
@@ -1020,8 +1034,53 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
           if (r < Sp) rec[r * FT + fr] = p0 | (p1 << 16);
           ex |= (e0 | (e1 << 1)) << (2 * r);
           real |= ((p0 != kNoPos ? 1u : 0u) | (p1 != kNoPos ? 2u : 0u)) << (2 * r);
-          c[2 * r] = proj(p0);
-          c[2 * r + 1] = proj(p1);
+        };
+        if constexpr (kRows) {
+          // a loop of fetches instead of unrolled loads: the columns of a rank
+          // replace its symbol in shared memory, so that all of them are under
+          // way together, and the code stays small (warps in different parts
+          // of the kernel compete for the instruction cache, which is what
+          // the solve waits for most): 300,000 frames of 32 symbols 68 -> 62 us
+          float2* sel = s_stage + warp * (kStages * kStageSyms) + lane;
+          const uint32_t at = (uint32_t)__cvta_generic_to_shared(sel);
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll 1
+          for (int r = 0; r < Sp; ++r) {
+            uint32_t p0, p1;
+            enter(r, rec[r * FT + fr], symbol_alt(sel[32 * r], ax, a.lik), p0, p1);
+            fetch4(at + r * 256, proj.tab + (p0 != kNoPos ? p0 : 0u), p0 != kNoPos);
+            fetch4(at + r * 256 + 4, proj.tab + (p1 != kNoPos ? p1 : 0u), p1 != kNoPos);
+          }
+          asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+          for (int r = 0; r < kRanks; ++r) {
+            const float2 v = r < Sp ? sel[32 * r] : make_float2(0.0f, 0.0f);
+            c[2 * r] = __float_as_uint(v.x);
+            c[2 * r + 1] = __float_as_uint(v.y);
+          }
+        } else {
+          const int64_t base = frame_base(fr);
+          float2 v[kRanks];
+          uint32_t idx[kRanks];
+#pragma unroll
+          for (int r = 0; r < kRanks; ++r) {
+            v[r] = make_float2(0.0f, 0.0f);
+            idx[r] = r < Sp ? rec[r * FT + fr] : 0u;
+            if constexpr (kOne) v[r] = s_sym[r * FT + fr];
+            else if constexpr (kFrom != kFromArrays) {
+              if (r < Sp) v[r] = a.symbols[base + idx[r]];
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < kRanks; ++r) {
+            Alt t;
+            if constexpr (kFrom == kFromArrays) t = array_alt(a, base + idx[r]);
+            else t = symbol_alt(v[r], ax, a.lik);
+            uint32_t p0, p1;
+            enter(r, idx[r], t, p0, p1);
+            c[2 * r] = proj(p0);
+            c[2 * r + 1] = proj(p1);
+          }
         }
       }
 
@@ -1183,9 +1242,10 @@ __global__ void __launch_bounds__(32 * kWarps, kMap == kThread ? kThreadCtas : 8
 }
 
 size_t decode_smem(bool mixed, int map, int slots, int T, int NWmax) {
-  const size_t FT = (size_t)kWarps * T;
+  const int warps = warps_of(map);
+  const size_t FT = (size_t)warps * T;
   return (mixed ? FT * 24 + 512 : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
-         (map == kThread ? (size_t)kWarps * kStages * kStageSyms * 8 : 0) +
+         (map >= kThread ? (size_t)warps * kStages * kStageSyms * 8 : 0) +
          4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
 }
 
@@ -1223,24 +1283,26 @@ int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const bool mixed = a.desc != nullptr, arrays = !mixed && a.symbols == nullptr;
   const QamConst qc = make_qam_const();
   for (int m = 1; m <= 6; ++m) a.ax[m] = axis_const(m, qc);
-  const int map = !mixed && !arrays && a.n_frames >= kThreadFrames ? kThread : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
+  const int map = !mixed && !arrays && a.n_frames >= kThreadFrames ? (m_of(a.M) <= 4 && !a.lik ? kThreadQam : kThread) : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
   // frames per warp: a thread per frame takes 32; else as many as keep every
   // SM full (each CTA holds the tile's solve in its first warps, so larger
   // tiles waste fewer lanes there)
+  const int warps = warps_of(map);
   const int64_t slots_cta = (int64_t)sm_count() * 7;
-  const int64_t T = map == kThread ? 32 : (a.n_frames + slots_cta * kWarps - 1) / (slots_cta * kWarps);
+  const int64_t T = map >= kThread ? 32 : (a.n_frames + slots_cta * warps - 1) / (slots_cta * warps);
   a.m = m_of(a.M);
   a.T = (int)(T < 1 ? 1 : (T > 32 ? 32 : T));
-  const int64_t grid = (a.n_frames + kWarps * a.T - 1) / (kWarps * a.T);
+  const int64_t grid = (a.n_frames + warps * a.T - 1) / (warps * a.T);
   const size_t smem = decode_smem(mixed, map, slots, a.T, a.NWmax);
   const void* kern = nullptr;
   if (mixed) kern = pick_slots<kFromMixed, kWarpLong>(Smax);
   else if (arrays) kern = pick_slots<kFromArrays, kWarpLong>(Smax);
+  else if (map == kThreadQam) kern = pick_slots<kFromUniform, kThreadQam>(Smax);
   else if (map == kThread) kern = pick_slots<kFromUniform, kThread>(Smax);
   else kern = map == kWarpShort ? pick_slots<kFromUniform, kWarpShort>(Smax) : pick_slots<kFromUniform, kWarpLong>(Smax);
   if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB
   void* args[] = {&a};
-  if (cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(32 * kWarps), args, smem, st) != cudaSuccess)
+  if (cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(32 * warps), args, smem, st) != cudaSuccess)
     return GRAND_E_CUDA;
   return GRAND_OK;
 }
