@@ -2646,12 +2646,32 @@ static DecodeArgs decode_args(const PrepArgs& a, const grand_params* p, int n_co
   return d;
 }
 
-// The one-kernel decode: no scratch but the counters of a call with stats.
+// The one-kernel decode: no scratch but the counters of a call with stats and
+// the order of a large uneven batch (where there is no memory for the order,
+// the batch is decoded as it comes).
 static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_params* p, int64_t n_frames,
                      grand_stats* stats, cudaStream_t st) {
   DecodeArgs a = decode_args(proto, p, n_codes, n_frames);
-  if (!stats) return launch_decode(a, Lmax, st);
-  if (scratch_alloc((void**)&a.scr, sizeof(Scratch), st) != cudaSuccess) return GRAND_E_NOMEM;
+  void* order = nullptr;
+  if (const size_t bytes = order_bytes(a)) {
+    if (scratch_alloc(&order, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
+      order = nullptr;
+    }
+  }
+  auto launch = [&]() {
+    const int rc = order ? launch_order(a, order, st) : GRAND_OK;
+    return rc == GRAND_OK ? launch_decode(a, Lmax, st) : rc;
+  };
+  if (!stats) {
+    const int rc = launch();
+    if (order) cudaFreeAsync(order, st);
+    return rc;
+  }
+  if (scratch_alloc((void**)&a.scr, sizeof(Scratch), st) != cudaSuccess) {
+    if (order) cudaFreeAsync(order, st);
+    return GRAND_E_NOMEM;
+  }
   int rc = GRAND_OK;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   do {
@@ -2661,7 +2681,7 @@ static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_p
       break;
     }
     cudaEventRecord(ev[0], st);
-    if ((rc = launch_decode(a, Lmax, st)) != GRAND_OK) break;
+    if ((rc = launch()) != GRAND_OK) break;
     cudaEventRecord(ev[1], st);
     Scratch h{};
     if (cudaMemcpyAsync(&h, a.scr, sizeof(Scratch), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -2678,6 +2698,7 @@ static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_p
   for (int i = 0; i < 2; ++i)
     if (ev[i]) cudaEventDestroy(ev[i]);
   cudaFreeAsync(a.scr, st);
+  if (order) cudaFreeAsync(order, st);
   return rc;
 }
 

@@ -12,11 +12,12 @@
 // after min(valid TEPs, cap) queries).
 //
 // k_decode works on tiles of 4 T frames per CTA:
-//   front  (small, uneven and demodulated batches) one warp per frame, T frames
+//   front  (small and demodulated batches) one warp per frame, T frames
 //          one after the other: symbols are read coalesced (the next 32 are in
 //          flight while 32 are worked on), the hard word is packed by byte
 //          stores, the S' least reliable symbols are picked by warp minima.
-//          (large uniform batches) one thread per frame: 8 symbols of each of a
+//          (large batches; uneven ones are first put in order by length) one
+//          thread per frame: 8 symbols of each of a
 //          warp's 32 frames at a time go through shared memory (asynchronous
 //          copies, 64 contiguous bytes a frame, the next 8 under way
 //          meanwhile); a thread packs its labels by multiplications and keeps
@@ -25,7 +26,7 @@
 //          of the issue rate and a label reduction a step: 416 warp
 //          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
 //          frames 137 -> 54 us, N=128 300,000 frames 91 -> 62 us, N=512 S=12
-//          80,000 frames 76 -> 38 us.
+//          80,000 frames 76 -> 38 us, uneven mix of 10^6 frames 904 -> 656 us.
 //          What is left of a frame is its hard word and S' symbol records in
 //          shared memory.
 //   solve  one thread per frame: the base syndrome by the polar transform of
@@ -553,18 +554,117 @@ enum {
   kWarpShort = 0,  // a warp per frame of at most 32 symbols (one per lane)
   kWarpLong = 1,   // a warp per frame, 32 symbols at a time
   kThread = 2,     // a thread per frame, kChunk symbols at a time
-  kThreadQam = 3,  // the same for at most 8 bits a symbol and the threshold likelihood (no other case in its inner loop)
 };
 //
 // Words of a hard word are kept bit-reversed in shared memory (the label bits
 // of a symbol arrive most significant first) until they are written out or
 // transformed.
-constexpr int warps_of(int map) { return map >= kThread ? kThreadWarps : kCtaWarps; }
+constexpr int warps_of(int map) { return map == kThread ? kThreadWarps : kCtaWarps; }
+
+// An uneven batch's frame: symbols | m << 10 | words << 13 | polar << 19;
+// kNoFrame (no symbols) for a descriptor that names none.
+constexpr uint32_t kNoFrame = 1u << 10;
+__device__ __forceinline__ uint32_t frame_par(const DecodeArgs& a, const CodeDev* codes, const grand_frame_desc& d) {
+  const int m = (31 - __clz(d.M)) >> 1;
+  if (d.code < 0 || d.code >= a.n_codes || m < 1 || m > 6 || d.M != 1 << (2 * m) || d.sym_offset < 0 || d.cw_offset < 0)
+    return kNoFrame;
+  const CodeDev* code = codes + d.code;
+  const int N = code->N, L = (N + 2 * m - 1) / (2 * m);
+  if (d.sym_offset > a.n_symbols - L || d.cw_offset > a.n_cw_words - (N >> 5)) return kNoFrame;
+  return (uint32_t)L | ((uint32_t)m << 10) | ((uint32_t)(N >> 5) << 13) | (code->polar ? 1u << 19 : 0u);
+}
+
+// ---------------------------------------------------------------------------
+// Order of an uneven batch: frames of as many steps of kChunk symbols and of
+// one constellation together, the longest first, for the thread-per-frame
+// front (the lanes of a warp then finish together). A counting sort: counts
+// per block, starts by the last block, indices by a second pass.
+// ---------------------------------------------------------------------------
+constexpr int kBins = 65 * 8;           // (64 - steps) * 8 + m
+constexpr int kSortThreads = 256, kSortEach = 4;
+constexpr size_t kSortHeader = 4 * (kBins + 8);  // bins, ticket
+
+struct SortTile {
+  uint32_t count[kBins];
+  uint32_t start[kBins];
+  CodeDev table[kInlineCodes];
+};
+
+__device__ __forceinline__ void count_bins(const DecodeArgs& a, SortTile& s, int (&bin)[kSortEach]) {
+  for (int b = threadIdx.x; b < kBins; b += kSortThreads) s.count[b] = 0u;
+  if (!a.codes && (int)threadIdx.x < a.n_codes) s.table[threadIdx.x] = a.code[threadIdx.x];
+  __syncthreads();
+  const CodeDev* codes = a.codes ? a.codes : s.table;
+#pragma unroll
+  for (int i = 0; i < kSortEach; ++i) {
+    const int64_t f = ((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x;
+    bin[i] = -1;
+    if (f < a.n_frames) {
+      const uint32_t par = frame_par(a, codes, a.desc[f]);
+      bin[i] = (64 - (int)(((par & 1023u) + kChunk - 1) / kChunk)) * 8 + (int)((par >> 10) & 7u);
+      atomicAdd(&s.count[bin[i]], 1u);
+    }
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_order_count(const __grid_constant__ DecodeArgs a, uint32_t* bins) {
+  __shared__ SortTile s;
+  __shared__ bool last;
+  int bin[kSortEach];
+  count_bins(a, s, bin);
+  for (int b = threadIdx.x; b < kBins; b += kSortThreads)
+    if (s.count[b]) atomicAdd(bins + b, s.count[b]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(bins + kBins, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  // starts: one warp, kEach bins a lane
+  constexpr int kEach = (kBins + 31) / 32;
+  uint32_t v[kEach], sum = 0;
+#pragma unroll
+  for (int i = 0; i < kEach; ++i) {
+    const int b = (int)threadIdx.x * kEach + i;
+    v[i] = b < kBins ? __ldcg(bins + b) : 0u;
+    sum += v[i];
+  }
+  uint32_t before = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(kAll, before, o);
+    if ((int)threadIdx.x >= o) before += t;
+  }
+  before -= sum;
+#pragma unroll
+  for (int i = 0; i < kEach; ++i) {
+    const int b = (int)threadIdx.x * kEach + i;
+    if (b < kBins) bins[b] = before;
+    before += v[i];
+  }
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_order_index(const __grid_constant__ DecodeArgs a, uint32_t* bins,
+                                                              uint32_t* order) {
+  __shared__ SortTile s;
+  int bin[kSortEach];
+  count_bins(a, s, bin);
+  for (int b = threadIdx.x; b < kBins; b += kSortThreads)
+    if (s.count[b]) {
+      s.start[b] = atomicAdd(bins + b, s.count[b]);
+      s.count[b] = 0u;
+    }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kSortEach; ++i)
+    if (bin[i] >= 0)
+      order[s.start[bin[i]] + atomicAdd(&s.count[bin[i]], 1u)] =
+          (uint32_t)(((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x);
+}
 
 template <int kFrom, int kMap, int kSlots>
-__global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWarps), kMap >= kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
-  constexpr int kWarps = kMap >= kThread ? kThreadWarps : kCtaWarps;
-  constexpr bool kOne = kMap == kWarpShort, kRows = kMap >= kThread;
+__global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWarps), kMap == kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
+  constexpr int kWarps = kMap == kThread ? kThreadWarps : kCtaWarps;
+  constexpr bool kOne = kMap == kWarpShort, kRows = kMap == kThread;
   extern __shared__ __align__(16) char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int FT = kWarps * a.T;
@@ -577,7 +677,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
   uint32_t* s_par = reinterpret_cast<uint32_t*>(s_stage + (kRows ? kWarps * kStages * kStageSyms : 0));  // [FT] mixed: L | m | words | polar
   uint32_t* s_code = s_par + (kFrom == kFromMixed ? FT : 0);         // [FT] mixed: index of the code
   uint32_t* s_plan = s_code + (kFrom == kFromMixed ? FT : 0);        // [4][32] mixed: pack_plan
-  uint32_t* pat = s_plan + (kFrom == kFromMixed ? 128 : 0);          // [32]
+  uint32_t* pat = s_plan + (kFrom == kFromMixed && !kRows ? 128 : 0);          // [32]
   uint32_t* s_f0 = pat + 32;                                         // [FT] projection of s(y) (H not of polar form)
   uint32_t* s_flag = s_f0 + FT;                                      // [FT] 0, or the abandon flag of an undecodable frame
   uint32_t* rec = s_flag + FT;                                       // [kRanks][FT] symbol index, later slot positions
@@ -595,23 +695,18 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       if ((int)threadIdx.x < a.n_codes) s_table[threadIdx.x] = a.code[threadIdx.x];
       __syncthreads();
     }
-    s_plan[threadIdx.x] = pack_plan(warp + 1, lane);
-    for (int t = threadIdx.x; t < n_here; t += 32 * kWarps) {
-      const grand_frame_desc d = a.desc[tile + t];
-      const int m = (31 - __clz(d.M)) >> 1;
-      bool ok = d.code >= 0 && d.code < a.n_codes && m >= 1 && m <= 6 && d.M == 1 << (2 * m) && d.sym_offset >= 0 &&
-                d.cw_offset >= 0;
-      uint32_t par = 1u << 10;  // L = 0: not decoded
-      if (ok) {
-        const CodeDev* code = codes + d.code;
-        const int N = code->N, L = (N + 2 * m - 1) / (2 * m);
-        ok = d.sym_offset + L <= a.n_symbols && d.cw_offset + (N >> 5) <= a.n_cw_words;
-        if (ok) par = (uint32_t)L | ((uint32_t)m << 10) | ((uint32_t)(N >> 5) << 13) | (code->polar ? 1u << 19 : 0u);
+    if constexpr (!kRows) s_plan[threadIdx.x] = pack_plan(warp + 1, lane);
+    for (int t = threadIdx.x; t < (kRows ? FT : n_here); t += 32 * kWarps) {
+      uint32_t par = kNoFrame;
+      grand_frame_desc d{};
+      if (t < n_here) {
+        d = a.desc[kRows ? (int64_t)a.order[tile + t] : tile + t];
+        par = frame_par(a, codes, d);
       }
       s_off[t] = d.sym_offset;
       s_cw[t] = d.cw_offset;
       s_par[t] = par;
-      s_code[t] = ok ? (uint32_t)d.code : 0u;
+      s_code[t] = par != kNoFrame ? (uint32_t)d.code : 0u;
     }
   }
   __syncthreads();
@@ -657,15 +752,26 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
   };
 
   if constexpr (kRows) {
-    constexpr bool kQam = kMap == kThreadQam;
-    const AxisRegs ax = axis_regs(a.ax[um]);
-    const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
     const int rows = n_here - 32 * warp, mine = 32 * warp + lane;
-    const int n_chunks = rows > 0 ? (uL + kChunk - 1) / kChunk : 0;
-    const uint32_t side2 = 1u << (2 * um);
+    const bool here = lane < rows;
+    // this thread's frame (uneven batch: its own length and constellation)
+    const uint32_t par = kFrom == kFromMixed ? s_par[mine] : 0u;
+    const int L = kFrom == kFromMixed ? (int)(par & 1023u) : uL;
+    const int m = kFrom == kFromMixed ? (int)((par >> 10) & 7u) : um;
+    const int NW = kFrom == kFromMixed ? (int)((par >> 13) & 63u) : a.NWmax;
+    const int Sp = a.S < L ? a.S : L;
+    const AxisRegs ax = axis_regs(a.ax[m]);
+    int n_chunks = rows > 0 ? (L + kChunk - 1) / kChunk : 0;
+    // the inner loop without the literal likelihood and symbols of more than 8 bits
+    bool usual = !a.lik && m <= 4;
+    if constexpr (kFrom == kFromMixed) {
+      n_chunks = __reduce_max_sync(kAll, n_chunks);
+      usual = __all_sync(kAll, usual);
+    }
+    const uint32_t side2 = 1u << (2 * m);
     // what the fixed exponent bits of four packed labels add up to
     const uint32_t fixed = __float_as_uint(kMagic) * (1u + side2 + side2 * side2 + side2 * side2 * side2);
-    const uint64_t below_top = a.ax[um].below_top;
+    const uint64_t below_top = a.ax[m].below_top;
     float2* stage = s_stage + warp * (kStages * kStageSyms);
     // a fetch takes 8 symbols of 4 frames: 64 contiguous bytes of each
     const int frow = lane >> 3, fcol = lane & 7;
@@ -673,17 +779,28 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     const uint32_t fdst = (uint32_t)__cvta_generic_to_shared(stage + frow * kRowPad + fcol);
     auto fetch = [&](int c) {
       if (c < n_chunks) {
-        const bool in = c * kChunk + fcol < uL;
         const uint32_t dst = fdst + (uint32_t)(c % kStages) * (kStageSyms * 8);
-        const float2* s = in ? src + c * kChunk : a.symbols;  // (a fetch of no bytes reads nothing)
-        if (rows >= 32) {
-          const int64_t step = in ? 4 * uL : 0;
+        if constexpr (kFrom == kFromMixed) {
+          const int i = c * kChunk + fcol;
 #pragma unroll
-          for (int k = 0; k < 8; ++k, s += step) fetch8(dst + k * (4 * kRowPad * 8), s, in);
-        } else {
           for (int k = 0; k < 8; ++k) {
-            const bool on = in && frow + 4 * k < rows;
-            fetch8(dst + k * (4 * kRowPad * 8), on ? s + (int64_t)(4 * k) * uL : a.symbols, on);
+            const int row = 32 * warp + frow + 4 * k;
+            const bool on = i < (int)(s_par[row] & 1023u);
+            const void* p = on ? (const void*)(a.symbols + s_off[row] + i) : (const void*)a.desc;  // (no bytes are read)
+            fetch8(dst + k * (4 * kRowPad * 8), p, on);
+          }
+        } else {
+          const bool in = c * kChunk + fcol < uL;
+          const float2* s = in ? src + c * kChunk : a.symbols;
+          if (rows >= 32) {
+            const int64_t step = in ? 4 * uL : 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k, s += step) fetch8(dst + k * (4 * kRowPad * 8), s, in);
+          } else {
+            for (int k = 0; k < 8; ++k) {
+              const bool on = in && frow + 4 * k < rows;
+              fetch8(dst + k * (4 * kRowPad * 8), on ? s + (int64_t)(4 * k) * uL : a.symbols, on);
+            }
           }
         }
       }
@@ -693,11 +810,9 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
 #pragma unroll
     for (int r = 0; r < kRanks; ++r) best[r] = kNone;
     bool nf = false;
-    fetch(0);
-    for (int c = 0; c < n_chunks; ++c) {
-      fetch(c + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      __syncwarp();
+    // one step; kUsual: no literal likelihood, at most 8 bits a symbol
+    auto step = [&](auto usual_form, int c) {
+      constexpr bool kUsual = decltype(usual_form)::value;
       float2* row = stage + (c % kStages) * kStageSyms + lane * kRowPad;
       F2 x[kChunk];
       float top = 0.0f;
@@ -723,45 +838,45 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       for (int j = 0; j < kChunk; ++j) {
         const Axes t = axes_fast(x[j], ax);
         float2 d = t.e;
-        if (!kQam && a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
+        if (!kUsual && a.lik) d = make_float2(axis_dist(d.x, 1), axis_dist(d.y, 1));
         const uint32_t key = __float_as_uint(__fadd_rn(__fmaf_rn(d.x, d.x, __fmul_rn(d.y, d.y)), 8388608.0f));
         kp[j] = key * 512u + (uint32_t)(c * kChunk + j);
         const float lI = __fadd_rn(t.k.x, __saturatef(__fadd_rn(t.e.x, 1.0f)));
         const float lQ = __fadd_rn(t.kb.y, __saturatef(__fadd_rn(t.e.y, 1.0f)));
         const uint32_t lv = __float_as_uint(__fmaf_rn(lI, ax.side, lQ));
-        if (kQam || um <= 4) four[j >> 2] = four[j >> 2] * side2 + lv;
-        else pair[j >> 1] = (pair[j >> 1] << (2 * um)) | (lv & (side2 - 1u));
+        if constexpr (kUsual) four[j >> 2] = four[j >> 2] * side2 + lv;
+        else pair[j >> 1] = (pair[j >> 1] << (2 * m)) | (lv & (side2 - 1u));
       }
       if (wide) {
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) {
           const float2 v = row[j], xs = unpack2(mul2(pack2(v), ax.q));
           if (!(fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim))
-            kp[j] = (min(symbol_key(v, unpack2(ax.q).x, um, a.lik), kKeySat) << 9) | (uint32_t)(c * kChunk + j);
+            kp[j] = (min(symbol_key(v, unpack2(ax.q).x, m, a.lik), kKeySat) << 9) | (uint32_t)(c * kChunk + j);
         }
       }
-      if ((c + 1) * kChunk > uL) {
+      if ((c + 1) * kChunk > L) {
 #pragma unroll
         for (int j = 0; j < kChunk; ++j)
-          if (c * kChunk + j >= uL) kp[j] = kNone;
+          if (c * kChunk + j >= L) kp[j] = kNone;
       }
       sort8(kp);
       merge_smallest<kRanks>(best, kp);
       // the labels' 16 m bits, most significant first (N ends with a word:
       // what lies beyond it is not stored)
-      if (kQam || um <= 4) {
+      if constexpr (kUsual) {
         const uint32_t g0 = gray4(four[0] - fixed, (uint32_t)below_top), g1 = gray4(four[1] - fixed, (uint32_t)below_top);
         uint32_t* y = buf + mine;
         auto half = [&](int h, uint32_t v) {
           if (h < 2 * NW)
             *(reinterpret_cast<uint16_t*>(y + (h >> 1) * stride) + (~h & 1)) = (uint16_t)v;
         };
-        if (um == 2) {
+        if (m == 2) {
           if (c < NW) y[c * stride] = (g0 << 16) | g1;
-        } else if (um == 4) {
+        } else if (m == 4) {
           if (2 * c < NW) y[2 * c * stride] = g0;
           if (2 * c + 1 < NW) y[(2 * c + 1) * stride] = g1;
-        } else if (um == 3) {
+        } else if (m == 3) {
           half(3 * c, g0 >> 8);
           half(3 * c + 1, (g0 << 8) | (g1 >> 16));
           half(3 * c + 2, g1);
@@ -772,19 +887,27 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
         uint8_t* yb = reinterpret_cast<uint8_t*>(buf + mine);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          const uint64_t g = gray4(((uint64_t)pair[2 * i] << (4 * um)) | pair[2 * i + 1], below_top);
-          for (int t = 0; t < um; ++t) {
-            const int b = (2 * c + i) * um + t;
-            if (b < 4 * NW) yb[(b >> 2) * (4 * stride) + (~b & 3)] = (uint8_t)(g >> (8 * (um - 1 - t)));
+          const uint64_t g = gray4(((uint64_t)pair[2 * i] << (4 * m)) | pair[2 * i + 1], below_top);
+          for (int t = 0; t < m; ++t) {
+            const int b = (2 * c + i) * m + t;
+            if (b < 4 * NW) yb[(b >> 2) * (4 * stride) + (~b & 3)] = (uint8_t)(g >> (8 * (m - 1 - t)));
           }
         }
       }
+    };
+    fetch(0);
+    for (int c = 0; c < n_chunks; ++c) {
+      fetch(c + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+      if (usual) step(std::true_type{}, c);
+      else step(std::false_type{}, c);
       __syncwarp();
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const bool here = lane < rows;
+    const bool searched = here && !nf && !(kFrom == kFromMixed && L == 0);
     if (here) {
-      if (nf) s_flag[mine] = 2u;
+      if (!searched) s_flag[mine] = L == 0 ? 3u : 2u;  // not a decodable descriptor, or not finite
 #pragma unroll
       for (int r = 0; r < kRanks; ++r) rec[r * FT + mine] = best[r] & 511u;
     }
@@ -792,17 +915,20 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     bool redo = false;
 #pragma unroll
     for (int r = 0; r < kRanks; ++r) redo = redo || (r < Sp && best[r] >= kKeySat << 9);
-    for (unsigned todo = __ballot_sync(kAll, here && !nf && redo); todo; todo &= todo - 1u)
-      reselect(32 * warp + __ffs(todo) - 1, uL, um, Sp, make_float2(0.0f, 0.0f));
-    if (!u_polar) {
-      __syncwarp();
-      for (int fr = 32 * warp; fr < min(n_here, 32 * warp + 32); ++fr)
-        if (!s_flag[fr]) general_syndrome(fr, NW);
+    for (unsigned todo = __ballot_sync(kAll, searched && redo); todo; todo &= todo - 1u) {
+      const int of = __ffs(todo) - 1;
+      reselect(32 * warp + of, __shfl_sync(kAll, L, of), __shfl_sync(kAll, m, of), __shfl_sync(kAll, Sp, of),
+               make_float2(0.0f, 0.0f));
+    }
+    const bool plain_h = kFrom == kFromMixed ? (par >> 19) != 0u : u_polar;
+    for (unsigned todo = __ballot_sync(kAll, searched && !plain_h); todo; todo &= todo - 1u) {
+      const int of = __ffs(todo) - 1;
+      general_syndrome(32 * warp + of, __shfl_sync(kAll, NW, of));
     }
     // the selected symbols, rank by rank, on their way to where the chunks were
     __syncwarp();
-    if (here && !nf) {
-      const float2* own_sym = a.symbols + (tile + mine) * (int64_t)uL;
+    if (searched) {
+      const float2* own_sym = a.symbols + frame_base(mine);
       const uint32_t sel = (uint32_t)__cvta_generic_to_shared(stage + lane);
 #pragma unroll
       for (int r = 0; r < kRanks; ++r)
@@ -1194,7 +1320,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
   }
 
   if (fr < n_here) {
-    const int64_t f = tile + fr;
+    const int64_t f = kFrom == kFromMixed && kRows ? (int64_t)a.order[tile + fr] : tile + fr;
     if (flag) {
       a.queries[f] = 0;
       a.abandon[f] = (uint8_t)flag;
@@ -1244,8 +1370,8 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
 size_t decode_smem(bool mixed, int map, int slots, int T, int NWmax) {
   const int warps = warps_of(map);
   const size_t FT = (size_t)warps * T;
-  return (mixed ? FT * 24 + 512 : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
-         (map >= kThread ? (size_t)warps * kStages * kStageSyms * 8 : 0) +
+  return (mixed ? FT * 24 + (map == kThread ? 0 : 512) : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
+         (map == kThread ? (size_t)warps * kStages * kStageSyms * 8 : 0) +
          4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
 }
 
@@ -1260,7 +1386,10 @@ const void* pick_slots(int Smax) {
 
 int preload_decode_kernels() {
   const void* kernels[] = {(const void*)k_decode<kFromMixed, kWarpLong, 16>, (const void*)k_decode<kFromMixed, kWarpLong, 20>,
-                           (const void*)k_decode<kFromMixed, kWarpLong, 24>};
+                           (const void*)k_decode<kFromMixed, kWarpLong, 24>,
+                           (const void*)k_decode<kFromMixed, kThread, 16>, (const void*)k_decode<kFromMixed, kThread, 20>,
+                           (const void*)k_decode<kFromMixed, kThread, 24>, (const void*)k_order_count,
+                           (const void*)k_order_index};
   for (const void* k : kernels) {
     cudaFuncAttributes attr;
     if (cudaFuncGetAttributes(&attr, k) != cudaSuccess) return GRAND_E_CUDA;
@@ -1277,27 +1406,49 @@ int preload_decode_kernels() {
 // 86: 22 / 23 / 36 against 18 / 25 / 61; 512: 57 / 57 / 125 against 42 / 60 / 219.
 constexpr int64_t kThreadFrames = 16384;
 
+// Uneven batches from here on are put in order first and prepared by a thread
+// per frame. A thread takes 50 us for a frame of 512 symbols whatever the
+// batch, so the warp per frame (45 us for 16,384 frames of every length, 62
+// for 32,768, 85 for 65,536, 160 for 131,072) is left only beyond 90,000
+// frames (88, 92, 100 and 132 us in order, the sort included).
+constexpr int64_t kOrderFrames = 98304;
+
+size_t order_bytes(const DecodeArgs& a) {
+  return a.desc && a.n_frames >= kOrderFrames && a.n_frames < (int64_t)1 << 31 ? kSortHeader + 4 * (size_t)a.n_frames : 0;
+}
+
+int launch_order(DecodeArgs& a, void* scratch, cudaStream_t st) {
+  uint32_t* bins = static_cast<uint32_t*>(scratch);
+  uint32_t* order = bins + kSortHeader / 4;
+  if (cudaMemsetAsync(bins, 0, kSortHeader, st) != cudaSuccess) return GRAND_E_CUDA;
+  const unsigned grid = (unsigned)((a.n_frames + kSortThreads * kSortEach - 1) / (kSortThreads * kSortEach));
+  k_order_count<<<grid, kSortThreads, 0, st>>>(a, bins);
+  k_order_index<<<grid, kSortThreads, 0, st>>>(a, bins, order);
+  if (cudaGetLastError() != cudaSuccess) return GRAND_E_CUDA;
+  a.order = order;
+  return GRAND_OK;
+}
+
 int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const int Smax = a.S < Lmax ? a.S : Lmax;
   const int slots = Smax <= 8 ? 16 : (Smax <= 10 ? 20 : 24);
   const bool mixed = a.desc != nullptr, arrays = !mixed && a.symbols == nullptr;
   const QamConst qc = make_qam_const();
   for (int m = 1; m <= 6; ++m) a.ax[m] = axis_const(m, qc);
-  const int map = !mixed && !arrays && a.n_frames >= kThreadFrames ? (m_of(a.M) <= 4 && !a.lik ? kThreadQam : kThread) : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
+  const int map = a.order ? kThread : !mixed && !arrays && a.n_frames >= kThreadFrames ? kThread : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
   // frames per warp: a thread per frame takes 32; else as many as keep every
   // SM full (each CTA holds the tile's solve in its first warps, so larger
   // tiles waste fewer lanes there)
   const int warps = warps_of(map);
   const int64_t slots_cta = (int64_t)sm_count() * 7;
-  const int64_t T = map >= kThread ? 32 : (a.n_frames + slots_cta * warps - 1) / (slots_cta * warps);
+  const int64_t T = map == kThread ? 32 : (a.n_frames + slots_cta * warps - 1) / (slots_cta * warps);
   a.m = m_of(a.M);
   a.T = (int)(T < 1 ? 1 : (T > 32 ? 32 : T));
   const int64_t grid = (a.n_frames + warps * a.T - 1) / (warps * a.T);
   const size_t smem = decode_smem(mixed, map, slots, a.T, a.NWmax);
   const void* kern = nullptr;
-  if (mixed) kern = pick_slots<kFromMixed, kWarpLong>(Smax);
+  if (mixed) kern = a.order ? pick_slots<kFromMixed, kThread>(Smax) : pick_slots<kFromMixed, kWarpLong>(Smax);
   else if (arrays) kern = pick_slots<kFromArrays, kWarpLong>(Smax);
-  else if (map == kThreadQam) kern = pick_slots<kFromUniform, kThreadQam>(Smax);
   else if (map == kThread) kern = pick_slots<kFromUniform, kThread>(Smax);
   else kern = map == kWarpShort ? pick_slots<kFromUniform, kWarpShort>(Smax) : pick_slots<kFromUniform, kWarpLong>(Smax);
   if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB

@@ -18,6 +18,7 @@ struct DecodeArgs {
   const uint8_t* nmask;
   const uint32_t* y_in;
   const grand_frame_desc* desc;  // NULL: uniform batch
+  const uint32_t* order;         // uneven batch: its frames by length (launch_order), or NULL
   int64_t n_symbols;             // mixed: length of the flat symbol array
   int64_t n_cw_words;            // mixed: length of the flat output array
   const CodeDev* codes;          // uneven batch: device table, or NULL: code[]
@@ -40,6 +41,11 @@ struct DecodeArgs {
   Scratch* scr;                  // statistics, or NULL
   CodeDev code[kInlineCodes];    // uniform batch: [0]
 };
+
+// Scratch that launch_order needs for the batch; 0: it is decoded in its own order.
+size_t order_bytes(const DecodeArgs& a);
+// Frames of an uneven batch by length and constellation (sets a.order).
+int launch_order(DecodeArgs& a, void* scratch, cudaStream_t st);
 
 // One launch on `st`; Lmax: the largest frame of the batch in symbols.
 int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st);
