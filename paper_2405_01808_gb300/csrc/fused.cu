@@ -484,6 +484,7 @@ constexpr int kStages = 2;
 // 32 spill and take 71, 50, 76.
 constexpr int kThreadCtas = 20;
 constexpr int kThreadWarps = 1;
+constexpr int kOrderCtas = 16;  // uneven batches: shared memory allows 17 with words of 1024 bits
 
 // 4 or 8 bytes global -> shared without passing the registers; off: zeros.
 __device__ __forceinline__ void fetch4(uint32_t dst, const void* src, bool on) {
@@ -578,11 +579,14 @@ __device__ __forceinline__ uint32_t frame_par(const DecodeArgs& a, const CodeDev
 // Order of an uneven batch: frames of as many steps of kChunk symbols and of
 // one constellation together, the longest first, for the thread-per-frame
 // front (the lanes of a warp then finish together). A counting sort: counts
-// per block, starts by the last block, indices by a second pass.
+// per block, starts by the last block, records by a second pass. A record
+// holds what the decode needs of its frame: the way from an index over the
+// descriptor and the code to the first symbol was three dependent loads.
 // ---------------------------------------------------------------------------
 constexpr int kBins = 65 * 8;           // (64 - steps) * 8 + m
 constexpr int kSortThreads = 256, kSortEach = 4;
 constexpr size_t kSortHeader = 4 * (kBins + 8);  // bins, ticket
+static_assert(kSortHeader % 32 == 0 && sizeof(OrderRec) == 32, "records on sectors");
 
 struct SortTile {
   uint32_t count[kBins];
@@ -644,7 +648,7 @@ __global__ void __launch_bounds__(kSortThreads) k_order_count(const __grid_const
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_order_index(const __grid_constant__ DecodeArgs a, uint32_t* bins,
-                                                              uint32_t* order) {
+                                                              OrderRec* order) {
   __shared__ SortTile s;
   int bin[kSortEach];
   count_bins(a, s, bin);
@@ -654,15 +658,20 @@ __global__ void __launch_bounds__(kSortThreads) k_order_index(const __grid_const
       s.count[b] = 0u;
     }
   __syncthreads();
+  const CodeDev* codes = a.codes ? a.codes : s.table;
 #pragma unroll
-  for (int i = 0; i < kSortEach; ++i)
-    if (bin[i] >= 0)
-      order[s.start[bin[i]] + atomicAdd(&s.count[bin[i]], 1u)] =
-          (uint32_t)(((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x);
+  for (int i = 0; i < kSortEach; ++i) {
+    if (bin[i] < 0) continue;
+    const int64_t f = ((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x;
+    const grand_frame_desc d = a.desc[f];
+    const uint32_t par = frame_par(a, codes, d);
+    order[s.start[bin[i]] + atomicAdd(&s.count[bin[i]], 1u)] =
+        OrderRec{d.sym_offset, d.cw_offset, par, par != kNoFrame ? (uint32_t)d.code : 0u, (uint32_t)f, 0u};
+  }
 }
 
 template <int kFrom, int kMap, int kSlots>
-__global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWarps), kMap == kThread ? kThreadCtas : 8) k_decode(const __grid_constant__ DecodeArgs a) {
+__global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWarps), kMap == kThread ? (kFrom == kFromMixed ? kOrderCtas : kThreadCtas) : 8) k_decode(const __grid_constant__ DecodeArgs a) {
   constexpr int kWarps = kMap == kThread ? kThreadWarps : kCtaWarps;
   constexpr bool kOne = kMap == kWarpShort, kRows = kMap == kThread;
   extern __shared__ __align__(16) char smem_raw[];
@@ -697,16 +706,21 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
     }
     if constexpr (!kRows) s_plan[threadIdx.x] = pack_plan(warp + 1, lane);
     for (int t = threadIdx.x; t < (kRows ? FT : n_here); t += 32 * kWarps) {
-      uint32_t par = kNoFrame;
-      grand_frame_desc d{};
-      if (t < n_here) {
-        d = a.desc[kRows ? (int64_t)a.order[tile + t] : tile + t];
-        par = frame_par(a, codes, d);
+      if constexpr (kRows) {
+        OrderRec o{0, 0, kNoFrame, 0, 0, 0};
+        if (t < n_here) o = a.order[tile + t];
+        s_off[t] = o.sym_offset;
+        s_cw[t] = o.cw_offset;
+        s_par[t] = o.par;
+        s_code[t] = o.code;
+      } else {
+        const grand_frame_desc d = a.desc[tile + t];
+        const uint32_t par = frame_par(a, codes, d);
+        s_off[t] = d.sym_offset;
+        s_cw[t] = d.cw_offset;
+        s_par[t] = par;
+        s_code[t] = par != kNoFrame ? (uint32_t)d.code : 0u;
       }
-      s_off[t] = d.sym_offset;
-      s_cw[t] = d.cw_offset;
-      s_par[t] = par;
-      s_code[t] = par != kNoFrame ? (uint32_t)d.code : 0u;
     }
   }
   __syncthreads();
@@ -777,17 +791,29 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
     const int frow = lane >> 3, fcol = lane & 7;
     const float2* src = a.symbols + (tile + 32 * warp + frow) * (int64_t)uL + fcol;
     const uint32_t fdst = (uint32_t)__cvta_generic_to_shared(stage + frow * kRowPad + fcol);
+    // uneven batch: first symbols of the 8 rows this lane fetches for, and the
+    // steps that are complete in every row
+    uint32_t first[8];
+    int n_full = 0;
+    if constexpr (kFrom == kFromMixed) {
+      n_full = __reduce_min_sync(kAll, L / kChunk);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) first[k] = (uint32_t)s_off[32 * warp + frow + 4 * k] + (uint32_t)fcol;
+    }
     auto fetch = [&](int c) {
       if (c < n_chunks) {
         const uint32_t dst = fdst + (uint32_t)(c % kStages) * (kStageSyms * 8);
         if constexpr (kFrom == kFromMixed) {
-          const int i = c * kChunk + fcol;
+          if (c < n_full) {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const int row = 32 * warp + frow + 4 * k;
-            const bool on = i < (int)(s_par[row] & 1023u);
-            const void* p = on ? (const void*)(a.symbols + s_off[row] + i) : (const void*)a.desc;  // (no bytes are read)
-            fetch8(dst + k * (4 * kRowPad * 8), p, on);
+            for (int k = 0; k < 8; ++k) fetch8(dst + k * (4 * kRowPad * 8), a.symbols + (first[k] + (uint32_t)(c * kChunk)), true);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const bool on = c * kChunk + fcol < (int)(s_par[32 * warp + frow + 4 * k] & 1023u);
+              const void* p = on ? (const void*)(a.symbols + (first[k] + (uint32_t)(c * kChunk))) : (const void*)a.desc;
+              fetch8(dst + k * (4 * kRowPad * 8), p, on);  // (off: no bytes are read)
+            }
           }
         } else {
           const bool in = c * kChunk + fcol < uL;
@@ -1081,10 +1107,14 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
   {
     const int first = own ? 32 * warp : 0, last = own ? min(n_here, first + 32) : n_here;
     if constexpr (kFrom == kFromMixed) {
-      for (int fr = own ? first : warp; fr < last; fr += own ? 1 : kWarps) {
+      // own: as many lanes a frame as its words at most (32 one-word frames in
+      // one step)
+      const int per = own ? max(__reduce_max_sync(kAll, (s_par[lane] >> 13) & 63u), 1u) : 32;
+      const int w = own ? lane % per : lane;
+      for (int fr = own ? first + lane / per : warp; fr < last; fr += own ? 32 / per : kWarps) {
         const uint32_t par = s_par[fr];
         const bool out = (par & 1023u) && ((par >> 19) || s_flag[fr]);  // a general matrix's word is out already
-        if (out && lane < (int)((par >> 13) & 63u)) a.cw[s_cw[fr] + lane] = __brev(buf[lane * stride + fr]);
+        if (out && w < (int)((par >> 13) & 63u)) a.cw[s_cw[fr] + w] = __brev(buf[w * stride + fr]);
       }
     } else {
       const int NW = a.NWmax, lg = 31 - __clz(NW);
@@ -1320,7 +1350,7 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
   }
 
   if (fr < n_here) {
-    const int64_t f = kFrom == kFromMixed && kRows ? (int64_t)a.order[tile + fr] : tile + fr;
+    const int64_t f = kFrom == kFromMixed && kRows ? (int64_t)a.order[tile + fr].frame : tile + fr;
     if (flag) {
       a.queries[f] = 0;
       a.abandon[f] = (uint8_t)flag;
@@ -1414,12 +1444,15 @@ constexpr int64_t kThreadFrames = 16384;
 constexpr int64_t kOrderFrames = 98304;
 
 size_t order_bytes(const DecodeArgs& a) {
-  return a.desc && a.n_frames >= kOrderFrames && a.n_frames < (int64_t)1 << 31 ? kSortHeader + 4 * (size_t)a.n_frames : 0;
+  const int64_t wide = (int64_t)1 << 31;  // the records' frame, and symbol offsets, in 32 bits
+  return a.desc && a.n_frames >= kOrderFrames && a.n_frames < wide && a.n_symbols < wide
+             ? kSortHeader + sizeof(OrderRec) * (size_t)a.n_frames
+             : 0;
 }
 
 int launch_order(DecodeArgs& a, void* scratch, cudaStream_t st) {
   uint32_t* bins = static_cast<uint32_t*>(scratch);
-  uint32_t* order = bins + kSortHeader / 4;
+  OrderRec* order = reinterpret_cast<OrderRec*>(bins + kSortHeader / 4);
   if (cudaMemsetAsync(bins, 0, kSortHeader, st) != cudaSuccess) return GRAND_E_CUDA;
   const unsigned grid = (unsigned)((a.n_frames + kSortThreads * kSortEach - 1) / (kSortThreads * kSortEach));
   k_order_count<<<grid, kSortThreads, 0, st>>>(a, bins);

@@ -11,6 +11,12 @@ namespace grand {
 // small table of an uneven one, which then needs no table in device memory.
 constexpr int kInlineCodes = 8;
 
+// A frame of an uneven batch in the order of launch_order.
+struct alignas(32) OrderRec {
+  int64_t sym_offset, cw_offset;
+  uint32_t par, code, frame, unused;  // par: frame_par
+};
+
 struct DecodeArgs {
   const float2* symbols;         // received symbols, or NULL: the demodulated arrays
   const uint16_t* hard_idx;
@@ -18,7 +24,7 @@ struct DecodeArgs {
   const uint8_t* nmask;
   const uint32_t* y_in;
   const grand_frame_desc* desc;  // NULL: uniform batch
-  const uint32_t* order;         // uneven batch: its frames by length (launch_order), or NULL
+  const OrderRec* order;         // uneven batch: its frames by length (launch_order), or NULL
   int64_t n_symbols;             // mixed: length of the flat symbol array
   int64_t n_cw_words;            // mixed: length of the flat output array
   const CodeDev* codes;          // uneven batch: device table, or NULL: code[]
