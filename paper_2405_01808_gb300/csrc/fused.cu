@@ -234,14 +234,27 @@ __device__ __forceinline__ bool consume_zero_polar(const Frame& f, uint32_t x) {
     const uint32_t p = slot_pos(f, __ffs(t) - 1);
     if (p == kNoPos) continue;
     const uint32_t pt = f.pat[p & 31u], sup = p >> 5;
-    uint32_t w = sup;
-    for (;;) {
-      f.buf[w * f.stride] ^= pt & __ldg(f.fmask + w);
-      if (w == 0) break;
-      w = (w - 1u) & sup;
+    // four subsets a round, so that their loads are in flight together
+    for (uint32_t top = sup;;) {
+      uint32_t w[4], y[4];
+      bool on = true, go[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        w[i] = top;
+        go[i] = on;
+        on = on && top != 0u;
+        top = (top - 1u) & sup;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) y[i] = f.buf[w[i] * f.stride] ^ (pt & __ldg(f.fmask + w[i]));
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (go[i]) f.buf[w[i] * f.stride] = y[i];
+      if (!on) break;
     }
   }
   uint32_t orr = 0;
+#pragma unroll 4
   for (int w = 0; w < f.nw; ++w) orr |= f.buf[w * f.stride];
   return orr == 0;
 }
@@ -594,18 +607,24 @@ struct SortTile {
   CodeDev table[kInlineCodes];
 };
 
-__device__ __forceinline__ void count_bins(const DecodeArgs& a, SortTile& s, int (&bin)[kSortEach]) {
+// The block's descriptors (loads first, all in flight together) and their bins' counts.
+__device__ __forceinline__ void count_bins(const DecodeArgs& a, SortTile& s, grand_frame_desc (&d)[kSortEach],
+                                           uint32_t (&par)[kSortEach], int (&bin)[kSortEach]) {
+  const int64_t f0 = (int64_t)blockIdx.x * (kSortEach * kSortThreads) + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < kSortEach; ++i)
+    d[i] = f0 + i * kSortThreads < a.n_frames ? a.desc[f0 + i * kSortThreads] : grand_frame_desc{};
   for (int b = threadIdx.x; b < kBins; b += kSortThreads) s.count[b] = 0u;
   if (!a.codes && (int)threadIdx.x < a.n_codes) s.table[threadIdx.x] = a.code[threadIdx.x];
   __syncthreads();
   const CodeDev* codes = a.codes ? a.codes : s.table;
 #pragma unroll
   for (int i = 0; i < kSortEach; ++i) {
-    const int64_t f = ((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x;
     bin[i] = -1;
-    if (f < a.n_frames) {
-      const uint32_t par = frame_par(a, codes, a.desc[f]);
-      bin[i] = (64 - (int)(((par & 1023u) + kChunk - 1) / kChunk)) * 8 + (int)((par >> 10) & 7u);
+    par[i] = kNoFrame;
+    if (f0 + i * kSortThreads < a.n_frames) {
+      par[i] = frame_par(a, codes, d[i]);
+      bin[i] = (64 - (int)(((par[i] & 1023u) + kChunk - 1) / kChunk)) * 8 + (int)((par[i] >> 10) & 7u);
       atomicAdd(&s.count[bin[i]], 1u);
     }
   }
@@ -615,8 +634,10 @@ __device__ __forceinline__ void count_bins(const DecodeArgs& a, SortTile& s, int
 __global__ void __launch_bounds__(kSortThreads) k_order_count(const __grid_constant__ DecodeArgs a, uint32_t* bins) {
   __shared__ SortTile s;
   __shared__ bool last;
+  grand_frame_desc d[kSortEach];
+  uint32_t par[kSortEach];
   int bin[kSortEach];
-  count_bins(a, s, bin);
+  count_bins(a, s, d, par, bin);
   for (int b = threadIdx.x; b < kBins; b += kSortThreads)
     if (s.count[b]) atomicAdd(bins + b, s.count[b]);
   __threadfence();
@@ -650,23 +671,22 @@ __global__ void __launch_bounds__(kSortThreads) k_order_count(const __grid_const
 __global__ void __launch_bounds__(kSortThreads) k_order_index(const __grid_constant__ DecodeArgs a, uint32_t* bins,
                                                               OrderRec* order) {
   __shared__ SortTile s;
+  grand_frame_desc d[kSortEach];
+  uint32_t par[kSortEach];
   int bin[kSortEach];
-  count_bins(a, s, bin);
+  count_bins(a, s, d, par, bin);
   for (int b = threadIdx.x; b < kBins; b += kSortThreads)
     if (s.count[b]) {
       s.start[b] = atomicAdd(bins + b, s.count[b]);
       s.count[b] = 0u;
     }
   __syncthreads();
-  const CodeDev* codes = a.codes ? a.codes : s.table;
 #pragma unroll
   for (int i = 0; i < kSortEach; ++i) {
     if (bin[i] < 0) continue;
     const int64_t f = ((int64_t)blockIdx.x * kSortEach + i) * kSortThreads + threadIdx.x;
-    const grand_frame_desc d = a.desc[f];
-    const uint32_t par = frame_par(a, codes, d);
     order[s.start[bin[i]] + atomicAdd(&s.count[bin[i]], 1u)] =
-        OrderRec{d.sym_offset, d.cw_offset, par, par != kNoFrame ? (uint32_t)d.code : 0u, (uint32_t)f, 0u};
+        OrderRec{d[i].sym_offset, d[i].cw_offset, par[i], par[i] != kNoFrame ? (uint32_t)d[i].code : 0u, (uint32_t)f, 0u};
   }
 }
 
@@ -1166,6 +1186,69 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
       const Frame F = frame_of(fr, proj);
       const bool exact = code->W == 1;
 
+      // base syndrome (polar form: the transform of y on the frozen bits) and its projection
+      if (F.polar) {
+        uint32_t* b = F.buf;
+        auto word = [&](int w) { return transform_word(__brev(b[w * stride])); };
+        // four words apart by dw at a time: two levels of the transform
+        // with one round of loads in flight together
+        auto two_levels = [&](int w, int dw, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
+          x0 ^= x1; x2 ^= x3;
+          x0 ^= x2; x1 ^= x3;
+          b[w * stride] = x0; b[(w + dw) * stride] = x1; b[(w + 2 * dw) * stride] = x2; b[(w + 3 * dw) * stride] = x3;
+        };
+        if (NW >= 4) {
+          for (int w = 0; w < NW; w += 4) two_levels(w, 1, word(w), word(w + 1), word(w + 2), word(w + 3));
+          int dw = 4;
+          for (; 2 * dw < NW; dw <<= 2)
+            for (int t = 0; t < NW / 4; ++t) {
+              const int w = ((t & ~(dw - 1)) << 2) | (t & (dw - 1));
+              two_levels(w, dw, b[w * stride], b[(w + dw) * stride], b[(w + 2 * dw) * stride], b[(w + 3 * dw) * stride]);
+            }
+          if (dw < NW)  // one level left: its words in groups of four (NW >= 8)
+            for (int t = 0; t < NW / 2; t += 4) {
+              uint32_t lo[4], hi[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int w = (((t + i) & ~(dw - 1)) << 1) | ((t + i) & (dw - 1));
+                lo[i] = b[w * stride];
+                hi[i] = b[(w + dw) * stride];
+              }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) b[((((t + i) & ~(dw - 1)) << 1) | ((t + i) & (dw - 1))) * stride] = lo[i] ^ hi[i];
+            }
+        } else {
+          const uint32_t x0 = word(0);
+          b[0] = x0;
+          if (NW == 2) {
+            const uint32_t x1 = word(1);
+            b[stride] = x1;
+            b[0] = x0 ^ x1;
+          }
+        }
+        f0 = 0;
+        if (exact && NW > 1) {  // at most 32 frozen bits: packed as the columns are
+          for (int r = 0; r < code->R; ++r) {
+            const uint32_t i = __ldg(code->frozen + r);
+            f0 |= ((b[(i >> 5) * stride] >> (i & 31u)) & 1u) << r;
+          }
+        } else {
+          for (int w0 = 0; w0 < NW; w0 += 4) {  // (NW is a power of two)
+            uint32_t s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[i] = w0 + i < NW ? b[(w0 + i) * stride] & __ldg(F.fmask + w0 + i) : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (w0 + i < NW) {
+                b[(w0 + i) * stride] = s[i];
+                f0 = syndrome_fold(f0, s[i]);
+              }
+          }
+        }
+      } else {
+        f0 = s_f0[fr];
+      }
+
       // the alternatives of each rank: flip positions, existing slots, and
       // the slots' columns
       uint32_t c[kSlots];
@@ -1238,48 +1321,6 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
             c[2 * r + 1] = proj(p1);
           }
         }
-      }
-
-      // base syndrome (polar form: the transform of y on the frozen bits) and its projection
-      if (F.polar) {
-        uint32_t* b = F.buf;
-        auto word = [&](int w) { return transform_word(__brev(b[w * stride])); };
-        if (NW >= 4) {
-          for (int w = 0; w < NW; w += 4) {
-            uint32_t x0 = word(w), x1 = word(w + 1), x2 = word(w + 2), x3 = word(w + 3);
-            x0 ^= x1; x2 ^= x3;
-            x0 ^= x2; x1 ^= x3;
-            b[w * stride] = x0; b[(w + 1) * stride] = x1; b[(w + 2) * stride] = x2; b[(w + 3) * stride] = x3;
-          }
-          for (int dw = 4; dw < NW; dw <<= 1)
-            for (int t = 0; t < NW / 2; ++t) {
-              const int w = ((t & ~(dw - 1)) << 1) | (t & (dw - 1));
-              b[w * stride] ^= b[(w + dw) * stride];
-            }
-        } else {
-          const uint32_t x0 = word(0);
-          b[0] = x0;
-          if (NW == 2) {
-            const uint32_t x1 = word(1);
-            b[stride] = x1;
-            b[0] = x0 ^ x1;
-          }
-        }
-        f0 = 0;
-        if (exact && NW > 1) {  // at most 32 frozen bits: packed as the columns are
-          for (int r = 0; r < code->R; ++r) {
-            const uint32_t i = __ldg(code->frozen + r);
-            f0 |= ((b[(i >> 5) * stride] >> (i & 31u)) & 1u) << r;
-          }
-        } else {
-          for (int w = 0; w < NW; ++w) {
-            const uint32_t s = b[w * stride] & __ldg(F.fmask + w);
-            b[w * stride] = s;
-            f0 = syndrome_fold(f0, s);
-          }
-        }
-      } else {
-        f0 = s_f0[fr];
       }
 
       // Gauss-Jordan on the columns: the pivot of column j is its lowest row
