@@ -26,7 +26,7 @@
 //          of the issue rate and a label reduction a step: 416 warp
 //          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
 //          frames 137 -> 54 us, N=128 300,000 frames 91 -> 62 us, N=512 S=12
-//          80,000 frames 76 -> 38 us, uneven mix of 10^6 frames 904 -> 656 us.
+//          80,000 frames 76 -> 38 us, uneven mix of 10^6 frames 904 -> 587 us.
 //          What is left of a frame is its hard word and S' symbol records in
 //          shared memory.
 //   solve  one thread per frame: the base syndrome by the polar transform of
@@ -568,12 +568,13 @@ enum {
   kWarpShort = 0,  // a warp per frame of at most 32 symbols (one per lane)
   kWarpLong = 1,   // a warp per frame, 32 symbols at a time
   kThread = 2,     // a thread per frame, kChunk symbols at a time
+  kThreadUsual = 3,  // the same without the inner loop for symbols of more than 8 bits and the literal likelihood
 };
 //
 // Words of a hard word are kept bit-reversed in shared memory (the label bits
 // of a symbol arrive most significant first) until they are written out or
 // transformed.
-constexpr int warps_of(int map) { return map == kThread ? kThreadWarps : kCtaWarps; }
+constexpr int warps_of(int map) { return map >= kThread ? kThreadWarps : kCtaWarps; }
 
 // An uneven batch's frame: symbols | m << 10 | words << 13 | polar << 19;
 // kNoFrame (no symbols) for a descriptor that names none.
@@ -691,9 +692,11 @@ __global__ void __launch_bounds__(kSortThreads) k_order_index(const __grid_const
 }
 
 template <int kFrom, int kMap, int kSlots>
-__global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWarps), kMap == kThread ? (kFrom == kFromMixed ? kOrderCtas : kThreadCtas) : 8) k_decode(const __grid_constant__ DecodeArgs a) {
-  constexpr int kWarps = kMap == kThread ? kThreadWarps : kCtaWarps;
-  constexpr bool kOne = kMap == kWarpShort, kRows = kMap == kThread;
+__global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWarps),
+                                  kMap >= kThread ? (kFrom == kFromMixed ? kOrderCtas : kThreadCtas) : 8)
+    k_decode(const __grid_constant__ DecodeArgs a) {
+  constexpr int kWarps = kMap >= kThread ? kThreadWarps : kCtaWarps;
+  constexpr bool kOne = kMap == kWarpShort, kRows = kMap >= kThread;
   extern __shared__ __align__(16) char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int FT = kWarps * a.T;
@@ -946,7 +949,8 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
       fetch(c + 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
       __syncwarp();
-      if (usual) step(std::true_type{}, c);
+      if constexpr (kMap == kThreadUsual) step(std::true_type{}, c);
+      else if (usual) step(std::true_type{}, c);
       else step(std::false_type{}, c);
       __syncwarp();
     }
@@ -1441,8 +1445,8 @@ __global__ void __launch_bounds__(32 * (kMap == kThread ? kThreadWarps : kCtaWar
 size_t decode_smem(bool mixed, int map, int slots, int T, int NWmax) {
   const int warps = warps_of(map);
   const size_t FT = (size_t)warps * T;
-  return (mixed ? FT * 24 + (map == kThread ? 0 : 512) : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
-         (map == kThread ? (size_t)warps * kStages * kStageSyms * 8 : 0) +
+  return (mixed ? FT * 24 + (map >= kThread ? 0 : 512) : 0) + (map == kWarpShort ? FT * 8 * (slots / 2) : 0) +
+         (map >= kThread ? (size_t)warps * kStages * kStageSyms * 8 : 0) +
          4 * (32 + 2 * FT + (slots / 2) * FT + NWmax * (FT + 1));
 }
 
@@ -1478,11 +1482,11 @@ int preload_decode_kernels() {
 constexpr int64_t kThreadFrames = 16384;
 
 // Uneven batches from here on are put in order first and prepared by a thread
-// per frame. A thread takes 50 us for a frame of 512 symbols whatever the
+// per frame. A thread takes 40 us for a frame of 512 symbols whatever the
 // batch, so the warp per frame (45 us for 16,384 frames of every length, 62
-// for 32,768, 85 for 65,536, 160 for 131,072) is left only beyond 90,000
-// frames (88, 92, 100 and 132 us in order, the sort included).
-constexpr int64_t kOrderFrames = 98304;
+// for 32,768, 85 for 65,536, 160 for 131,072) is left only near 40,000 frames
+// (65, 67, 73 and 103 us in order, the sort included).
+constexpr int64_t kOrderFrames = 49152;
 
 size_t order_bytes(const DecodeArgs& a) {
   const int64_t wide = (int64_t)1 << 31;  // the records' frame, and symbol offsets, in 32 bits
@@ -1509,13 +1513,16 @@ int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const bool mixed = a.desc != nullptr, arrays = !mixed && a.symbols == nullptr;
   const QamConst qc = make_qam_const();
   for (int m = 1; m <= 6; ++m) a.ax[m] = axis_const(m, qc);
-  const int map = a.order ? kThread : !mixed && !arrays && a.n_frames >= kThreadFrames ? kThread : (!mixed && !arrays && Lmax <= 32 ? kWarpShort : kWarpLong);
+  const bool uniform = !mixed && !arrays, usual = m_of(a.M) <= 4 && !a.lik;
+  int map = uniform && Lmax <= 32 ? kWarpShort : kWarpLong;
+  if (a.order) map = kThread;
+  else if (uniform && a.n_frames >= kThreadFrames) map = usual ? kThreadUsual : kThread;
   // frames per warp: a thread per frame takes 32; else as many as keep every
   // SM full (each CTA holds the tile's solve in its first warps, so larger
   // tiles waste fewer lanes there)
   const int warps = warps_of(map);
   const int64_t slots_cta = (int64_t)sm_count() * 7;
-  const int64_t T = map == kThread ? 32 : (a.n_frames + slots_cta * warps - 1) / (slots_cta * warps);
+  const int64_t T = map >= kThread ? 32 : (a.n_frames + slots_cta * warps - 1) / (slots_cta * warps);
   a.m = m_of(a.M);
   a.T = (int)(T < 1 ? 1 : (T > 32 ? 32 : T));
   const int64_t grid = (a.n_frames + warps * a.T - 1) / (warps * a.T);
@@ -1523,9 +1530,10 @@ int launch_decode(DecodeArgs a, int Lmax, cudaStream_t st) {
   const void* kern = nullptr;
   if (mixed) kern = a.order ? pick_slots<kFromMixed, kThread>(Smax) : pick_slots<kFromMixed, kWarpLong>(Smax);
   else if (arrays) kern = pick_slots<kFromArrays, kWarpLong>(Smax);
+  else if (map == kThreadUsual) kern = pick_slots<kFromUniform, kThreadUsual>(Smax);
   else if (map == kThread) kern = pick_slots<kFromUniform, kThread>(Smax);
   else kern = map == kWarpShort ? pick_slots<kFromUniform, kWarpShort>(Smax) : pick_slots<kFromUniform, kWarpLong>(Smax);
-  if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB
+  if (smem > 48 * 1024) return GRAND_E_CUDA;  // not reachable: 4 x 32 frames of 32 words take 28 KB, a warp of rows 12 KB
   void* args[] = {&a};
   if (cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(32 * warps), args, smem, st) != cudaSuccess)
     return GRAND_E_CUDA;

@@ -71,7 +71,7 @@ def test_large_uneven_batch(S, lik, membership):
     H = r.integers(0, 2, (20, 64))
     H[:, r.permutation(64)[:20]] = np.eye(20, dtype=np.int64)
     codes.append(g.Code(g.H_from_dense(H), 64, 44))
-    F = 98304 + 1111
+    F = 49152 + 1111
     ci = r.integers(0, len(codes), F)
     M = np.asarray([4, 16, 64, 256, 1024, 4096])[r.integers(0, 6, F)]
     N = np.asarray([c.N for c in codes])[ci]
