@@ -991,7 +991,7 @@ def run_config(args, cfg, g, ctx):
                      "latency_ms": {"p50": float(np.percentile(s_ms, 50)), "p99": float(np.percentile(s_ms, 99))},
                      "kernel_ms": {"prep": rs["prep_ms"], "search": rs["search_ms"]},
                      "frames_to_tep_search": int(rs["hard_frames"]), "ranked_solutions": int(rs["evaluated_checks"]),
-                     "outputs_equal": bool(same), "graph": True, "profile": "profiles/k_prep_solve_c2_small.md",
+                     "outputs_equal": bool(same), "graph": True, "profile": "profiles/k_decode_thread.md",
                      "what": "the same batch with the first hit found by Gaussian elimination over each frame's TEP "
                              "coordinates (the codewords of the TEP space are the solutions of a GF(2) linear "
                              "system; the first hit is the one of smallest canonical rank): same outputs, no TEP "
@@ -1059,7 +1059,21 @@ def run_config(args, cfg, g, ctx):
 
     # ---- roofline of the dominant kernel (the TEP search)
     roofline = None
-    if sum(search_ms) > 0 and args.membership == "auto":  # TEPs tested one by one
+    if cfg["kind"] in ("qam", "mixed") and args.membership == "auto" and not any(p.tiles[:2]):
+        # automatic tiles: one kernel decides all TEPs of a frame at once, so
+        # its unit is the data it cannot do without
+        alg_bytes = d_sym.numel() * d_sym.element_size() + 5 * n_frames + 4 * d_cw.numel()
+        if cfg["kind"] == "mixed":
+            alg_bytes += d_desc.numel()
+        peak, peak_source = hbm_peak()
+        t_ms = statistics.mean(step_ms)
+        roofline = {"bound": "hbm", "kernel": "k_decode", "kernel_ms": t_ms, "peak": peak, "unit": "GB/s",
+                    "peak_source": peak_source, "achieved": alg_bytes / t_ms / 1e6,
+                    "frac": alg_bytes / t_ms / 1e6 / peak, "algorithmic_bytes": int(alg_bytes), "traffic": None,
+                    "note": "first hit from the frame's GF(2) system: useful checks are the positions of the first "
+                            "hits (or the cap), none is tested by itself; issue-bound in ncu",
+                    "profile": "profiles/k_decode_thread.md"}
+    elif sum(search_ms) > 0 and args.membership == "auto":  # TEPs tested one by one
         roofline = search_roofline(cfg, evaluated / args.steps, search_useful / args.steps, hard / args.steps,
                                    statistics.mean(search_ms), alg_words, frames=n_frames)
 
@@ -1151,7 +1165,7 @@ def run_serve_config(args, cfg, g, ctx):
             "config": {"workload": cfg["desc"], "requests_per_rate": len(inputs["N"]),
                        "server": f"max_slots 262144, budget 1 GiB, max_batch {args.serve_batch}, "
                                  f"{args.serve_streams} streams",
-                       "membership": {"auto": "split search (TEP by TEP)", "hash": "hash join",
+                       "membership": {"auto": "library's choice", "hash": "hash join",
                                       "solve": "linear solve (GRAND_MEMBERSHIP_SOLVE)"}[args.membership]},
             "latency_us": head["latency_us"], "rates": rows, "one_frame_per_launch": one, "clocks": clk,
             "e2e": {"value": head["frames_per_s"], "unit": "frames/s",

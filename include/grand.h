@@ -92,8 +92,8 @@ typedef enum grand_order {
  *   AUTO        the library's choice. QAM_NNE / QAM_NEARER with automatic
  *               tiles[0] and tiles[1] and no deadline: the linear system of
  *               SOLVE below, which decides all valid TEPs of a frame at once
- *               (one kernel; scratch, 32 B a frame, only
- *               for uneven batches of 49,152 frames and more). With an explicit tiles[0] or
+ *               (one kernel; scratch, 32 B a frame, only for uneven batches
+ *               of 49,152 frames and more). With an explicit tiles[0] or
  *               tiles[1], a deadline, or in the resumable search: syndrome
  *               deltas (Alg. 2 Step 4: s(y) xor the H columns a TEP flips)
  *               compared TEP by TEP in the split search. QAM_NNE5: DELTA for
