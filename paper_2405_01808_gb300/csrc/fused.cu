@@ -25,7 +25,7 @@
 //          lanes, where the warp per frame spends 10 warp minima at a quarter
 //          of the issue rate and a label reduction a step: 416 warp
 //          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
-//          frames 137 -> 54 us, N=128 300,000 frames 91 -> 62 us, N=512 S=12
+//          frames 137 -> 53 us, N=128 300,000 frames 91 -> 65 us, N=512 S=12
 //          80,000 frames 76 -> 38 us, uneven mix of 10^6 frames 904 -> 587 us.
 //          What is left of a frame is its hard word and S' symbol records in
 //          shared memory.
