@@ -352,7 +352,7 @@ __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, c
         if (hi && wd + 1 < NW) atomicOr(&sm.y[wd + 1], hi);
       } else {
         const int64_t o = f * (int64_t)L + i;
-        key = a.key[o];
+        key = selection_key(a.key[o]);
         const uint32_t hidx = a.hard_idx[o];
         const uint32_t nm = a.nmask[o];
         nonfinite |= (nm & 128u) != 0;
@@ -430,7 +430,7 @@ __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, c
     if (L <= 32) {
       // one symbol per lane: S' rounds of the warp minimum of the keys; ties
       // go to the lowest index (the lowest lane of the ballot)
-      uint32_t k_i = lane < L ? sm.key[lane] : 0xFFFFFFFFu;  // keys are < 2^31
+      uint32_t k_i = lane < L ? sm.key[lane] : 0xFFFFFFFFu;  // (above every key)
       for (int r = 0; r < Sp; ++r) {
         const uint32_t kmin = __reduce_min_sync(kFull, k_i);
         const int win = __ffs(__ballot_sync(kFull, k_i == kmin)) - 1;
@@ -446,7 +446,7 @@ __device__ __forceinline__ bool prep_frame(const PrepArgs& a, const int64_t f, c
       }
       const uint32_t kmin = __reduce_min_sync(kFull, best_k);
       const uint32_t imin = __reduce_min_sync(kFull, best_k == kmin ? best_i : 0xFFFFFFFFu);
-      if (lane == (int)(imin & 31u)) sm.key[imin] = 0xFFFFFFFFu;  // keys are < 2^31
+      if (lane == (int)(imin & 31u)) sm.key[imin] = 0xFFFFFFFFu;  // above every key
       if (lane == r) my_sel = (int)imin;
       __syncwarp();
     }

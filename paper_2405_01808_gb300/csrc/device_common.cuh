@@ -144,22 +144,33 @@ __device__ __forceinline__ uint32_t make_nmask(const AxisDemod& I, const AxisDem
   return m;
 }
 
-// Frame bit positions flipped by the horizontal / vertical alternative of a
-// symbol (a neighbouring level differs from the hard level in exactly one bit
-// of the binary-reflected Gray label: bit ctz(max(l, l')) of the m-bit label).
-// Labels are MSB first: I label bits occupy [2m i, 2m i + m), Q label bits
-// [2m i + m, 2m i + 2m). Returns kNoPos if the position is beyond N.
-__device__ __forceinline__ uint16_t flip_pos_I(int i, int m, int l, int dir, int N) {
-  const int hi = l > l + dir ? l : l + dir;
-  const int b = __ffs(hi) - 1;
-  const int p = 2 * m * i + (m - 1 - b);
-  return p < N ? (uint16_t)p : kNoPos;
+// Frame bit position flipped by an axis's alternative (a neighbouring level
+// differs from the hard level in exactly one bit of the binary-reflected Gray
+// label: bit ctz(hi) of the m-bit label, hi = the larger of the two levels).
+// Labels are MSB first: symbol i's I label ends before `end` = 2m i + m, its Q
+// label before 2m i + 2m. kNoPos outside the word: padding, or a level that the
+// constellation does not have (a caller's demodulated arrays are not checked:
+// such a level can name a position before the word or far behind it).
+__host__ __device__ __forceinline__ uint32_t flip_pos(int end, int hi, int N) {
+#ifdef __CUDA_ARCH__
+  const int p = end - __ffs(hi);
+#else
+  const int p = end - __builtin_ffs(hi);
+#endif
+  return (uint32_t)p < (uint32_t)N ? (uint32_t)p : (uint32_t)kNoPos;
 }
-__device__ __forceinline__ uint16_t flip_pos_Q(int i, int m, int l, int dir, int N) {
-  const int hi = l > l + dir ? l : l + dir;
-  const int b = __ffs(hi) - 1;
-  const int p = 2 * m * i + (2 * m - 1 - b);
-  return p < N ? (uint16_t)p : kNoPos;
+__host__ __device__ __forceinline__ uint16_t flip_pos_I(int i, int m, int l, int dir, int N) {
+  return (uint16_t)flip_pos(2 * m * i + m, l > l + dir ? l : l + dir, N);
+}
+__host__ __device__ __forceinline__ uint16_t flip_pos_Q(int i, int m, int l, int dir, int N) {
+  return (uint16_t)flip_pos(2 * m * i + 2 * m, l > l + dir ? l : l + dir, N);
+}
+
+// Ordering key of a caller's demodulated array as the selections take it: the
+// largest 32-bit value marks "no symbol" there, so it is read as the one below
+// (demodulation stays below 2^31).
+__host__ __device__ __forceinline__ uint32_t selection_key(uint32_t key) {
+  return key < 0xFFFFFFFEu ? key : 0xFFFFFFFEu;
 }
 
 // ---------------------------------------------------------------------------

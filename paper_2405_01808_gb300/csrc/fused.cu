@@ -130,7 +130,7 @@ enum { kFromUniform = 0, kFromMixed = 1, kFromArrays = 2 };
 __device__ __forceinline__ Alt array_alt(const DecodeArgs& a, int64_t o) {
   const uint32_t h = a.hard_idx[o], nm = a.nmask[o];
   // the threshold toward the neighbour (where there is none the value is not used)
-  return Alt{((h >> 8) + ((nm >> 3) & 1u) - 1u) & 63u, ((h & 0xFFu) + ((nm >> 4) & 1u) - 1u) & 63u, (nm & 1u) != 0,
+  return Alt{(h >> 8) + ((nm >> 3) & 1u) - 1u, (h & 0xFFu) + ((nm >> 4) & 1u) - 1u, (nm & 1u) != 0,
              (nm & 2u) != 0, (nm & 32u) != 0};
 }
 
@@ -161,7 +161,7 @@ __device__ __noinline__ int select_exact(const DecodeArgs& a, int64_t base, int 
     uint32_t bk = kNone, bi = kNone;
     for (int i = lane; i < L; i += 32) {
       uint32_t k;
-      if constexpr (kFrom == kFromArrays) k = a.key[base + i];
+      if constexpr (kFrom == kFromArrays) k = selection_key(a.key[base + i]);
       else k = symbol_key(a.symbols[base + i], a.ax[m].q.x, m, a.lik);
       const bool after = k > last_k || (k == last_k && i > last_i);
       if (after && k < bk) { bk = k; bi = (uint32_t)i; }
@@ -1262,13 +1262,12 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
         // slots of rank r (symbol idx) from its alternatives: their positions,
         // entered in rec, ex and real
         auto enter = [&](int r, uint32_t idx, const Alt& t, uint32_t& p0, uint32_t& p1) {
-          // the neighbour across threshold k differs from the hard level in
-          // the Gray label's bit ctz(k + 1)
-          const int pI = 2 * m * (int)idx + m - __ffs((int)t.kI + 1);
-          const int pQ = 2 * m * (int)idx + 2 * m - __ffs((int)t.kQ + 1);
+          // (threshold k lies between the levels k and k + 1)
+          const uint32_t pI = flip_pos(2 * m * (int)idx + m, (int)(t.kI + 1u), N);
+          const uint32_t pQ = flip_pos(2 * m * (int)idx + 2 * m, (int)(t.kQ + 1u), N);
           uint32_t e0 = r < Sp && t.exI, e1 = r < Sp && t.exQ;
-          p0 = e0 && pI < N ? (uint32_t)pI : kNoPos;
-          p1 = e1 && pQ < N ? (uint32_t)pQ : kNoPos;
+          p0 = e0 ? pI : kNoPos;
+          p1 = e1 ? pQ : kNoPos;
           if (a.nearer && t.near) {  // the nearer (vertical) alternative takes the first slot
             const uint32_t tp = p0, te = e0;
             p0 = p1; p1 = tp;
