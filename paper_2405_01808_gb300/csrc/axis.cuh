@@ -12,6 +12,7 @@ namespace grand {
 // arithmetic on both axes (axes_fast): each value twice.
 struct AxisConst {
   float2 q;      // 256 / d
+  float2 nz;     // -0 (see grid2)
   float2 t0;     // -(1.5 * 2^23 - 256 sqrt(M) + 512)
   float2 g;      // sqrt(M) - 2: the range of the thresholds' indices
   float s, c;    // t s + c: that range scaled to [0, 1]
@@ -29,6 +30,7 @@ inline AxisConst axis_const(int m, const QamConst& qc) {
   auto twice = [](double v) { return make_float2((float)v, (float)v); };
   AxisConst c;
   c.q = make_float2(qc.q[m], qc.q[m]);
+  c.nz = make_float2(-0.0f, -0.0f);
   c.t0 = twice(-(12582912.0 - 256.0 * side + 512.0));
   c.g = twice(range);
   c.s = m > 1 ? (float)(1.0 / (512.0 * range)) : 0.0f;
@@ -89,12 +91,13 @@ struct Axes {
 // the compiler from building the pairs anew for every symbol (packed
 // instructions take no immediates), which was 30 of 240 instructions a frame.
 struct AxisRegs {
-  F2 q, t0, g, magic, unmagic, m512;
+  F2 q, nz, t0, g, magic, unmagic, m512;
   float s, c, lim, side;
 };
-__device__ __forceinline__ AxisRegs axis_regs(const AxisConst& a) {
+__device__ __forceinline__ AxisRegs axis_regs(const AxisConst& a, float2 nz) {
   AxisRegs r;
   r.q = pack2(a.q);
+  r.nz = pack2(nz);
   r.t0 = pack2(a.t0);
   r.g = pack2(a.g);
   r.magic = pack2(kMagic, kMagic);
@@ -107,6 +110,14 @@ __device__ __forceinline__ AxisRegs axis_regs(const AxisConst& a) {
   r.side = a.side;
   return r;
 }
+// Both coordinates on the grid, rounded to float as the definition has it. A
+// multiply-add with -0, which no compiler can know to be one: left as a product
+// (mul.rn.f32x2), it was joined with the addition of 1.5 * 2^23 that follows,
+// .rn notwithstanding, and a product that rounds to a half (-768.5) went to the
+// other integer. That moved a threshold's distance by one: 4 of 200,000 frames
+// had an alternative too few.
+__device__ __forceinline__ F2 grid2(F2 v, const AxisRegs& c) { return fma2(v, c.q, c.nz); }
+
 __device__ __forceinline__ Axes axes_fast(F2 x, const AxisRegs& c) {
   const F2 t = add2(add2(x, c.magic), c.t0);  // round(x) + 256 sqrt(M) - 512
   const float2 ts = unpack2(t);

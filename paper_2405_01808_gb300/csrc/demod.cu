@@ -65,7 +65,7 @@ __device__ __noinline__ Out demod_far(float q, float inv_d, float2 v) {
 template <int kM, int kLit>
 __device__ __forceinline__ Out demod_one(const AxisRegs& ax, F2 inv_d, float2 v) {
   const F2 raw = pack2(v);
-  const F2 x = mul2(raw, ax.q);
+  const F2 x = grid2(raw, ax);
   const float2 xs = unpack2(x);
   if (!(fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim)) 
     return demod_far<kM, kLit>(unpack2(ax.q).x, unpack2(inv_d).x, v);
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kThreads, kV == 4 ? 6 : 8) k_demod(const __gri
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int64_t s0 = t * kV;
   const int n = (int)min((int64_t)kV, max((int64_t)0, a.n_sym - s0));  // symbols of this thread
-  const AxisRegs ax = axis_regs(a.ax);
+  const AxisRegs ax = axis_regs(a.ax, a.ax.nz);
   const F2 inv_d = pack2(a.inv_d);
   float2 v[kV];
 #pragma unroll

@@ -92,7 +92,7 @@ struct Alt {
   bool exI, exQ, near;
 };
 __device__ __forceinline__ Alt symbol_alt(float2 v, const AxisRegs& c, int lik) {
-  const Axes x = axes_fast(mul2(pack2(v), c.q), c);
+  const Axes x = axes_fast(grid2(pack2(v), c), c);
   const float2 e = x.e;
   return Alt{__float_as_uint(x.kb.x) & 63u, __float_as_uint(x.kb.y) & 63u, fabsf(e.x) <= 256.0f, fabsf(e.y) <= 256.0f,
              axis_dist(e.y, lik) < axis_dist(e.x, lik)};
@@ -422,7 +422,7 @@ struct Step {
 // nf: set when a symbol is not finite (its coordinates are read as 0).
 __device__ __forceinline__ Step demod_step(const DecodeArgs& a, const AxisRegs& ax, float2 cur, int m, uint32_t index,
                                            bool on, bool& nf) {
-  F2 x = mul2(pack2(cur), ax.q);
+  F2 x = grid2(pack2(cur), ax);
   const float2 xs = unpack2(x);
   const bool plain = fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim;
   uint32_t big = 0;  // key of a symbol outside the plain range
@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     const int m = kFrom == kFromMixed ? (int)((par >> 10) & 7u) : um;
     const int NW = kFrom == kFromMixed ? (int)((par >> 13) & 63u) : a.NWmax;
     const int Sp = a.S < L ? a.S : L;
-    const AxisRegs ax = axis_regs(a.ax[m]);
+    const AxisRegs ax = axis_regs(a.ax[m], a.ax[1].nz);
     int n_chunks = rows > 0 ? (L + kChunk - 1) / kChunk : 0;
     // the inner loop without the literal likelihood and symbols of more than 8 bits
     bool usual = !a.lik && m <= 4;
@@ -867,7 +867,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       float top = 0.0f;
 #pragma unroll
       for (int j = 0; j < kChunk; ++j) {
-        x[j] = mul2(pack2(row[j]), ax.q);
+        x[j] = grid2(pack2(row[j]), ax);
         const float2 xs = unpack2(x[j]);
         top = max_abs(top, xs.x, xs.y);
       }
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       if (wide) {
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) {
-          const float2 v = row[j], xs = unpack2(mul2(pack2(v), ax.q));
+          const float2 v = row[j], xs = unpack2(grid2(pack2(v), ax));
           if (!(fabsf(xs.x) <= ax.lim && fabsf(xs.y) <= ax.lim))
             kp[j] = (min(symbol_key(v, unpack2(ax.q).x, m, a.lik), kKeySat) << 9) | (uint32_t)(c * kChunk + j);
         }
@@ -986,7 +986,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   } else if constexpr (kOne) {
-    const AxisRegs ax = axis_regs(a.ax[um]);
+    const AxisRegs ax = axis_regs(a.ax[um], a.ax[1].nz);
     const int NW = a.NWmax, Sp = a.S < uL ? a.S : uL;
     const bool on = lane < uL;
     const uint32_t plan = pack_plan(um, lane);
@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
         nf = __any_sync(kAll, mine);
         if (lane < NW) y[lane * stride] = __brev(a.y_in[(tile + fr) * NW + lane]);
       } else {
-        const AxisRegs ax = axis_regs(a.ax[m]);
+        const AxisRegs ax = axis_regs(a.ax[m], a.ax[1].nz);
         const uint32_t plan = kFrom == kFromMixed ? s_plan[32 * ((m - 1) & 3) + lane] : pack_plan(um, lane);
         const int byte0 = (int)(plan >> 13);
         uint8_t* yb = reinterpret_cast<uint8_t*>(y) + (byte0 >> 2) * (4 * stride) + (~byte0 & 3);
@@ -1258,7 +1258,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       uint32_t c[kSlots];
       uint32_t real = 0;  // ex: existing slots; real: those whose flip lies inside the word
       {
-        const AxisRegs ax = axis_regs(a.ax[m]);
+        const AxisRegs ax = axis_regs(a.ax[m], a.ax[1].nz);
         // slots of rank r (symbol idx) from its alternatives: their positions,
         // entered in rec, ex and real
         auto enter = [&](int r, uint32_t idx, const Alt& t, uint32_t& p0, uint32_t& p1) {
