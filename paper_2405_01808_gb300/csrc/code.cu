@@ -95,13 +95,14 @@ extern "C" int grand_code_create(const uint32_t* H, int N, int K, grand_code** o
   // per-column projections hf[j] (a fixed pseudo-random 32-bit word per row,
   // from the splitmix64 finaliser of the row index)
   // layout of the device copy: hcol [N*W], hf [N], prow [R], frozen [R] (u16, packed 2 per word),
-  // hrow [R * N/32] (the rows as given), hx [N], fmask [N/32]
-  const size_t words = (size_t)N * W + N + R + (R + 1) / 2 + (size_t)R * (N / 32) + N + N / 32;
+  // hrow [R * N/32] (the rows as given, on 16 bytes), hx [N], fmask [N/32]
+  const size_t to_rows = ((size_t)R + (R + 1) / 2 + 3) / 4 * 4;  // words from prow to hrow
+  const size_t words = (size_t)N * W + N + to_rows + (size_t)R * (N / 32) + N + N / 32;
   std::vector<uint32_t> hcol(words, 0);
   uint32_t* hf = hcol.data() + (size_t)N * W;
   uint32_t* prow = hf + N;
   uint16_t* frozen = reinterpret_cast<uint16_t*>(prow + R);
-  uint32_t* hrow = prow + R + (R + 1) / 2;
+  uint32_t* hrow = prow + to_rows;
   uint32_t* hx = hrow + (size_t)R * (N / 32);
   uint32_t* fmask = hx + N;
   memcpy(hrow, H, sizeof(uint32_t) * (size_t)R * (N / 32));
@@ -167,7 +168,7 @@ extern "C" int grand_code_create(const uint32_t* H, int N, int K, grand_code** o
   c->dev.hf = c->d_hcol + (size_t)N * W;
   c->dev.prow = c->dev.hf + N;
   c->dev.frozen = reinterpret_cast<const uint16_t*>(c->dev.prow + R);
-  c->dev.hrow = c->dev.prow + R + (R + 1) / 2;
+  c->dev.hrow = c->dev.prow + to_rows;
   c->dev.hx = c->dev.hrow + (size_t)R * (N / 32);
   c->dev.fmask = c->dev.hx + N;
   c->dev.status = c->d_status;

@@ -559,6 +559,61 @@ __device__ __forceinline__ void merge_smallest(uint32_t (&best)[R], const uint32
 template <typename T>
 __device__ __forceinline__ T gray4(T v, T below_top) { return v ^ ((v >> 1) & below_top); }
 
+// Base syndrome of this thread's frame for H not of polar form: the parities of
+// its hard word under the rows, eight rows at a time (word w of the hard word
+// at y[w * stride], of the syndrome at out[32 w]). Returns the projection. A
+// row's words are the same in every thread of a code, so they come as
+// broadcasts, and the work is one three-input operation per row and word of a
+// warp's 32 frames; the sum of the columns of the one-bits, a warp per frame
+// and the frames one after the other, waited for its scattered loads: 20,000
+// frames of 1024 bits and 512 rows 1165 us, so 144.
+__device__ __noinline__ uint32_t row_syndrome(const uint32_t* __restrict__ hrow, const uint32_t* __restrict__ prow, int R,
+                                              int NW, const uint32_t* y, int stride, uint32_t* out) {
+  constexpr int kRowsAtOnce = 8;  // divides a word
+  uint32_t f0 = 0, word = 0;
+#pragma unroll 1
+  for (int r0 = 0; r0 < R; r0 += kRowsAtOnce) {
+    const int last = R - 1 - r0;  // rows beyond the last one repeat it
+    const uint32_t* h = hrow + (size_t)r0 * NW;
+    uint32_t acc[kRowsAtOnce];
+#pragma unroll
+    for (int i = 0; i < kRowsAtOnce; ++i) acc[i] = 0u;
+    if (NW >= 4) {
+#pragma unroll 1
+      for (int w = 0; w < NW; w += 4) {
+        const uint32_t y0 = y[w * stride], y1 = y[(w + 1) * stride], y2 = y[(w + 2) * stride], y3 = y[(w + 3) * stride];
+#pragma unroll
+        for (int i = 0; i < kRowsAtOnce; ++i) {
+          const uint4 v = __ldg(reinterpret_cast<const uint4*>(h + min(i, last) * NW + w));
+          acc[i] ^= v.x & y0;
+          acc[i] ^= v.y & y1;
+          acc[i] ^= v.z & y2;
+          acc[i] ^= v.w & y3;
+        }
+      }
+    } else {
+      for (int w = 0; w < NW; ++w) {
+        const uint32_t yw = y[w * stride];
+#pragma unroll
+        for (int i = 0; i < kRowsAtOnce; ++i) acc[i] ^= __ldg(h + min(i, last) * NW + w) & yw;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kRowsAtOnce; ++i) {
+      if (i <= last && (__popc(acc[i]) & 1)) {
+        word |= 1u << ((r0 & 31) + i);
+        f0 ^= __ldg(prow + r0 + i);
+      }
+    }
+    if ((r0 & 31) == 32 - kRowsAtOnce || last < kRowsAtOnce) {
+      out[r0 & ~31] = word;
+      if (R <= 32 && last < kRowsAtOnce) return word;  // one word: the syndrome itself
+      word = 0;
+    }
+  }
+  return f0;
+}
+
 // ---------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------
@@ -970,10 +1025,24 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       reselect(32 * warp + of, __shfl_sync(kAll, L, of), __shfl_sync(kAll, m, of), __shfl_sync(kAll, Sp, of),
                make_float2(0.0f, 0.0f));
     }
-    const bool plain_h = kFrom == kFromMixed ? (par >> 19) != 0u : u_polar;
-    for (unsigned todo = __ballot_sync(kAll, searched && !plain_h); todo; todo &= todo - 1u) {
-      const int of = __ffs(todo) - 1;
-      general_syndrome(32 * warp + of, __shfl_sync(kAll, NW, of));
+    const bool general = searched && !(kFrom == kFromMixed ? (par >> 19) != 0u : u_polar);
+    if (const unsigned todo = __ballot_sync(kAll, general)) {  // H not of polar form: the syndromes now
+      const CodeDev* code = codes + (kFrom == kFromMixed && general ? s_code[mine] : 0u);
+      uint32_t* y = buf + mine;
+      uint32_t* s = reinterpret_cast<uint32_t*>(stage) + lane;
+      if (general) {
+        for (int w = 0; w < NW; ++w) y[w * stride] = __brev(y[w * stride]);
+        s_f0[mine] = row_syndrome(code->hrow, code->prow, code->R, NW, y, stride, s);
+      }
+      __syncwarp();
+      for (unsigned t = todo; t; t &= t - 1u) {  // the hard words out before the syndromes take their place
+        const int of = 32 * warp + __ffs(t) - 1, words = __shfl_sync(kAll, NW, __ffs(t) - 1);
+        const int64_t co = kFrom == kFromMixed ? s_cw[of] : (tile + of) * (int64_t)words;
+        if (lane < words) a.cw[co + lane] = buf[lane * stride + of];
+      }
+      __syncwarp();
+      if (general)
+        for (int v = 0; v < code->W; ++v) y[v * stride] = s[32 * v];
     }
     // the selected symbols, rank by rank, on their way to where the chunks were
     __syncwarp();

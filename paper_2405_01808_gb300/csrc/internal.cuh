@@ -28,7 +28,8 @@ constexpr uint16_t kNoPos = 0xFFFF;  // alternative bit beyond N (padding): no s
 //          preparation computes it with log2 N butterfly stages instead of
 //          column loads; prow[r] = p_r (the projection word of row r).
 //   hrow[r * (N/32) + w] bit b = H[r][32 w + b]   (row r of H, as given to
-//          grand_code_create): the row-parity membership test.
+//          grand_code_create, 16-byte aligned): the row-parity membership
+//          test, base syndromes of large batches.
 //   status[0]: set (atomicOr 1) by a kernel that cut a frame at the call's
 //          deadline; status[1]: where grand_stream_status takes it to.
 //   polar form also: fmask[w] = the frozen bits among indices 32 w .. 32 w + 31
