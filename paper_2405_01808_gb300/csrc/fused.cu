@@ -1446,7 +1446,9 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
           for (int t = 0; t < d; ++t, free_slots &= free_slots - 1u)
             kv[t] = pivots_of(kv[t]) | (free_slots & (0u - free_slots));
           shared = d > kOwnDim;
-          if (shared && exact && d > 10) {  // few parity bits: most first hits weigh at most 1
+          // few parity bits: most first hits weigh at most 1 (20,000 frames of
+          // 32 bits with 2 parity bits 111 -> 33 us, of 128 with 16 54 -> 38)
+          if (shared && exact) {
             if (f0 == 0u) x = 0u;
             for (int r = 0; r < Sp && x == kNone; ++r) {
               const uint32_t e = (ex >> (2 * r)) & 3u;

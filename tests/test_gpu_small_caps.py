@@ -49,25 +49,35 @@ def test_outputs(g, N, K, M, S):
     code.close()
 
 
+def time(g, code, x, **kw):
+    import torch
+
+    ms = []
+    for _ in range(22):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        g.decode_symbols(code, g.Params.make(**kw), x)
+        b.record()
+        b.synchronize()
+        ms.append(a.elapsed_time(b))
+    return float(np.median(ms[2:]))
+
+
 def test_a_small_cap_bounds_the_work(g):
     """10 parity bits: half of the frames have no codeword among the 300 TEPs of the cap, and their 2^14 solutions
     are not walked for one."""
-    import torch
-
     code = g.Code.polar(128, 118)
     x = frames_of(g, 128, 118, 16, 20000, 4.0)
-
-    def time(cap):
-        ms = []
-        for _ in range(22):
-            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            a.record()
-            g.decode_symbols(code, g.Params.make(M=16, S=12, query_cap=cap), x)
-            b.record()
-            b.synchronize()
-            ms.append(a.elapsed_time(b))
-        return float(np.median(ms[2:]))
-
-    few, all_of_them = time(300), time(1 << 24)
+    few, all_of_them = (time(g, code, x, M=16, S=12, query_cap=cap) for cap in (300, 1 << 24))
     assert few < 0.7 * all_of_them, (few, all_of_them)
+    code.close()
+
+
+def test_two_parity_bits_are_not_slower_than_the_search(g):
+    """Two parity bits: nearly every frame has a codeword among the TEPs of one altered symbol. (A budget selects the
+    preparation and the search.)"""
+    code = g.Code.polar(32, 30)
+    x = frames_of(g, 32, 30, 16, 20000, 10.0)
+    one, search = (time(g, code, x, M=16, S=8, query_cap=1 << 16, deadline_ns=ns) for ns in (0, 10 ** 10))
+    assert one < search, (one, search)
     code.close()
