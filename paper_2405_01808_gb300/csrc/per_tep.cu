@@ -671,8 +671,14 @@ int run_per_tep(const grand_code* c, const grand_params* p, const void* symbols,
   a.queries = queries;
   a.abandon = abandon;
   // the join decides every TEP at once; DELTA and ROW_PARITY ask for the test
-  // of each
-  const bool join = p->order == GRAND_ORDER_QAM_NNE5 && p->membership == GRAND_MEMBERSHIP_AUTO;
+  // of each. Its cost does not depend on the cap (the lower side's table above
+  // all), the walk's grows with it: 3,000 frames of 128 bits, S' = 10 (a table
+  // of 3,125 entries) 114 - 142 us whatever the cap, the walk 43 us at 300
+  // TEPs, 60 at 800, 115 at 3,125; S' = 9, a table of 625 entries, 57 us.
+  int64_t table = 1;
+  for (int r = 0; r < a.Sp / 2; ++r) table *= 5;
+  const bool join =
+      p->order == GRAND_ORDER_QAM_NNE5 && p->membership == GRAND_MEMBERSHIP_AUTO && p->query_cap > table;
   // Weight 1 (41 TEPs) decides most frames that decode; walking weight 2 (720
   // more) costs more than it saves the join (134 against 125 us for 6,000 N=128
   // frames), except where it decides nearly every frame: with few parity bits,
