@@ -24,7 +24,7 @@
 // 5^5 = 3,125) go into a hash table in shared memory and those of the upper
 // ranks are looked up. 6,250 table steps take the place of up to 5^10 =
 // 9,765,625 TEPs tested one by one: 6,000 frames (N=128 16-QAM, 6/8/10 dB,
-// S=10, cap 2^20) 32 ms -> 0.12 ms. What is left is latency (37 % issue): the
+// S=10, cap 2^20) 32 ms -> 0.11 ms. What is left is latency (37 % issue): the
 // CTA's warps wait for one another between the preparation and the joins.
 
 #include <stdint.h>
@@ -169,16 +169,33 @@ __device__ __forceinline__ int join_unpack(uint32_t code, uint64_t& pp, uint32_t
   return w;
 }
 
+// Entry n of the lower side's table (its number) and the code c of projection z,
+// where projections are syndromes: 0 when they differ, else 1 when the entry
+// comes first in the order, 2 when c does.
+__device__ __noinline__ int join_alike(const JoinFrame& f, int loA, const uint2* high, uint32_t n, uint32_t c,
+                                       uint32_t z) {
+  bool none;
+  const Part lo = join_part(f, 0, loA, n & 127u, none);
+  if ((lo.z ^ high[n >> 7].y) != z) return 0;
+  return join_key(lo.code | high[n >> 7].x) < join_key(c) ? 1 : 2;
+}
+
 // Hash join of the lower ranks [0, S'/2) with the upper ones, by the whole
 // CTA. A thread holds one digit vector of a side's first three ranks and goes
 // through those of the other two (at most 25, kept in `high`), kJoinStep table
 // accesses in flight at a time. Slots hold 20 bits of the mixed key and the
 // entry's number + 1 (low index + 128 x high index); equal ones are confirmed
-// on every syndrome word. *best: the smallest join_key of a codeword
+// on every syndrome word. Where a syndrome has one word (and is its own
+// projection) the first in the order of the lower codes that change it alike
+// stays alone: with the same upper code the others come after it. (Few parity
+// bits leave few syndromes; all of their codes in the table made chains that
+// every look-up walked: 300 frames of 128 bits with 6 parity bits 4509 us, so
+// 75.) *best: the smallest join_key of a codeword
 // (initialised by the caller).
 __device__ void join_sides(const CodeDev& code, const JoinFrame& f, uint32_t* table, uint2 (*high)[32],
                            unsigned long long* best) {
   constexpr int kThreads = 32 * kTepWarps;
+  const bool exact = code.W == 1;
   const int nA = f.Sp >> 1, nB = f.Sp - nA;
   const int loA = min(nA, kLowRanks), loB = min(nB, kLowRanks);
   const uint32_t t = threadIdx.x;
@@ -205,11 +222,23 @@ __device__ void join_sides(const CodeDev& code, const JoinFrame& f, uint32_t* ta
         was[u] = h < sizeA ? atomicCAS(table + (k[u] >> (32 - kSlotBits)), 0u, (k[u] << 12) | (t + 128u * h + 1u)) : 0u;
       }
 #pragma unroll
-      for (int u = 0; u < kJoinStep; ++u) {  // taken: the next free slot
+      for (int u = 0; u < kJoinStep; ++u) {  // taken: alike, or the next free slot
+        const uint32_t entry = (k[u] << 12) | (t + 128u * (h0 + u) + 1u);
         uint32_t slot = k[u] >> (32 - kSlotBits);
         while (was[u] != 0u) {
+          if (exact && !((was[u] ^ entry) >> 12)) {
+            const uint2 hi = high[0][(h0 + u) & 31u];
+            const int alike = join_alike(f, loA, high[0], (was[u] & 4095u) - 1u, lo.code | hi.x, lo.z ^ hi.y);
+            if (alike == 1) break;
+            if (alike == 2) {
+              const uint32_t seen = atomicCAS(table + slot, was[u], entry);
+              if (seen == was[u]) break;
+              was[u] = seen;  // another thread was here: look again
+              continue;
+            }
+          }
           slot = (slot + 1u) & (kSlots - 1u);
-          was[u] = atomicCAS(table + slot, 0u, (k[u] << 12) | (t + 128u * (h0 + u) + 1u));
+          was[u] = atomicCAS(table + slot, 0u, entry);
         }
       }
     }
@@ -281,6 +310,7 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
   const int warp = threadIdx.x >> 5;
   const CodeDev& code = a.code;
   const int N = code.N, NW = N >> 5, L = a.L, Sp = a.Sp, m = a.m;
+  const uint32_t* proj = kJoin && code.W == 1 ? code.hcol : code.hf;  // one word: the syndrome itself
   const size_t warp_bytes = tep_warp_bytes(L, NW, a.rowparity);
   uint32_t* table = reinterpret_cast<uint32_t*>(smem_raw);  // [kSlots], join only
   char* const bases = smem_raw + (kJoin ? sizeof(uint32_t) * kSlots : 0);
@@ -388,7 +418,7 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
 #pragma unroll
           for (int k = 0; k < kWMax; ++k)
             if (k < code.W) s[k] ^= __ldg(code.hcol + (size_t)j * code.W + k);
-          f0 ^= __ldg(code.hf + j);
+          f0 ^= __ldg(proj + j);
         }
       }
 #pragma unroll
@@ -452,7 +482,7 @@ __global__ void __launch_bounds__(32 * kTepWarps) k_per_tep(TepArgs a) {
         const uint32_t p0 = ap & 0xFFFFu, p1 = ap >> 16;
         apos[lane * kAltMax + k] = ap;
         aproj[lane * kAltMax + k] =
-            (p0 != kNoPos ? __ldg(code.hf + p0) : 0u) ^ (p1 != kNoPos ? __ldg(code.hf + p1) : 0u);
+            (p0 != kNoPos ? __ldg(proj + p0) : 0u) ^ (p1 != kNoPos ? __ldg(proj + p1) : 0u);
       }
       kk[lane] = (uint8_t)n;
     }
@@ -675,15 +705,22 @@ int run_per_tep(const grand_code* c, const grand_params* p, const void* symbols,
   // all), the walk's grows with it: 3,000 frames of 128 bits, S' = 10 (a table
   // of 3,125 entries) 114 - 142 us whatever the cap, the walk 43 us at 300
   // TEPs, 60 at 800, 115 at 3,125; S' = 9, a table of 625 entries, 57 us.
-  int64_t table = 1;
+  int64_t table = 1, walked = 0;
   for (int r = 0; r < a.Sp / 2; ++r) table *= 5;
-  const bool join =
-      p->order == GRAND_ORDER_QAM_NNE5 && p->membership == GRAND_MEMBERSHIP_AUTO && p->query_cap > table;
   // Weight 1 (41 TEPs) decides most frames that decode; walking weight 2 (720
   // more) costs more than it saves the join (134 against 125 us for 6,000 N=128
-  // frames), except where it decides nearly every frame: with few parity bits,
-  // whose space is full of codewords for the join to compare.
-  a.walk = c->R <= 12 ? 2 : 1;
+  // frames). With few parity bits, whose space is full of codewords, weights 2
+  // and 3 (8,400 TEPs) leave the join little but frames that the walk would
+  // search to the cap: 300 frames of 128 bits with 6 parity bits 75 us (137 with
+  // weight 2, 92 without the join), 6 frames with 11 parity bits 72 (159, 89).
+  a.walk = c->R <= 12 ? 3 : 1;
+  int64_t count = 1;  // TEPs of weight w: C(S', w) 4^w
+  for (int w = 0; w <= a.walk && w <= a.Sp; ++w) {
+    walked += count;
+    count = count * 4 * (a.Sp - w) / (w + 1);
+  }
+  const bool join = p->order == GRAND_ORDER_QAM_NNE5 && p->membership == GRAND_MEMBERSHIP_AUTO &&
+                    p->query_cap > (table > walked ? table : walked);
   auto kern = join ? k_per_tep<true> : k_per_tep<false>;
   char* scratch = nullptr;
   if (scratch_alloc((void**)&scratch, 64, st) != cudaSuccess) return GRAND_E_NOMEM;

@@ -43,3 +43,25 @@ def test_small_caps(g, S, cap):  # noqa: F811
 @pytest.mark.parametrize("S,cap", [(10, 3126), (10, 3127), (9, 626), (8, 626), (1, 2)])
 def test_first_caps_of_the_join(g, S, cap):  # noqa: F811
     both(g, 128, 64, S, cap, 6.0, 500, reps=3)
+
+
+@pytest.mark.parametrize("N,K,S,cap,snr", [(128, 122, 10, 1 << 20, 8.0), (128, 120, 10, 1 << 20, 8.0),
+                                           (128, 116, 10, 5000, 6.0), (32, 24, 8, 1 << 20, 3.0), (128, 118, 9, 1 << 20, 6.0)])
+def test_few_parity_bits(g, N, K, S, cap, snr):  # noqa: F811
+    chosen, walk = both(g, N, K, S, cap, snr, 300)
+    assert chosen < 1.5 * walk, (chosen, walk)
+
+
+@pytest.mark.parametrize("kind,N,R,S", [("units", 128, 40, 10), ("units", 64, 14, 10), ("sparse", 256, 36, 9),
+                                        ("sparse", 128, 14, 10)])
+def test_repeated_columns(g, kind, N, R, S):  # noqa: F811
+    """Many lower codes of one syndrome, confirmed on one and two syndrome words."""
+    import torch
+    from test_gpu_fused import matrix, symbols_of
+
+    code = g.Code(g.H_from_dense(matrix(kind, N, R, N + S)), N, N - R)
+    x = torch.from_numpy(symbols_of(N, 4, 90, 4.0, R)).cuda()
+    a, b = (g.decode_symbols(code, g.Params.make(order=g.ORDER_QAM_NNE5, M=4, S=S, query_cap=1 << 20, membership=m), x)
+            for m in (g.MEMBERSHIP_AUTO, g.MEMBERSHIP_DELTA))
+    assert_equal(a, b, kind)
+    code.close()
