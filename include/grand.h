@@ -131,7 +131,8 @@ typedef enum grand_order {
  *               Outputs are those of AUTO (decoded word, query count = the
  *               hit's position in the canonical order, abandon flag); stats
  *               count the solutions looked at as checks and no searched
- *               frames. tiles are not used, and a deadline cuts no frame.
+ *               frames. tiles are not used. A deadline cuts the frames whose
+ *               solution set has more than 2^8 members and is walked late.
  *               QAM_NNE / QAM_NEARER (uniform and uneven batches); not for
  *               QAM_NNE5, HAMMING, the resumable search, the autotuner or
  *               the no-allocation entry point. */
@@ -185,8 +186,10 @@ typedef enum grand_lik {
  *               warp that fetches a frame after the budget ran out does not
  *               search it: the frame gets abandon = 5, cw = the hard word and
  *               queries = the number of leading valid TEPs already tested
- *               without a hit (those of the preparation stage; 0 for
- *               HAMMING, QAM_NNE5 and the DELTA / ROW_PARITY tests), and the
+ *               without a hit (those of the preparation stage; SOLVE: those
+ *               of at most one altered symbol where H has at most 32 rows,
+ *               else 0; 0 for HAMMING, QAM_NNE5 and the DELTA / ROW_PARITY
+ *               tests), and the
  *               code's status word is set for grand_stream_status. A frame
  *               whose search has started finishes (at most one frame's search
  *               per warp beyond the budget); frames the preparation resolves

@@ -2646,9 +2646,10 @@ static DecodeArgs decode_args(const PrepArgs& a, const grand_params* p, int n_co
   return d;
 }
 
-// The one-kernel decode: no scratch but the counters of a call with stats and
-// the order of a large uneven batch (where there is no memory for the order,
-// the batch is decoded as it comes).
+// The one-kernel decode: no scratch but the counters of a call with stats, the
+// clock of one with a deadline (linear solve) and the order of a large uneven
+// batch (where there is no memory for the order, the batch is decoded as it
+// comes).
 static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_params* p, int64_t n_frames,
                      grand_stats* stats, cudaStream_t st) {
   DecodeArgs a = decode_args(proto, p, n_codes, n_frames);
@@ -2663,20 +2664,31 @@ static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_p
     const int rc = order ? launch_order(a, order, st) : GRAND_OK;
     return rc == GRAND_OK ? launch_decode(a, Lmax, st) : rc;
   };
-  if (!stats) {
+  if (!stats && p->deadline_ns == 0) {
     const int rc = launch();
     if (order) cudaFreeAsync(order, st);
     return rc;
   }
-  if (scratch_alloc((void**)&a.scr, sizeof(Scratch), st) != cudaSuccess) {
+  Scratch* scr = nullptr;
+  if (scratch_alloc((void**)&scr, sizeof(Scratch), st) != cudaSuccess) {
     if (order) cudaFreeAsync(order, st);
     return GRAND_E_NOMEM;
   }
+  a.scr = stats ? scr : nullptr;
+  a.t0 = &scr->t0;
+  a.deadline = p->deadline_ns;
   int rc = GRAND_OK;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   do {
-    if (cudaMemsetAsync(a.scr, 0, sizeof(Scratch), st) != cudaSuccess || cudaEventCreate(&ev[0]) != cudaSuccess ||
-        cudaEventCreate(&ev[1]) != cudaSuccess) {
+    if (cudaMemsetAsync(scr, 0, sizeof(Scratch), st) != cudaSuccess) {
+      rc = GRAND_E_CUDA;
+      break;
+    }
+    if (!stats) {
+      rc = launch();
+      break;
+    }
+    if (cudaEventCreate(&ev[0]) != cudaSuccess || cudaEventCreate(&ev[1]) != cudaSuccess) {
       rc = GRAND_E_CUDA;
       break;
     }
@@ -2684,7 +2696,7 @@ static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_p
     if ((rc = launch()) != GRAND_OK) break;
     cudaEventRecord(ev[1], st);
     Scratch h{};
-    if (cudaMemcpyAsync(&h, a.scr, sizeof(Scratch), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(&h, scr, sizeof(Scratch), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
       rc = GRAND_E_CUDA;
       break;
@@ -2697,7 +2709,7 @@ static int run_fused(const PrepArgs& proto, int Lmax, int n_codes, const grand_p
   } while (0);
   for (int i = 0; i < 2; ++i)
     if (ev[i]) cudaEventDestroy(ev[i]);
-  cudaFreeAsync(a.scr, st);
+  cudaFreeAsync(scr, st);
   if (order) cudaFreeAsync(order, st);
   return rc;
 }

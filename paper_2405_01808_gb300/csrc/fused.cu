@@ -53,6 +53,8 @@ constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low 
 constexpr uint32_t kPicked = 0xFFFFFFE0u;  // above those: a key taken as rank (low bits)
 constexpr int kLanePick = 4;            // smallest keys kept per lane of a long frame
 constexpr int kOwnDim = 3;              // kernels of up to this dimension are walked by the frame's thread
+constexpr int kCutDim = 8;              // frames of larger kernels are cut at the call's deadline
+constexpr uint32_t kCut = 0xFFFFFFFEu;  // in the place of a solution: cut at the deadline
 
 // e_v(n1, n3): valid TEPs altering exactly v of n1 ranks with one alternative
 // and n3 ranks with three = the coefficient of x^v in (1 + x)^n1 (1 + 3x)^n3;
@@ -421,6 +423,16 @@ __device__ __noinline__ uint32_t first_solution_warp(const Frame f, const Proj p
   return __reduce_min_sync(kAll, bk == kmin ? bx : kNone);
 }
 
+// The call's deadline has passed and the walk of a frame is not begun (all
+// arguments the same in every lane of the warp). Weights <= 1 have been tested
+// where the projection is the syndrome; a cap among them leaves nothing to walk.
+__device__ __noinline__ bool walk_is_late(const DecodeArgs& a, uint32_t ex, int Sp, bool exact) {
+  if (exact && (int64_t)valid_up_to(ex, Sp, 1) >= a.cap) return false;
+  int late = 0;
+  if ((threadIdx.x & 31) == 0) late = past_deadline(a.t0, a.deadline);
+  return __shfl_sync(kAll, late, 0) != 0;
+}
+
 // ---------------------------------------------------------------------------
 // Front helpers (one warp per frame, one symbol per lane and step)
 // ---------------------------------------------------------------------------
@@ -785,6 +797,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
   const int64_t tile = (int64_t)blockIdx.x * FT;
   const int n_here = (int)min((int64_t)FT, a.n_frames - tile);
 
+  if (a.deadline > 0 && threadIdx.x == 0) past_deadline(a.t0, a.deadline);  // start the call's clock
   if (threadIdx.x < 32) pat[threadIdx.x] = subset_pattern(threadIdx.x);
   for (int t = threadIdx.x; t < a.NWmax * stride; t += 32 * kWarps) buf[t] = 0u;
   for (int t = threadIdx.x; t < FT; t += 32 * kWarps) s_flag[t] = 0u;
@@ -1471,7 +1484,8 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     const Frame F = frame_of(of, proj);
     const int sp = __shfl_sync(kAll, Sp, src), dim = __shfl_sync(kAll, d, src);
     const uint32_t e = __shfl_sync(kAll, ex, src), p0 = __shfl_sync(kAll, f0, src), s0 = __shfl_sync(kAll, x0, src);
-    const uint32_t got = first_solution_warp(F, proj, e, sp, p0, F.W == 1, s0, kv, dim, src, a.cap);
+    const bool late = a.deadline > 0 && dim > kCutDim && walk_is_late(a, e, sp, F.W == 1);
+    const uint32_t got = late ? kCut : first_solution_warp(F, proj, e, sp, p0, F.W == 1, s0, kv, dim, src, a.cap);
     if (lane == src) x = got;
   }
 
@@ -1486,11 +1500,18 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       const uint32_t exh = ex & 0x55555555u, exv = (ex >> 1) & 0x55555555u;
       const uint32_t one = exh ^ exv, both = exh & exv;
       const uint32_t total = 1u << __popc(ex);
-      const uint32_t pos = x != kNone ? tep_position(x, one, both) : 0u;
-      const bool hit = x != kNone && (uint64_t)pos <= (uint64_t)a.cap;
-      const uint32_t qn = hit ? pos : (uint32_t)((uint64_t)total < (uint64_t)a.cap ? total : (uint64_t)a.cap);
+      const uint32_t pos = x < kCut ? tep_position(x, one, both) : 0u;
+      const bool hit = x < kCut && (uint64_t)pos <= (uint64_t)a.cap;
+      uint32_t qn = hit ? pos : (uint32_t)((uint64_t)total < (uint64_t)a.cap ? total : (uint64_t)a.cap);
+      uint8_t ab = hit ? 0 : 1;
+      if (x == kCut) {
+        const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
+        qn = code->W == 1 ? valid_up_to(ex, Sp, 1) : 0u;
+        ab = 5;
+        atomicOr(code->status, 1u);
+      }
       a.queries[f] = qn;
-      a.abandon[f] = hit ? 0 : 1;
+      a.abandon[f] = ab;
       if (hit) {
         for (uint32_t t = x; t; t &= t - 1u) {
           const int b = __ffs(t) - 1;
@@ -1501,7 +1522,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       if (a.scr) {
         // searched: no codeword among the TEPs of the first w0 weights
         const uint32_t done = g_esp.cum[__popc(one)][__popc(both)][min(a.w0, Sp) + 1];
-        evaluated = !a.solve ? (unsigned long long)total : (solvable ? 1ull << d : 0ull);
+        evaluated = !a.solve ? (unsigned long long)total : (solvable && x != kCut ? 1ull << d : 0ull);
         if (!a.solve && qn > done) {
           hard = 1;
           useful = qn - done;

@@ -45,6 +45,8 @@ struct DecodeArgs {
   uint32_t* queries;
   uint8_t* abandon;
   Scratch* scr;                  // statistics, or NULL
+  unsigned long long* t0;        // the call's clock start (deadline), or NULL
+  long long deadline;            // grand_params.deadline_ns of a linear solve (0: none)
   CodeDev code[kInlineCodes];    // uniform batch: [0]
 };
 
