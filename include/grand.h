@@ -443,17 +443,23 @@ int grand_plan_destroy(grand_plan* plan);
  * TEPs and table slices share an SM). Times every candidate `tiles` setting (preparation
  * weights, search register budget, and for S' > 10 the warps per CTA) on the
  * given sample with CUDA events (median of 3 runs after one untimed run) and
- * writes the fastest into params->tiles. With params->membership =
+ * writes the fastest into params->tiles. With AUTO the shapes are timed in the
+ * TEP search, which calls with a deadline, weight windows and the serving
+ * loop's continued frames run (no frame of the sample is cut, whatever
+ * params->deadline_ns); without a deadline the warps per CTA stay automatic,
+ * so that the call keeps the one-kernel decode. With params->membership =
  * GRAND_MEMBERSHIP_FASTEST the candidates also span the membership test (the
- * TEP-by-TEP split search and the hash join, with the hash join's own launch
+ * call as AUTO runs it and the hash join, with the hash join's own launch
  * shapes) and the chosen one is written into params->membership. Results
  * never depend on the choice.
  *   cache_path  host path of a text cache (NULL: no cache). Lines are
  *               "key t0 t1 t2 t3 ms membership"; the key holds the GPU name
  *               and the workload (N, K, M, S, cap, likelihood variant, the
- *               membership asked for; the codes of a mixed batch). A cached
- *               key is used without timing.
- *   out         host, may be NULL: best time, candidates tried, cache hit,
+ *               membership asked for, deadline or none; the codes of a mixed
+ *               batch) and the cache's version. A cached key is used without
+ *               timing.
+ *   out         host, may be NULL: best time (of the call; with AUTO and a
+ *               deadline, of its search in full), candidates tried, cache hit,
  *               the membership test chosen.
  * The sample buffers are device memory; the tuner allocates its own outputs
  * (cudaMalloc) and synchronises `stream`. Errors: as the decode calls. */

@@ -2,7 +2,16 @@
 // GRAND_MEMBERSHIP_FASTEST, the two exact membership tests) on a sample batch
 // with CUDA events and keeps the fastest; results do not depend on the
 // choice, only the time does. Choices are cached in a text file keyed by the
-// GPU name and the workload (code sizes, constellation, cut-off, cap).
+// GPU name and the workload (code sizes, constellation, cut-off, cap, with or
+// without a deadline).
+//
+// What is timed is what the tiles are used for. Calls with a deadline search
+// TEP by TEP, and every shape of that search is a candidate. Calls without one
+// are decided by one kernel that reads no tiles, as long as warps and split
+// stay automatic: those shapes alone are candidates, timed in the search (the
+// serving loop's continued frames and weight windows read them), and the call
+// itself is timed against the hash join. (Timed in the call, nine shapes of
+// one kernel that ignores them made the choice noise.)
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -45,19 +54,8 @@ void shapes(int S, int membership, std::vector<Candidate>& out) {
   }
 }
 
-// The candidates: the launch shapes of the params' membership test, or with
-// GRAND_MEMBERSHIP_FASTEST those of both exact tests (the TEP-by-TEP split
-// search and the hash join), whose outputs are identical.
-std::vector<Candidate> candidates(int S, int membership) {
-  std::vector<Candidate> out;
-  if (membership == GRAND_MEMBERSHIP_FASTEST) {
-    shapes(S, GRAND_MEMBERSHIP_AUTO, out);
-    shapes(S, GRAND_MEMBERSHIP_HASH, out);
-  } else {
-    shapes(S, membership, out);
-  }
-  return out;
-}
+// A budget that no call reaches: it selects the search and cuts nothing.
+constexpr int64_t kAmpleNs = 3600ll * 1000000000ll;
 
 std::string device_name() {
   int dev = 0;
@@ -68,6 +66,11 @@ std::string device_name() {
     if (c == ' ' || c == '|') c = '_';
   return n;
 }
+
+// End of a cache key: whether the call has a deadline, and the version of what
+// is timed (lines of earlier versions name shapes that take the call away from
+// the kernel it runs by default, and are not used).
+const char* key_end(const grand_params* p) { return p->deadline_ns > 0 ? "|dl=1|v=2" : "|dl=0|v=2"; }
 
 // Cache lines: "key t0 t1 t2 t3 ms membership" (lines without the membership
 // field keep the params' membership).
@@ -144,18 +147,40 @@ int tune(const std::string& key, grand_params* p, const char* cache_path, cudaSt
   float best = 1e30f;
   Candidate best_c{{0, 0, 0, 0}, p->membership};
   int tried = 0;
-  for (const Candidate& c : candidates(p->S, p->membership)) {
+  auto time_one = [&](const Candidate& c, int64_t deadline, float* ms) {
     grand_params q = *p;
     for (int i = 0; i < 4; ++i) q.tiles[i] = c.tiles[i];
     q.membership = c.membership;
-    q.deadline_ns = 0;  // time every candidate in full
-    float ms = 0;
-    const int rc = time_runs([&](cudaStream_t s) { return run(&q, s); }, st, 3, &ms);
-    if (rc != GRAND_OK) return rc;
-    ++tried;
+    q.deadline_ns = deadline;
+    return time_runs([&](cudaStream_t s) { return run(&q, s); }, st, 3, ms);
+  };
+  // the exact tests asked for (FASTEST: the call's own and the hash join, whose
+  // outputs are identical)
+  for (const int membership : {GRAND_MEMBERSHIP_AUTO, GRAND_MEMBERSHIP_HASH}) {
+    if (p->membership != GRAND_MEMBERSHIP_FASTEST && p->membership != membership) continue;
+    const bool one_kernel = membership == GRAND_MEMBERSHIP_AUTO && p->deadline_ns == 0;
+    std::vector<Candidate> all;
+    shapes(p->S, membership, all);
+    float ms = 1e30f;
+    Candidate fastest{};
+    for (const Candidate& c : all) {
+      if (one_kernel && (c.tiles[0] || c.tiles[1])) continue;
+      float t = 0;
+      const int rc = time_one(c, membership == GRAND_MEMBERSHIP_AUTO ? kAmpleNs : 0, &t);
+      if (rc != GRAND_OK) return rc;
+      ++tried;
+      if (t < ms) {
+        ms = t;
+        fastest = c;
+      }
+    }
+    if (one_kernel) {
+      const int rc = time_one(fastest, 0, &ms);
+      if (rc != GRAND_OK) return rc;
+    }
     if (ms < best) {
       best = ms;
-      best_c = c;
+      best_c = fastest;
     }
   }
   for (int i = 0; i < 4; ++i) p->tiles[i] = best_c.tiles[i];
@@ -191,8 +216,8 @@ extern "C" int grand_autotune(const grand_code* c, grand_params* p, const void* 
     return GRAND_E_NOMEM;
   }
   char key[384];
-  snprintf(key, sizeof key, "%s|sym|N=%d|K=%d|M=%d|S=%d|cap=%lld|lik=%d|ord=%d|mem=%d", device_name().c_str(), N,
-           c->K, p->M, p->S, (long long)p->query_cap, p->lik_variant, p->order, p->membership);
+  snprintf(key, sizeof key, "%s|sym|N=%d|K=%d|M=%d|S=%d|cap=%lld|lik=%d|ord=%d|mem=%d%s", device_name().c_str(), N,
+           c->K, p->M, p->S, (long long)p->query_cap, p->lik_variant, p->order, p->membership, key_end(p));
   const int rc = tune(
       key, p, cache_path, st,
       [&](const grand_params* pp, cudaStream_t s) {
@@ -235,7 +260,7 @@ extern "C" int grand_autotune_mixed(const grand_code* const* codes, int n_codes,
   }
   key += "|S=" + std::to_string(p->S) + "|cap=" + std::to_string((long long)p->query_cap) +
          "|lik=" + std::to_string(p->lik_variant) + "|ord=" + std::to_string(p->order) +
-         "|mem=" + std::to_string(p->membership);
+         "|mem=" + std::to_string(p->membership) + key_end(p);
   const int rc = tune(
       key, p, cache_path, st,
       [&](const grand_params* pp, cudaStream_t s) {
