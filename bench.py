@@ -81,6 +81,12 @@ CONFIGS = {
                        "400000 requests; long frames whole in their batch vs carried as device-resident cursors"),
 }
 METRIC = "TEP syndrome checks/s & frames/s per GB300; p50/p99 decode latency"
+# A deadline that no call reaches. The default call is decided by one kernel
+# that tests no TEP; a call with a deadline runs the TEP search, whose checks
+# are what checks/s counts.
+SEARCH_NS = 3600 * 10 ** 9
+# The printed line has to be readable from the last 3 KB of a run's output.
+LINE_BYTES = 2600
 CONFIG_IDS = {"c1": 1, "c2": 2, "c3a": 3, "c3b": 4, "c4": 5, "c5": 6, "c5adv": 8, "c5long": 9, "bler": 7, "orders": 2,
               "membership": 2}
 # ALU roofline: 152 SMs x 64 integer-ALU lanes per clock (LOP3/ISETP class)
@@ -693,7 +699,7 @@ def run_membership(args, cfg, g):
                       ("per-TEP syndrome deltas", g.MEMBERSHIP_DELTA),
                       ("per-TEP row parity (Alg. 1 product)", g.MEMBERSHIP_ROW_PARITY),
                       ("hash join of the split (decision, no per-TEP test)", g.MEMBERSHIP_HASH)):
-        p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], membership=mem)
+        p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], membership=mem, deadline_ns=SEARCH_NS)
         _timed_decode(g, code, p, sym[:2000])
         r, secs = _timed_decode(g, code, p, sym)
         q = r["queries"].cpu().numpy().view(np.uint32).astype(np.int64)
@@ -706,12 +712,14 @@ def run_membership(args, cfg, g):
                      "evaluated_checks": int(r["evaluated_checks"]),
                      "evaluated_checks_per_s": r["evaluated_checks"] / (kern_ms / 1e3),
                      "results_equal_split_search": bool(same)})
-    # the default workload's whole batch (300,000 frames): split search against the hash join
+    # the default workload's whole batch (300,000 frames): split search against the hash join, and the
+    # default call (one kernel, the linear system), which tests no TEP
     full = dict(cfg, frames=100000)
     code2, sym2, _ = _c2_like_batch(full, g)
     base = None
-    for name, mem in (("split search (default)", g.MEMBERSHIP_AUTO), ("hash join", g.MEMBERSHIP_HASH)):
-        p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], membership=mem)
+    for name, mem, ns in (("split search", g.MEMBERSHIP_AUTO, SEARCH_NS), ("hash join", g.MEMBERSHIP_HASH, 0),
+                          ("default call (linear system)", g.MEMBERSHIP_AUTO, 0)):
+        p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], membership=mem, deadline_ns=ns)
         _timed_decode(g, code2, p, sym2)
         ms = []
         for _ in range(5):
@@ -723,8 +731,9 @@ def run_membership(args, cfg, g):
         base = base or out
         rows.append({"membership": name + ", 300,000-frame batch", "kernel_ms": statistics.median(ms),
                      "search_ms": float(r["search_ms"]), "frames_per_s": len(q) / (statistics.median(ms) / 1e3),
-                     "useful_checks_per_s": float(q.sum()) / (statistics.median(ms) / 1e3),
-                     "evaluated_checks": int(r["evaluated_checks"]), "results_equal_split_search": bool(same)})
+                     "useful_checks_per_s": float(q.sum()) / (statistics.median(ms) / 1e3) if mem or ns else None,
+                     "evaluated_checks": int(r["evaluated_checks"]) if mem or ns else None,
+                     "results_equal_split_search": bool(same)})
     code2.close()
     code.close()
     return rows
@@ -756,7 +765,9 @@ def run_config(args, cfg, g, ctx):
         d_desc = torch.from_numpy(desc.view(np.uint8)).to(dev)
         n_frames = len(inputs["N"])
         n_cw = inputs["n_cw_words"]
-        p = g.Params.make(M=0, S=cfg["S"], query_cap=cfg["cap"], tiles=tiles, membership=membership)
+        p = g.Params.make(M=0, S=cfg["S"], query_cap=cfg["cap"], tiles=tiles, membership=membership,
+                          deadline_ns=SEARCH_NS)
+        p_call = g.Params.make(M=0, S=cfg["S"], query_cap=cfg["cap"])
         alg_words = None
     else:
         codes = [g.Code.polar(cfg["N"], cfg["K"])]
@@ -765,7 +776,9 @@ def run_config(args, cfg, g, ctx):
         if cfg["kind"] == "ab":
             p = g.Params.make(order=g.ORDER_HAMMING, M=2, max_weight=cfg["max_weight"], query_cap=cfg["cap"])
         else:
-            p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], tiles=tiles, membership=membership)
+            p = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"], tiles=tiles, membership=membership,
+                              deadline_ns=SEARCH_NS)
+            p_call = g.Params.make(M=cfg["M"], S=cfg["S"], query_cap=cfg["cap"])
         alg_words = (cfg["N"] - cfg["K"]) / 32.0
     h_sym = torch.from_numpy(inputs["symbols"]).pin_memory()
     d_sym = h_sym.to(dev)
@@ -906,11 +919,51 @@ def run_config(args, cfg, g, ctx):
                  "timing": "CUDA events around 8 calls back to back on 4 rotating copies of the batch (each "
                            "call's symbols evicted from L2 by the others); per-call mean"}
 
-    # ---- the fastest exact decode of the same batch: the autotuner chooses
-    #      between the TEP-by-TEP split search and the hash join of the split
-    #      (GRAND_MEMBERSHIP_FASTEST; identical outputs) and their launch
-    #      shapes; frames/s and latency on the chosen path (a CUDA-graph plan
-    #      for the uneven batch), reported beside the checks/s headline
+    # ---- the default call on the same batch: one kernel that solves each
+    #      frame's linear system (no TEP is tested, so frames/s), as the
+    #      headline is timed: one CUDA-graph replay per step; end to end from
+    #      page-locked host memory below
+    default_call = None
+    if cfg["kind"] in ("qam", "mixed") and args.membership == "auto":
+        ref_out = (d_cw.clone(), d_q.clone(), d_ab.clone())
+        if cfg["kind"] == "mixed":
+            cplan = g.plan_mixed(codes, p_call, d_desc, d_sym, d_cw, d_q, d_ab)
+        else:
+            cplan = g.plan_symbols(codes[0], p_call, d_sym, d_cw.view(n_frames, -1), d_q, d_ab)
+        for _ in range(args.warmup):
+            cplan.launch()
+        c_ms = []
+        for _ in range(args.steps):
+            flush.zero_()
+            e0 = torch.cuda.Event(enable_timing=True)
+            e1 = torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            cplan.launch()
+            e1.record(stream)
+            e1.synchronize()
+            c_ms.append(e0.elapsed_time(e1))
+        same = all(torch.equal(x, y) for x, y in zip((d_cw, d_q, d_ab), ref_out))
+        cplan.close()
+        # its unit is the data it cannot do without
+        call_bytes = d_sym.numel() * d_sym.element_size() + 5 * n_frames + 4 * d_cw.numel()
+        if cfg["kind"] == "mixed":
+            call_bytes += d_desc.numel()
+        peak, peak_source = hbm_peak()
+        t_ms = statistics.mean(c_ms)
+        default_call = {"what": "one kernel, the frame's linear system (no TEP is tested)", "ms_per_step": t_ms,
+                        "frames_per_s": n_frames / (t_ms / 1e3),
+                        "latency_ms": {"p50": float(np.percentile(c_ms, 50)), "p99": float(np.percentile(c_ms, 99))},
+                        "outputs_equal": bool(same),
+                        "roofline": {"bound": "hbm", "kernel": "k_decode", "kernel_ms": t_ms, "peak": peak,
+                                     "unit": "GB/s", "peak_source": peak_source,
+                                     "achieved": call_bytes / t_ms / 1e6, "frac": call_bytes / t_ms / 1e6 / peak,
+                                     "algorithmic_bytes": int(call_bytes), "traffic": None,
+                                     "note": "issue-bound in ncu", "profile": "profiles/k_decode_thread.md"}}
+
+    # ---- the autotuner's choice for the same batch: the default call or the
+    #      hash join of the split (GRAND_MEMBERSHIP_FASTEST; identical outputs);
+    #      frames/s and latency on the chosen path (a CUDA-graph plan for the
+    #      uneven batch), reported beside the checks/s headline
     fastest = None
     if cfg["kind"] in ("qam", "mixed") and args.membership == "auto":
         ref_out = (d_cw.clone(), d_q.clone(), d_ab.clone())
@@ -944,13 +997,13 @@ def run_config(args, cfg, g, ctx):
         same = all(torch.equal(x, y) for x, y in zip((d_cw, d_q, d_ab), ref_out))
         if fplan is not None:
             fplan.close()
-        fastest = {"membership": {0: "split search (TEP by TEP)", 3: "hash join"}.get(ftune["membership"]),
+        fastest = {"membership": {0: "default call (linear system)", 3: "hash join"}.get(ftune["membership"]),
                    "tiles": list(ftune["tiles"]), "ms_per_step": statistics.mean(f_ms),
                    "frames_per_s": n_frames / (statistics.mean(f_ms) / 1e3),
                    "latency_ms": {"p50": float(np.percentile(f_ms, 50)), "p99": float(np.percentile(f_ms, 99))},
                    "outputs_equal": bool(same), "graph": cfg["kind"] == "mixed",
-                   "what": "the autotuner's fastest exact membership test (GRAND_MEMBERSHIP_FASTEST) on the same "
-                           "batch: same outputs; a hash join decides the queries without testing them one by "
+                   "what": "the autotuner's choice between the default call and the hash join "
+                           "(GRAND_MEMBERSHIP_FASTEST) on the same batch: same outputs; neither tests TEPs one by "
                            "one, so this line reports frames/s, not checks"}
 
     # ---- the same batch through GRAND_MEMBERSHIP_SOLVE: the first hit by
@@ -1010,33 +1063,41 @@ def run_config(args, cfg, g, ctx):
     host_api = cfg["kind"] in ("qam", "ab", "mixed")
     if cfg["kind"] == "mixed":  # the descriptors are host input too, page-locked like the symbols
         h_desc = torch.from_numpy(desc.view(np.uint8)).pin_memory()
-    e2e_ms = []
-    for it in range(1 + max(2, min(args.steps, 5))):  # the first call is untimed (pool growth, streams)
-        flush.zero_()
-        e0 = torch.cuda.Event(enable_timing=True)
-        e1 = torch.cuda.Event(enable_timing=True)
-        e0.record(stream)
-        if host_api and cfg["kind"] == "mixed":
-            g.decode_mixed_host(codes, p, h_desc, h_sym, n_cw, cw=h_cw, queries=h_q, abandon=h_ab, stream=stream)
-        elif host_api:
-            g.decode_symbols_host(codes[0], p, h_sym, cw=h_cw, queries=h_q, abandon=h_ab, stream=stream)
-        else:
-            d_sym2.copy_(h_sym, non_blocking=True)
-            step(d_sym2, stats=False)
-            h_cw.copy_(d_cw, non_blocking=True)
-            h_q.copy_(d_q, non_blocking=True)
-            h_ab.copy_(d_ab, non_blocking=True)
-        e1.record(stream)
-        e1.synchronize()
-        if it:
-            e2e_ms.append(e0.elapsed_time(e1))
-    e2e_value = (useful_total / args.steps) / (statistics.mean(e2e_ms) / 1e3)
-    e2e_equal = bool(torch.equal(h_cw, d_cw.cpu()) and torch.equal(h_q, d_q.cpu()) and torch.equal(h_ab, d_ab.cpu()))
+
+    def time_e2e(pe):
+        ms = []
+        for it in range(1 + max(2, min(args.steps, 5))):  # the first call is untimed (pool growth, streams)
+            flush.zero_()
+            e0 = torch.cuda.Event(enable_timing=True)
+            e1 = torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            if host_api and cfg["kind"] == "mixed":
+                g.decode_mixed_host(codes, pe, h_desc, h_sym, n_cw, cw=h_cw, queries=h_q, abandon=h_ab, stream=stream)
+            elif host_api:
+                g.decode_symbols_host(codes[0], pe, h_sym, cw=h_cw, queries=h_q, abandon=h_ab, stream=stream)
+            else:
+                d_sym2.copy_(h_sym, non_blocking=True)
+                step(d_sym2, stats=False)
+                h_cw.copy_(d_cw, non_blocking=True)
+                h_q.copy_(d_q, non_blocking=True)
+                h_ab.copy_(d_ab, non_blocking=True)
+            e1.record(stream)
+            e1.synchronize()
+            if it:
+                ms.append(e0.elapsed_time(e1))
+        equal = bool(torch.equal(h_cw, d_cw.cpu()) and torch.equal(h_q, d_q.cpu()) and torch.equal(h_ab, d_ab.cpu()))
+        return statistics.mean(ms), equal
+
+    if default_call:
+        call_ms, call_equal = time_e2e(p_call)
+        default_call["e2e"] = {"value": n_frames / (call_ms / 1e3), "unit": "frames/s", "ms_per_step": call_ms,
+                               "outputs_equal_device": call_equal}
+    e2e_ms, e2e_equal = time_e2e(p)
+    e2e_value = (useful_total / args.steps) / (e2e_ms / 1e3)
 
     # ---- the plain one-frame-per-launch GPU path on a sample (same frames, same results)
     one = None
     if cfg["kind"] in ("qam", "mixed"):
-        # S' = 12 frames that abandon run 2^24 queries each in one warp: a smaller sample
         n_one = min(2000 if cfg.get("S", 10) <= 10 else 200, n_frames)
         idx = np.linspace(0, n_frames - 1, n_one).astype(np.int64)
         torch.cuda.synchronize()
@@ -1046,10 +1107,10 @@ def run_config(args, cfg, g, ctx):
         for f in idx.tolist():
             if cfg["kind"] == "mixed":
                 dsz = g.FRAME_DESC_DTYPE.itemsize
-                g.decode_mixed(codes, p, d_desc[f * dsz:(f + 1) * dsz], d_sym, n_cw, cw=d_cw, queries=d_q[f:f + 1],
+                g.decode_mixed(codes, p_call, d_desc[f * dsz:(f + 1) * dsz], d_sym, n_cw, cw=d_cw, queries=d_q[f:f + 1],
                                abandon=d_ab[f:f + 1])
             else:
-                g.decode_symbols(codes[0], p, d_sym[f:f + 1], cw=d_cw.view(n_frames, -1)[f:f + 1],
+                g.decode_symbols(codes[0], p_call, d_sym[f:f + 1], cw=d_cw.view(n_frames, -1)[f:f + 1],
                                  queries=d_q[f:f + 1], abandon=d_ab[f:f + 1])
         e1.record(stream)
         e1.synchronize()
@@ -1059,21 +1120,7 @@ def run_config(args, cfg, g, ctx):
 
     # ---- roofline of the dominant kernel (the TEP search)
     roofline = None
-    if cfg["kind"] in ("qam", "mixed") and args.membership == "auto" and not any(p.tiles[:2]):
-        # automatic tiles: one kernel decides all TEPs of a frame at once, so
-        # its unit is the data it cannot do without
-        alg_bytes = d_sym.numel() * d_sym.element_size() + 5 * n_frames + 4 * d_cw.numel()
-        if cfg["kind"] == "mixed":
-            alg_bytes += d_desc.numel()
-        peak, peak_source = hbm_peak()
-        t_ms = statistics.mean(step_ms)
-        roofline = {"bound": "hbm", "kernel": "k_decode", "kernel_ms": t_ms, "peak": peak, "unit": "GB/s",
-                    "peak_source": peak_source, "achieved": alg_bytes / t_ms / 1e6,
-                    "frac": alg_bytes / t_ms / 1e6 / peak, "algorithmic_bytes": int(alg_bytes), "traffic": None,
-                    "note": "first hit from the frame's GF(2) system: useful checks are the positions of the first "
-                            "hits (or the cap), none is tested by itself; issue-bound in ncu",
-                    "profile": "profiles/k_decode_thread.md"}
-    elif sum(search_ms) > 0 and args.membership == "auto":  # TEPs tested one by one
+    if sum(search_ms) > 0 and args.membership == "auto":  # TEPs tested one by one
         roofline = search_roofline(cfg, evaluated / args.steps, search_useful / args.steps, hard / args.steps,
                                    statistics.mean(search_ms), alg_words, frames=n_frames)
 
@@ -1110,7 +1157,8 @@ def run_config(args, cfg, g, ctx):
             "data": "synthetic (seeded random polar codewords over AWGN)",
             "config": {"workload": cfg["desc"], "frames_per_step_per_gpu": n_frames, "tiles": list(p.tiles),
                        "l2": "flushed before every timed step (256 MiB write)",
-                       "membership": args.membership,
+                       "membership": "TEP search (a deadline that nothing reaches)" if args.membership == "auto"
+                                     and cfg["kind"] != "ab" else args.membership,
                        "parallelism": f"frames sharded, {world} replica(s)"},
             "frames_per_s": frames_per_s,
             "latency_ms": {"p50": float(np.percentile(step_ms, 50)), "p99": float(np.percentile(step_ms, 99)),
@@ -1122,6 +1170,7 @@ def run_config(args, cfg, g, ctx):
             "kernel_ms": ({"prep": statistics.mean(prep_ms), "search": statistics.mean(search_ms)} if search_ms
                           else None),
             "roofline": roofline,
+            "default_call": default_call,
             "fastest_exact": fastest,
             "solve": solve,
             "demod": demod,
@@ -1129,7 +1178,7 @@ def run_config(args, cfg, g, ctx):
             "autotune": tune,
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "checks/s", "h2d_bytes_per_step": int(h_sym.numel() * h_sym.element_size()),
-                    "d2h_bytes_per_step": int(n_cw * 4 + n_frames * 5), "ms_per_step": statistics.mean(e2e_ms),
+                    "d2h_bytes_per_step": int(n_cw * 4 + n_frames * 5), "ms_per_step": e2e_ms,
                     "api": ("grand_decode_mixed_host" if cfg["kind"] == "mixed" else "grand_decode_symbols_host")
                            + " (chunks on two streams, copies overlapped with decoding)",
                     "outputs_equal_device": e2e_equal},
@@ -1177,6 +1226,51 @@ def run_serve_config(args, cfg, g, ctx):
     return line
 
 
+def short(v):
+    """Numbers to six figures, in records of any depth."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: short(x) for k, x in v.items()}
+    return [short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def short_line(line):
+    """The record's main figures in at most LINE_BYTES: the headline's keys and one entry for each other workload,
+    entries that do not fit left out from the last on."""
+    def some(rec, *keys):
+        return {k: rec[k] for k in keys if k in rec} if rec else None
+
+    out = some(line, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+               "vs_baseline", "dtype", "data", "config", "frames_per_s", "bler", "gpu_launches", "clocks")
+    out["latency_ms"] = some(line["latency_ms"], "p50", "p99")
+    out["e2e"] = some(line["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step")
+    out["roofline"] = some(line.get("roofline"), "bound", "kernel", "kernel_ms", "peak", "unit", "achieved", "frac")
+    call = some(line.get("default_call"), "ms_per_step", "frames_per_s", "outputs_equal", "roofline", "e2e")
+    if call:
+        call["roofline"] = some(call["roofline"], "bound", "achieved", "frac")
+        call["e2e"] = some(call["e2e"], "value", "unit")
+    out["default_call"] = call
+    out["demod"] = some(line.get("demod"), "ms", "frac")
+    cpu = some(line.get("cpu_baseline"), "value", "unit", "cores", "kind", "frames_per_s")
+    out["cpu_baseline"] = cpu
+    out = short(out)
+    out["configs"] = {}
+    for name, rec in line.get("configs", {}).items():
+        entry = some(rec, "value", "unit", "ms_per_step", "frames_per_s")
+        if rec.get("latency_us"):
+            entry["latency_us"] = some(rec["latency_us"], "p50", "p99")
+        if rec.get("default_call"):
+            entry["default_call"] = some(rec["default_call"], "ms_per_step", "frames_per_s")
+        out["configs"][name] = short(entry)
+    while len(json.dumps(out)) > LINE_BYTES and out["configs"]:
+        out["configs"].popitem()
+    for key in ("cpu_baseline", "demod", "default_call", "roofline"):
+        if len(json.dumps(out)) > LINE_BYTES:
+            out.pop(key)
+    return out
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1193,8 +1287,11 @@ def main():
     ap.add_argument("--frames", type=int, default=0, help="override frames per SNR (for quick runs)")
     ap.add_argument("--tiles", default="0,0,0,0", help="launch shape (grand_params.tiles), 0 = automatic")
     ap.add_argument("--membership", default="auto", choices=("auto", "hash", "solve"),
-                    help="membership test of the search (the headline uses the TEP-by-TEP search; "
-                         "solve: serving configs only -- the other records carry it under 'solve')")
+                    help="auto: the headline is the TEP-by-TEP search, selected by a deadline that nothing reaches "
+                         "(the default call tests no TEP and stands under 'default_call'); hash: the hash join; "
+                         "solve: serving configs only -- the other records carry it under 'solve'")
+    ap.add_argument("--record", default=None, help="file for the whole record of the run (the printed line holds its "
+                                                   "main figures)")
     ap.add_argument("--serve-batch", type=int, default=65536, help="serving: frames per launch")
     ap.add_argument("--serve-streams", type=int, default=4, help="serving: batches in flight")
     ap.add_argument("--serve-resume-step", type=int, default=0,
@@ -1286,7 +1383,10 @@ def main():
         if line is not None:
             line["configs"] = subs
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.record:
+            with open(args.record, "w") as fh:
+                json.dump(line, fh)
+        print(json.dumps(short_line(line)), flush=True)
     if dist:
         dist.destroy_process_group()
     return 0
