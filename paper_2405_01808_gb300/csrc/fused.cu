@@ -150,21 +150,49 @@ __device__ __forceinline__ uint32_t pack_plan(int m, int lane) {
   return (1u << 12) | ((uint32_t)lane << 13);
 }
 
-// Exact selection of the S' smallest (key, index) pairs, S' scans of the
-// frame: for the rare frame whose packed keys do not settle it (a selected
-// key saturates, or one lane of a long frame ran out of kept keys). Lane r
-// returns the index of rank r.
+// Exact selection of the S' smallest (key, index) pairs, for frames whose
+// packed keys do not settle it (a selected key saturates: a receiver whose gain
+// is many times the constellation's, or one lane of a long frame ran out of
+// kept keys). Lane r returns the index of rank r. One pass with whole keys,
+// each lane keeping its kLanePick smallest; a scan for every rank left when a
+// lane runs out of them. (Scans for all ranks computed every key S' times:
+// 18,000 frames of 512 symbols, 60 times too large, 581 us, so 212.)
 template <int kFrom>
 __device__ __noinline__ int select_exact(const DecodeArgs& a, int64_t base, int L, int Sp, int m) {
   const int lane = threadIdx.x & 31;
+  auto key_of = [&](int i) {
+    if constexpr (kFrom == kFromArrays) return selection_key(a.key[base + i]);
+    else return symbol_key(a.symbols[base + i], a.ax[m].q.x, m, a.lik);
+  };
+  typedef unsigned long long Kept;  // key, index (9 bits)
+  constexpr Kept kEmpty = ~0ull;
+  Kept b0 = kEmpty, b1 = kEmpty, b2 = kEmpty, b3 = kEmpty;  // ascending
+  static_assert(kLanePick == 4, "kept keys");
+  for (int i = lane; i < L; i += 32) {
+    Kept t = ((Kept)key_of(i) << 9) | (Kept)i, u;
+    u = max(b0, t); b0 = min(b0, t);
+    t = max(b1, u); b1 = min(b1, u);
+    u = max(b2, t); b2 = min(b2, t);
+    b3 = min(b3, u);
+  }
   uint32_t last_k = 0;
-  int last_i = -1, sel = 0;
-  for (int r = 0; r < Sp; ++r) {
+  int last_i = -1, sel = 0, r = 0;
+  for (bool out = false; r < Sp && !out; ++r) {
+    const uint32_t hi = (uint32_t)(b0 >> 32), hmin = __reduce_min_sync(kAll, hi);
+    const uint32_t lo = hi == hmin ? (uint32_t)b0 : kNone, lmin = __reduce_min_sync(kAll, lo);
+    if (hi == hmin && lo == lmin) {
+      b0 = b1; b1 = b2; b2 = b3; b3 = kEmpty;
+    }
+    const Kept best = ((Kept)hmin << 32) | lmin;
+    last_k = (uint32_t)(best >> 9);
+    last_i = (int)(best & 511u);
+    if (lane == r) sel = last_i;
+    out = __any_sync(kAll, b0 == kEmpty && L > 32 * kLanePick + lane);
+  }
+  for (; r < Sp; ++r) {
     uint32_t bk = kNone, bi = kNone;
     for (int i = lane; i < L; i += 32) {
-      uint32_t k;
-      if constexpr (kFrom == kFromArrays) k = selection_key(a.key[base + i]);
-      else k = symbol_key(a.symbols[base + i], a.ax[m].q.x, m, a.lik);
+      const uint32_t k = key_of(i);
       const bool after = k > last_k || (k == last_k && i > last_i);
       if (after && k < bk) { bk = k; bi = (uint32_t)i; }
     }
