@@ -605,6 +605,62 @@ __device__ __forceinline__ void merge_smallest(uint32_t (&best)[R], const uint32
       if (!(i & dist)) order2(best[o + i], best[o + i + dist]);
 }
 
+// Base syndrome of one frame for H not of polar form, by one warp: the sum of
+// the columns of its hard word's one-bits (lane w holds word w), four words of
+// every column in one load and four columns a lane in flight. Word v goes to
+// out[v * stride]; returns the projection. (A word of a column at a time waited
+// for each of 16 x 32 scattered loads: 30,000 demodulated frames of 1024 bits and
+// 512 rows, cap 30, 334 us, so 162.)
+__device__ __noinline__ uint32_t column_syndrome(const uint32_t* __restrict__ hcol, const uint32_t* __restrict__ hf,
+                                                 int W, int NW, uint32_t yw, uint32_t* out, int stride) {
+  constexpr int kCols = 4, kWords = 4;
+  const int lane = threadIdx.x & 31;
+  uint32_t f0 = 0;
+  for (int v0 = 0; v0 < W; v0 += kWords) {
+    uint32_t acc[kWords] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+    for (int w0 = 0; w0 < NW; w0 += kCols) {
+      uint4 c[kCols];
+      uint32_t f[kCols];
+#pragma unroll
+      for (int i = 0; i < kCols; ++i) {
+        const int w = w0 + i;  // (words beyond the last are zero in yw)
+        const bool on = (__shfl_sync(kAll, yw, w & 31) >> lane) & 1u;
+        c[i] = make_uint4(0u, 0u, 0u, 0u);
+        f[i] = 0u;
+        if (on) {
+          const uint32_t* p = hcol + (size_t)(32 * w + lane) * W + v0;
+          if (!(W & 3)) {  // columns start on 16 bytes
+            c[i] = __ldg(reinterpret_cast<const uint4*>(p));
+          } else {
+            c[i].x = __ldg(p);
+            if (v0 + 1 < W) c[i].y = __ldg(p + 1);
+            if (v0 + 2 < W) c[i].z = __ldg(p + 2);
+            if (v0 + 3 < W) c[i].w = __ldg(p + 3);
+          }
+          if (v0 == 0 && W > 1) f[i] = __ldg(hf + 32 * w + lane);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kCols; ++i) {
+        acc[0] ^= c[i].x;
+        acc[1] ^= c[i].y;
+        acc[2] ^= c[i].z;
+        acc[3] ^= c[i].w;
+        f0 ^= f[i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kWords; ++i) {
+      if (v0 + i >= W) break;
+      const uint32_t s = __reduce_xor_sync(kAll, acc[i]);
+      if (lane == 0) out[(v0 + i) * stride] = s;
+      if (W == 1) return s;  // one word: the syndrome itself
+    }
+  }
+  return __reduce_xor_sync(kAll, f0);
+}
+
 // Natural labels of four symbols (m bits an axis, I then Q, the first symbol
 // highest) to Gray labels.
 template <typename T>
@@ -876,22 +932,11 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     __syncwarp();
     uint32_t* y = buf + fr;
     const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
-    const int W = code->W;
     const uint32_t yw = lane < NW ? __brev(y[lane * stride]) : 0u;
     const int64_t co = kFrom == kFromMixed ? s_cw[fr] : (tile + fr) * (int64_t)NW;
     if (lane < NW) a.cw[co + lane] = yw;
-    uint32_t f0 = 0;
-    for (int w = 0; w < NW; ++w)
-      if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) f0 ^= __ldg(code->hf + 32 * w + lane);
-    f0 = __reduce_xor_sync(kAll, f0);
-    for (int v = 0; v < W; ++v) {
-      uint32_t acc = 0;
-      for (int w = 0; w < NW; ++w)
-        if ((__shfl_sync(kAll, yw, w) >> lane) & 1u) acc ^= __ldg(code->hcol + (size_t)(32 * w + lane) * W + v);
-      acc = __reduce_xor_sync(kAll, acc);
-      if (lane == 0) y[v * stride] = acc;  // the hard word is no longer needed here
-      if (W == 1) f0 = acc;
-    }
+    __syncwarp();  // the hard word makes place for the syndrome
+    const uint32_t f0 = column_syndrome(code->hcol, code->hf, code->W, NW, yw, y, stride);
     if (lane == 0) s_f0[fr] = f0;
   };
 
