@@ -187,9 +187,8 @@ typedef enum grand_lik {
  *               search it: the frame gets abandon = 5, cw = the hard word and
  *               queries = the number of leading valid TEPs already tested
  *               without a hit (those of the preparation stage; SOLVE: those
- *               of at most one altered symbol where H has at most 32 rows,
- *               else 0; 0 for HAMMING, QAM_NNE5 and the DELTA / ROW_PARITY
- *               tests), and the
+ *               of at most one altered symbol; 0 for HAMMING, QAM_NNE5 and
+ *               the DELTA / ROW_PARITY tests), and the
  *               code's status word is set for grand_stream_status. A frame
  *               whose search has started finishes (at most one frame's search
  *               per warp beyond the budget); frames the preparation resolves

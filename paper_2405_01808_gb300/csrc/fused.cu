@@ -53,6 +53,8 @@ constexpr uint32_t kOff = 0xFFFFFE00u;     // above every packed key: lane (low 
 constexpr uint32_t kPicked = 0xFFFFFFE0u;  // above those: a key taken as rank (low bits)
 constexpr int kLanePick = 4;            // smallest keys kept per lane of a long frame
 constexpr int kOwnDim = 3;              // kernels of up to this dimension are walked by the frame's thread
+constexpr int kPairDim = 10;            // of larger ones, TEPs of two altered ranks are tested before any walk
+constexpr int kPairTeps = 631;          // and where the query cap may lie among those (at most as many)
 constexpr int kCutDim = 8;              // frames of larger kernels are cut at the call's deadline
 constexpr uint32_t kCut = 0xFFFFFFFEu;  // in the place of a solution: cut at the deadline
 
@@ -233,24 +235,26 @@ struct Frame {
   const uint32_t* pat;  // shared: subset_pattern of 0..31
   int nw;               // syndrome words in buf
   int polar;
+  const float2* cols;   // rank r: its slots' projections (as bits) at cols[32 r]; NULL: read from the table
 };
 
 __device__ __forceinline__ uint32_t slot_pos(const Frame& f, int b) {
   return (f.pos[(b >> 1) * f.pstride] >> (16 * (b & 1))) & 0xFFFFu;
 }
 
-// Word w of slot b's syndrome change.
-__device__ __forceinline__ uint32_t column_word(const Frame& f, uint32_t p, int w) {
-  if (p == kNoPos) return 0u;
-  if (f.polar) return ((uint32_t)w & ~(p >> 5)) ? 0u : f.pat[p & 31u] & __ldg(f.fmask + w);
-  return __ldg(f.hcol + (size_t)p * f.W + w);
-}
-
 // XOR of the slot columns over x (and the base syndrome) is zero everywhere.
+// Without the base the packed columns are summed, which are fewer words than
+// the transform's for polar-form H (2 instead of 32 at 1024 bits and 40 rows).
 __device__ __noinline__ bool sum_zero(const Frame f, uint32_t x, bool base) {
-  for (int w = 0; w < f.nw; ++w) {
+  const bool packed = !base || !f.polar;
+  for (int w = 0; w < (packed ? f.W : f.nw); ++w) {
     uint32_t acc = base ? f.buf[w * f.stride] : 0u;
-    for (uint32_t t = x; t; t &= t - 1u) acc ^= column_word(f, slot_pos(f, __ffs(t) - 1), w);
+    for (uint32_t t = x; t; t &= t - 1u) {
+      const uint32_t p = slot_pos(f, __ffs(t) - 1);
+      if (p == kNoPos) continue;
+      if (packed) acc ^= __ldg(f.hcol + (size_t)p * f.W + w);
+      else if (!((uint32_t)w & ~(p >> 5))) acc ^= f.pat[p & 31u] & __ldg(f.fmask + w);
+    }
     if (acc) return false;
   }
   return true;
@@ -357,50 +361,104 @@ __device__ __forceinline__ uint32_t valid_up_to(uint32_t ex, int Sp, int w) {
   return g_esp.cum[__popc(h ^ v)][__popc(h & v)][min(w, Sp) + 1];
 }
 
-// First TEP of weight <= wmax (at most 3) in canonical order whose projection
-// equals f0 and which passes the full test, or kNone: by one warp, 32 TEPs of
-// the order at a time (all arguments the same in every lane). A weight's TEPs
-// are numbered by their rank set in colex order, then by their alternatives.
-__device__ __noinline__ uint32_t light_hit_warp(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
-                                                bool exact, int wmax) {
-  const int lane = threadIdx.x & 31;
-  uint32_t dl[3 * kSMax];
+// First TEP of weight <= wmax (at most 2) in canonical order whose projection
+// equals f0 and which passes the full test, or kNone: by the frame's thread. A
+// warp instruction compares a pair of alternatives of 32 frames; by the warp,
+// one frame after the other, the pairs waited for each other: 18,000 frames of
+// 1024 bits with 10 parity bits, S = 12 and a cap of 300 352 us, so 63. The
+// projections are read where the elimination's were put (local arrays would be
+// read from L2, as shared memory leaves the first level little room).
+__device__ __noinline__ uint32_t light_hit(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0, bool exact,
+                                           int wmax, int64_t cap) {
+  auto full = [&](uint32_t x) { return exact || sum_zero(f, x, true); };
+  auto columns = [&](int r, uint32_t& a, uint32_t& b) {
+    if (f.cols) {
+      const float2 v = f.cols[32 * r];
+      a = __float_as_uint(v.x);
+      b = __float_as_uint(v.y);
+    } else {
+      a = proj(slot_pos(f, 2 * r));
+      b = proj(slot_pos(f, 2 * r + 1));
+    }
+  };
+  if (f0 == 0u && full(0u)) return 0u;
   for (int r = 0; r < Sp; ++r) {
-    dl[3 * r] = proj(slot_pos(f, 2 * r));
-    dl[3 * r + 1] = proj(slot_pos(f, 2 * r + 1));
-    dl[3 * r + 2] = dl[3 * r] ^ dl[3 * r + 1];
+    uint32_t a, b;
+    columns(r, a, b);
+    const uint32_t e = (ex >> (2 * r)) & 3u;
+    if ((e & 1u) && a == f0 && full(1u << (2 * r))) return 1u << (2 * r);
+    if ((e & 2u) && b == f0 && full(2u << (2 * r))) return 2u << (2 * r);
+    if (e == 3u && (a ^ b) == f0 && full(3u << (2 * r))) return 3u << (2 * r);
   }
-  if (f0 == 0 && (exact || sum_zero(f, 0u, true))) return 0u;
-  for (int w = 1; w <= min(wmax, Sp); ++w) {
-    const int alts = w == 1 ? 3 : (w == 2 ? 9 : 27);
-    const int n = alts * (w == 1 ? Sp : (w == 2 ? Sp * (Sp - 1) / 2 : Sp * (Sp - 1) * (Sp - 2) / 6));
-    for (int b = 0; b < n; b += 32) {
-      const int i = b + lane;
-      bool hit = false;
-      uint32_t x = 0;
-      if (i < n) {
-        int set = i / alts, alt = i % alts;  // the largest rank's alternative is the leading digit
-        uint32_t z = f0;
-        bool valid = true;
-        int lead = alts;
-        for (int j = w; j >= 1; --j) {  // colex: the largest rank first
-          int p = j - 1;
-          if (j == 1) p = set;
-          else if (j == 2) while ((p + 1) * p / 2 <= set) ++p;
-          else while ((p + 1) * p * (p - 1) / 6 <= set) ++p;
-          set -= j == 1 ? set : (j == 2 ? p * (p - 1) / 2 : p * (p - 1) * (p - 2) / 6);
-          lead /= 3;
-          const int c = alt / lead;
-          alt -= c * lead;
-          const uint32_t code = (uint32_t)c + 1u;
-          valid = valid && ((ex >> (2 * p)) & code) == code;
-          x |= code << (2 * p);
-          z ^= dl[3 * p + c];
+  if (cap <= 3 * kSMax && (int64_t)valid_up_to(ex, Sp, 1) >= cap) return kNone;  // the others lie beyond the cap
+  for (int hi = 1; wmax >= 2 && hi < Sp; ++hi) {
+    uint32_t h0, h1;
+    columns(hi, h0, h1);
+    const uint32_t t1 = f0 ^ h0, t2 = f0 ^ h1, t3 = t1 ^ h1;
+#pragma unroll 2
+    for (int lo = 0; lo < hi; ++lo) {
+      uint32_t a, b;
+      columns(lo, a, b);
+      const uint32_t ab = a ^ b;
+      if (t1 == a || t1 == b || t1 == ab || t2 == a || t2 == b || t2 == ab || t3 == a || t3 == b || t3 == ab) {
+        for (uint32_t c = 0; c < 9; ++c) {  // which of them, in order
+          const uint32_t h = c / 3u + 1u, l = c % 3u + 1u, x = (h << (2 * hi)) | (l << (2 * lo));
+          const uint32_t z = (l & 1u ? a : 0u) ^ (l & 2u ? b : 0u);
+          if ((h == 1u ? t1 : (h == 2u ? t2 : t3)) == z && (ex & x) == x && full(x)) return x;
         }
-        hit = valid && z == 0u && (exact || sum_zero(f, x, true));
       }
-      const unsigned m = __ballot_sync(kAll, hit);
-      if (m) return __shfl_sync(kAll, x, __ffs(m) - 1);
+    }
+  }
+  return kNone;
+}
+
+// The same for weight 3 alone (5,940 TEPs), by one warp (all arguments the same
+// in every lane): a lane holds one or two of the 3 S' alternatives as the
+// TEP's lowest altered rank and compares their projections with what the two
+// higher ranks leave; those are looped over in order.
+__device__ __noinline__ uint32_t third_weight_warp(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
+                                                   bool exact) {
+  const int lane = threadIdx.x & 31;
+  uint32_t z[2], own[2];  // own: the alternative at its rank, 0 where it does not exist
+  int rank[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int t = lane + 32 * h;
+    const uint32_t code = (uint32_t)(t % 3) + 1u;
+    rank[h] = t / 3;
+    z[h] = own[h] = 0u;
+    if (rank[h] < Sp && ((ex >> (2 * rank[h])) & code) == code) {
+      own[h] = code << (2 * rank[h]);
+      if (code & 1u) z[h] = proj(slot_pos(f, 2 * rank[h]));
+      if (code & 2u) z[h] ^= proj(slot_pos(f, 2 * rank[h] + 1));
+    }
+  }
+  auto proj_of = [&](int r, int c) {  // 0 where it does not exist
+    const int t = 3 * r + c;
+    return t < 32 ? __shfl_sync(kAll, z[0], t) : __shfl_sync(kAll, z[1], t - 32);
+  };
+  for (int hi = 2; hi < Sp; ++hi) {
+    uint32_t zh[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) zh[c] = f0 ^ proj_of(hi, c);
+    for (int mid = 1; mid < hi; ++mid) {
+      uint32_t key = kNone;  // lowest rank, then the alternatives from the largest rank down
+#pragma unroll
+      for (int cm = 0; cm < 3; ++cm) {
+        const uint32_t zm = proj_of(mid, cm), xm = (uint32_t)(cm + 1) << (2 * mid);
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          const uint32_t x = xm | ((uint32_t)(ch + 1) << (2 * hi));
+          const bool on = (ex & x) == x;
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (on && own[h] && rank[h] < mid && z[h] == (zh[ch] ^ zm) && (exact || sum_zero(f, x | own[h], true)))
+              key = min(key, (uint32_t)(rank[h] * 27 + ch * 9 + cm * 3) + (own[h] >> (2 * rank[h])) - 1u);
+        }
+      }
+      const uint32_t k = __reduce_min_sync(kAll, key);
+      if (k != kNone)
+        return ((k / 9u % 3u + 1u) << (2 * hi)) | ((k / 3u % 3u + 1u) << (2 * mid)) | ((k % 3u + 1u) << (2 * (k / 27u)));
     }
   }
   return kNone;
@@ -409,10 +467,11 @@ __device__ __noinline__ uint32_t light_hit_warp(const Frame f, const Proj proj, 
 // first_solution by one warp (all arguments but kv the same in every lane; kv
 // is read in lane src). The walk over 2^d solutions takes 2^(d-5) steps; codes
 // with few parity bits have large kernels, and then their first hit is light:
-// above 2^10 solutions weights <= 2 (631 TEPs at most) are tested first, above
-// 2^13 weight 3 (5,940) as well. Once the TEPs tested are as many as the cap, a
-// solution among the others lies beyond it and there is nothing to look for:
-// 20,000 frames of 128 bits, 8 parity bits, S = 12 and a cap of 300 348 -> 69 us.
+// above 2^kPairDim solutions the frame's thread has tested weights <= 2
+// (light_hit), above 2^13 weight 3 is tested before the walk. Once the TEPs
+// tested are as many as the cap, a solution among the others lies beyond it and
+// there is nothing to look for: 20,000 frames of 128 bits, 8 parity bits,
+// S = 12 and a cap of 300 348 -> 69 us.
 __device__ __noinline__ uint32_t first_solution_warp(const Frame f, const Proj proj, uint32_t ex, int Sp, uint32_t f0,
                                                      bool exact, uint32_t x0, const uint32_t* kv, int d, int src,
                                                      int64_t cap) {
@@ -428,11 +487,9 @@ __device__ __noinline__ uint32_t first_solution_warp(const Frame f, const Proj p
     each = __any_sync(kAll, lane < d && !sum_zero(f, mine, false));
     if (!each && !sum_zero(f, x0, true)) return kNone;
   }
-  if (d > 10) {
-    int wmax = d > 13 ? 3 : 2;
-    while (wmax > 0 && (int64_t)valid_up_to(ex, Sp, wmax - 1) >= cap) --wmax;
-    const uint32_t x = light_hit_warp(f, proj, ex, Sp, f0, exact || !each, wmax);
-    if (x != kNone || (int64_t)valid_up_to(ex, Sp, wmax) >= cap) return x;
+  if (d > 13) {
+    const uint32_t x = third_weight_warp(f, proj, ex, Sp, f0, exact || !each);
+    if (x != kNone || (int64_t)valid_up_to(ex, Sp, 3) >= cap) return x;
   }
   uint32_t x = x0, bk = kNone, bx = kNone;
   for (int t = 0; t < 5 && t < d; ++t)
@@ -451,11 +508,8 @@ __device__ __noinline__ uint32_t first_solution_warp(const Frame f, const Proj p
   return __reduce_min_sync(kAll, bk == kmin ? bx : kNone);
 }
 
-// The call's deadline has passed and the walk of a frame is not begun (all
-// arguments the same in every lane of the warp). Weights <= 1 have been tested
-// where the projection is the syndrome; a cap among them leaves nothing to walk.
-__device__ __noinline__ bool walk_is_late(const DecodeArgs& a, uint32_t ex, int Sp, bool exact) {
-  if (exact && (int64_t)valid_up_to(ex, Sp, 1) >= a.cap) return false;
+// The call's deadline has passed and the walk of a frame is not begun.
+__device__ __noinline__ bool walk_is_late(const DecodeArgs& a) {
   int late = 0;
   if ((threadIdx.x & 31) == 0) late = past_deadline(a.t0, a.deadline);
   return __shfl_sync(kAll, late, 0) != 0;
@@ -1333,6 +1387,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     F.pat = pat;
     F.polar = code->polar;
     F.nw = F.polar ? code->N >> 5 : code->W;
+    F.cols = kRows ? s_stage + warp * (kStages * kStageSyms) + (fr & 31) : nullptr;
     // one syndrome word: the columns themselves, and the elimination is the full test
     proj.tab = code->W == 1 && !(F.polar && F.nw == 1) ? code->hcol : (F.polar ? code->hx : code->hf);
     return F;
@@ -1533,19 +1588,15 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
             kv[t] = pivots_of(kv[t]) | (free_slots & (0u - free_slots));
           shared = d > kOwnDim;
           // few parity bits: most first hits weigh at most 1 (20,000 frames of
-          // 32 bits with 2 parity bits 111 -> 33 us, of 128 with 16 54 -> 38)
-          if (shared && exact) {
-            if (f0 == 0u) x = 0u;
-            for (int r = 0; r < Sp && x == kNone; ++r) {
-              const uint32_t e = (ex >> (2 * r)) & 3u;
-              const uint32_t d0 = proj(slot_pos(F, 2 * r)), d1 = proj(slot_pos(F, 2 * r + 1));
-              if ((e & 1u) && d0 == f0) x = 1u << (2 * r);
-              else if ((e & 2u) && d1 == f0) x = 2u << (2 * r);
-              else if (e == 3u && (d0 ^ d1) == f0) x = 3u << (2 * r);
-            }
-            shared = x == kNone;
+          // 32 bits with 2 parity bits 111 -> 33 us, of 128 with 16 54 -> 38);
+          // where the query cap lies among the TEPs tested, nothing is left
+          if (shared) {
+            const int tested = d > kPairDim || a.cap <= kPairTeps ? 2 : 1;
+            x = light_hit(F, proj, ex, Sp, f0, exact, tested, a.cap);
+            shared = x == kNone && (a.cap > kPairTeps || (int64_t)valid_up_to(ex, Sp, tested) < a.cap);
+          } else {
+            x = first_solution(F, exact, x0, kv, d);
           }
-          if (!shared && x == kNone) x = first_solution(F, exact, x0, kv, d);
         }
       }
     }
@@ -1557,7 +1608,7 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
     const Frame F = frame_of(of, proj);
     const int sp = __shfl_sync(kAll, Sp, src), dim = __shfl_sync(kAll, d, src);
     const uint32_t e = __shfl_sync(kAll, ex, src), p0 = __shfl_sync(kAll, f0, src), s0 = __shfl_sync(kAll, x0, src);
-    const bool late = a.deadline > 0 && dim > kCutDim && walk_is_late(a, e, sp, F.W == 1);
+    const bool late = a.deadline > 0 && dim > kCutDim && walk_is_late(a);
     const uint32_t got = late ? kCut : first_solution_warp(F, proj, e, sp, p0, F.W == 1, s0, kv, dim, src, a.cap);
     if (lane == src) x = got;
   }
@@ -1578,10 +1629,9 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
       uint32_t qn = hit ? pos : (uint32_t)((uint64_t)total < (uint64_t)a.cap ? total : (uint64_t)a.cap);
       uint8_t ab = hit ? 0 : 1;
       if (x == kCut) {
-        const CodeDev* code = codes + (kFrom == kFromMixed ? s_code[fr] : 0u);
-        qn = code->W == 1 ? valid_up_to(ex, Sp, 1) : 0u;
+        qn = valid_up_to(ex, Sp, 1);
         ab = 5;
-        atomicOr(code->status, 1u);
+        atomicOr(codes[kFrom == kFromMixed ? s_code[fr] : 0u].status, 1u);
       }
       a.queries[f] = qn;
       a.abandon[f] = ab;
