@@ -438,23 +438,17 @@ __device__ __noinline__ uint32_t third_weight_warp(const Frame f, const Proj pro
     return t < 32 ? __shfl_sync(kAll, z[0], t) : __shfl_sync(kAll, z[1], t - 32);
   };
   for (int hi = 2; hi < Sp; ++hi) {
-    uint32_t zh[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) zh[c] = f0 ^ proj_of(hi, c);
     for (int mid = 1; mid < hi; ++mid) {
       uint32_t key = kNone;  // lowest rank, then the alternatives from the largest rank down
+#pragma unroll 1
+      for (int c = 0; c < 9; ++c) {
+        const uint32_t x = ((uint32_t)(c / 3 + 1) << (2 * hi)) | ((uint32_t)(c % 3 + 1) << (2 * mid));
+        if ((ex & x) != x) continue;
+        const uint32_t want = f0 ^ proj_of(hi, c / 3) ^ proj_of(mid, c % 3);
 #pragma unroll
-      for (int cm = 0; cm < 3; ++cm) {
-        const uint32_t zm = proj_of(mid, cm), xm = (uint32_t)(cm + 1) << (2 * mid);
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-          const uint32_t x = xm | ((uint32_t)(ch + 1) << (2 * hi));
-          const bool on = (ex & x) == x;
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            if (on && own[h] && rank[h] < mid && z[h] == (zh[ch] ^ zm) && (exact || sum_zero(f, x | own[h], true)))
-              key = min(key, (uint32_t)(rank[h] * 27 + ch * 9 + cm * 3) + (own[h] >> (2 * rank[h])) - 1u);
-        }
+        for (int h = 0; h < 2; ++h)
+          if (own[h] && rank[h] < mid && z[h] == want && (exact || sum_zero(f, x | own[h], true)))
+            key = min(key, (uint32_t)(rank[h] * 27 + 3 * c) + (own[h] >> (2 * rank[h])) - 1u);
       }
       const uint32_t k = __reduce_min_sync(kAll, key);
       if (k != kNone)
@@ -1587,21 +1581,23 @@ __global__ void __launch_bounds__(32 * (kMap >= kThread ? kThreadWarps : kCtaWar
           for (int t = 0; t < d; ++t, free_slots &= free_slots - 1u)
             kv[t] = pivots_of(kv[t]) | (free_slots & (0u - free_slots));
           shared = d > kOwnDim;
-          // few parity bits: most first hits weigh at most 1 (20,000 frames of
-          // 32 bits with 2 parity bits 111 -> 33 us, of 128 with 16 54 -> 38);
-          // where the query cap lies among the TEPs tested, nothing is left
-          if (shared) {
-            const int tested = d > kPairDim || a.cap <= kPairTeps ? 2 : 1;
-            x = light_hit(F, proj, ex, Sp, f0, exact, tested, a.cap);
-            shared = x == kNone && (a.cap > kPairTeps || (int64_t)valid_up_to(ex, Sp, tested) < a.cap);
-          } else {
-            x = first_solution(F, exact, x0, kv, d);
-          }
+          if (!shared) x = first_solution(F, exact, x0, kv, d);
         }
       }
     }
   }
-  // frames with many solutions, one after the other
+  // frames with many solutions: few parity bits, and then most first hits weigh
+  // at most 1 (20,000 frames of 32 bits with 2 parity bits 111 -> 33 us, of 128
+  // with 16 54 -> 38); where the query cap lies among the TEPs tested, nothing
+  // is left. (Apart from the elimination: among its registers the call spilled.)
+  if (shared) {
+    Proj proj;
+    const Frame F = frame_of(fr, proj);
+    const int tested = d > kPairDim || a.cap <= kPairTeps ? 2 : 1;
+    x = light_hit(F, proj, ex, Sp, f0, F.W == 1, tested, a.cap);
+    shared = x == kNone && (a.cap > kPairTeps || (int64_t)valid_up_to(ex, Sp, tested) < a.cap);
+  }
+  // the others one after the other
   for (unsigned todo = __ballot_sync(kAll, shared); todo; todo &= todo - 1u) {
     const int src = __ffs(todo) - 1, of = (int)(threadIdx.x & ~31u) + src;
     Proj proj;
