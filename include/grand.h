@@ -417,9 +417,9 @@ int grand_decode_mixed(const grand_code* const* codes, int n_codes, const grand_
  * replays it with one launch): one decode call captured into a CUDA graph, replayed by
  * grand_plan_launch on any stream with the buffers given at creation (the
  * caller refills the inputs between launches; outputs are overwritten). The
- * captured sequence is the same as the direct call's (counter reset,
- * preparation kernel, persistent search kernel with its work queue, scratch as
- * graph memory nodes), so results are identical. Creation runs the call once
+ * captured sequence is the same as the direct call's (the one-kernel decode,
+ * or counter reset, preparation and persistent search kernel with its work
+ * queue; scratch as graph memory nodes), so results are identical. Creation runs the call once
  * eagerly on a private stream and synchronises it; it must not be called
  * while the calling thread captures a stream. A plan's launches must not
  * overlap each other in time (they share the buffers); the caller orders them.
