@@ -243,10 +243,12 @@ __device__ __forceinline__ uint32_t slot_pos(const Frame& f, int b) {
 }
 
 // XOR of the slot columns over x (and the base syndrome) is zero everywhere.
-// Without the base the packed columns are summed, which are fewer words than
-// the transform's for polar-form H (2 instead of 32 at 1024 bits and 40 rows).
+// Without the base the packed columns are summed where they have few words (2
+// instead of the transform's 32 at 1024 bits and 40 rows); else the
+// transform's for polar-form H, whose patterns lie in shared memory (80,000
+// frames of 512 bits, 8 words instead of 16: 43 us packed, 40.6 so).
 __device__ __noinline__ bool sum_zero(const Frame f, uint32_t x, bool base) {
-  const bool packed = !base || !f.polar;
+  const bool packed = !f.polar || (!base && (f.W <= 2 || 4 * f.W <= f.nw));
   for (int w = 0; w < (packed ? f.W : f.nw); ++w) {
     uint32_t acc = base ? f.buf[w * f.stride] : 0u;
     for (uint32_t t = x; t; t &= t - 1u) {
