@@ -26,7 +26,7 @@
 //          of the issue rate and a label reduction a step: 416 warp
 //          instructions a frame of 43 symbols (N=256, S=8). 250,000 such
 //          frames 137 -> 56 us, N=128 300,000 frames 91 -> 64 us, N=512 S=12
-//          80,000 frames 76 -> 42 us, uneven mix of 10^6 frames 904 -> 589 us.
+//          80,000 frames 76 -> 41 us, uneven mix of 10^6 frames 904 -> 590 us.
 //          What is left of a frame is its hard word and S' symbol records in
 //          shared memory.
 //   solve  one thread per frame: the base syndrome by the polar transform of
@@ -594,7 +594,7 @@ constexpr int kStages = 2;
 // between warps, and the last wave is finer (against 4 warps: 20,000 frames of
 // 128 symbols 34 -> 30 us, 300,000 of 32 70 -> 68 us). 20 of them an SM leave 96
 // registers a thread: against 24 (80 registers) 56 for 59 us on 250,000 frames
-// of 43 symbols, 43 for 52 us on 80,000 of 86, 64 for 62 us on 300,000 of 32;
+// of 43 symbols, 41 for 52 us on 80,000 of 86, 64 for 62 us on 300,000 of 32;
 // 32 spill and take 74, 53, 75.
 constexpr int kThreadCtas = 20;
 constexpr int kThreadWarps = 1;
